@@ -84,6 +84,24 @@ __global__ void cn_table_kernel(TableArgs a, cx<T> *table) {
     }
 }
 
+// Row j's coefficients: sl, sh from their FP64 values, rounded once; the lo
+// parts hold the rounding errors (zero in FP64).
+template <typename T>
+__device__ __forceinline__ CnCoef<T> cn_coef_row(const TableArgs &a, int j) {
+    CnCoef<T> c = CnCoef<T>{};
+    if (j < a.nr - 1) {
+        const double vl = j == 0 ? 0.0 : a.s * a.lo[j];
+        const double vh = j == 0 ? 4.0 * a.s : a.s * a.hi[j];
+        c.sl = T(vl);
+        c.sh = T(vh);
+        c.sll = T(vl - double(c.sl));
+        c.shl = T(vh - double(c.sh));
+        c.c0 = T((j == 0 ? 4.0 : 2.0) * a.s);
+        c.d = T(1);
+    }
+    return c;
+}
+
 // ---- FP32 tables in double-float arithmetic --------------------------------
 // A value h + l (two floats, |l| <= ulp(h)/2) carries ~48 significant bits
 // with FP32 latencies (Dekker / Knuth error-free transformations; products
@@ -191,8 +209,14 @@ __global__ void cn_table_kernel_f32(TableArgs a, cx<float> *table) {
 //      that z and stores the table.
 // The entering z comes from the matrix products instead of the recurrence
 // itself, so the two kernels agree to double-float precision (~1e-14), not
-// bit for bit.  Lane = frequency bin (32 per CTA).
-constexpr int kTabChunks = 16;
+// bit for bit.  A CTA has 16 bins x 32 chunks: a table is ~230 double-float
+// instructions per entry, and the 129 CTAs of Nt = 4096 spread them over
+// nearly all SMs (32 bins x 16 chunks: 65 SMs, 72 us for Nr = 1024).
+// The kernel also leaves the row coefficients (a.coef) and the products of
+// the sweep factors over kProdRows rows (a.prod): the rows and pivots are at
+// hand here, and an adaptive run builds two tables per attempt.
+constexpr int kTabChunks = 32;
+constexpr int kTabBins = 16;
 struct c2 {
     f2 re, im;
 };
@@ -223,39 +247,57 @@ __device__ __forceinline__ void c2_norm(c2 *v, int n) {
     for (int k = 0; k < n; ++k) v[k] = c2_scale(v[k], p2);
 }
 
-__global__ void __launch_bounds__(32 * kTabChunks) cn_table_kernel_f32_chunked(TableArgs a, cx<float> *table) {
+__global__ void __launch_bounds__(kTabBins * kTabChunks + 32) cn_table_kernel_f32_chunked(TableArgs a, cx<float> *table) {
     extern __shared__ double sh_tab[];
     f2 *kap = reinterpret_cast<f2 *>(sh_tab);                         // [nr]
-    c2 *G = reinterpret_cast<c2 *>(kap + a.nr);                      // [kTabChunks][32][4]
-    c2 *Z = G + kTabChunks * 32 * 4;                                 // [kTabChunks][32]
+    float2 *sw = reinterpret_cast<float2 *>(kap + a.nr);              // [nr]: (sl, sh) as the sweeps use them
+    c2 *G = reinterpret_cast<c2 *>(sw + a.nr);                       // [kTabChunks][kTabBins][4]
+    c2 *Z = G + kTabChunks * kTabBins * 4;                           // [kTabChunks][kTabBins]
+    __shared__ f2 byc[2][kTabBins], limc[2][kTabBins];               // per bin: by0, by1; the pivots' limit
     const double s2 = a.s * a.s;
     for (int j = threadIdx.x; j < a.nr; j += blockDim.x) {
         double k = 0.0;
         if (j == 1) k = s2 * a.lo[FCN_IDX(1, a.nr, 31)] * 4.0;
         else if (j >= 2 && j < a.nr - 1) k = s2 * a.lo[FCN_IDX(j, a.nr, 31)] * a.hi[FCN_IDX(j - 1, a.nr, 32)];
         kap[j] = to_f2(k);
+        const CnCoef<float> f = cn_coef_row<float>(a, j);
+        sw[j] = make_float2(f.sl, f.sh);
+        if (a.coef && blockIdx.x == 0) a.coef[FCN_IDX(j, a.nr, 76)] = f;
     }
-    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    const int lane = threadIdx.x % kTabBins, c = threadIdx.x / kTabBins;
     const int nq = a.nt / 2 + 1;
     const int tp = a.tp ? a.tp : nq;
-    const int q = blockIdx.x * 32 + lane;
+    const int q = blockIdx.x * kTabBins + lane;
     const bool on = q < nq;
     const int qc = on ? q : nq - 1;             // lanes past the last bin compute bin nq-1, store nothing
-    const double delta = a.dk * double(qc) * double(qc);
-    const cx<double> lim = (a.cc || a.pivlim) ? piv_limit(a.s, a.dk, qc) : cx<double>{0.0, 0.0};
-    if (a.cc && on && c == 0) {
-        const CdCol<float> cd = cd_col<float>(a.s, a.dk, q);
-        const float hx = float(lim.x), hy = float(lim.y);
-        a.cc[q].lim = make_float4(hx, hy, float(lim.x - double(hx)), float(lim.y - double(hy)));
-        a.cc[q].cd = make_float4(cd.ah, cd.al, cd.ih, cd.il);
+    // the per-bin constants in FP64, once per bin: a warp of their own (FP64
+    // in every chunk's thread was more than half of the kernel)
+    const bool extra = c >= kTabChunks;
+    if (threadIdx.x >= kTabBins * kTabChunks && threadIdx.x < kTabBins * (kTabChunks + 1)) {
+        const double delta = a.dk * double(qc) * double(qc);
+        byc[0][lane] = to_f2(4.0 * a.s - delta);
+        byc[1][lane] = to_f2(2.0 * a.s - delta);
     }
-    const f2 by0 = to_f2(4.0 * a.s - delta), by1 = to_f2(2.0 * a.s - delta);
     const f2 zero = {0.f, 0.f}, one = {1.f, 0.f};
-    const int L = (a.nr + kTabChunks - 1) / kTabChunks;
+    // whole product blocks per chunk
+    const int L = ((a.nr + kTabChunks - 1) / kTabChunks + kProdRows<float> - 1) / kProdRows<float> * kProdRows<float>;
     const int j0 = min(a.nr, c * L), j1 = min(a.nr, j0 + L);
-    auto by_of = [&](int j) { return (j == 0) ? by0 : ((j < a.nr - 1) ? by1 : zero); };
     __syncthreads();
-    {
+    const f2 by0 = byc[0][lane], by1 = byc[1][lane];
+    auto by_of = [&](int j) { return (j == 0) ? by0 : ((j < a.nr - 1) ? by1 : zero); };
+    if (extra) {
+        if (threadIdx.x < kTabBins * (kTabChunks + 1)) {
+            const cx<double> lim = (a.cc || a.pivlim) ? piv_limit(a.s, a.dk, qc) : cx<double>{0.0, 0.0};
+            limc[0][lane] = to_f2(lim.x);
+            limc[1][lane] = to_f2(lim.y);
+            if (a.cc && on) {
+                const CdCol<float> cd = cd_col<float>(a.s, a.dk, q);
+                const float hx = float(lim.x), hy = float(lim.y);
+                a.cc[q].lim = make_float4(hx, hy, float(lim.x - double(hx)), float(lim.y - double(hy)));
+                a.cc[q].cd = make_float4(cd.ah, cd.al, cd.ih, cd.il);
+            }
+        }
+    } else {
         // 1. this chunk's matrix
         c2 g[4] = {{one, zero}, {zero, zero}, {zero, zero}, {one, zero}};   // g00 g01 g10 g11
         for (int j = j0; j < j1; ++j) {
@@ -269,7 +311,7 @@ __global__ void __launch_bounds__(32 * kTabChunks) cn_table_kernel_f32_chunked(T
             if (((j - j0) & 7) == 7) c2_norm(g, 4);
         }
         c2_norm(g, 4);
-        for (int k = 0; k < 4; ++k) G[(c * 32 + lane) * 4 + k] = g[k];
+        for (int k = 0; k < 4; ++k) G[(c * kTabBins + lane) * 4 + k] = g[k];
     }
     __syncthreads();
     if (c == 0) {
@@ -279,22 +321,25 @@ __global__ void __launch_bounds__(32 * kTabChunks) cn_table_kernel_f32_chunked(T
             const c2 n = v[0], d = v[1];
             const f2 rn = df_recip(df_add(df_mul(d.re, d.re), df_mul(d.im, d.im)));
             const c2 z = c2_mul(n, c2{d.re, df_neg(d.im)});
-            Z[k * 32 + lane] = c2{df_mul(z.re, rn), df_mul(z.im, rn)};
-            const c2 *gk = G + (k * 32 + lane) * 4;
+            Z[k * kTabBins + lane] = c2{df_mul(z.re, rn), df_mul(z.im, rn)};
+            const c2 *gk = G + (k * kTabBins + lane) * 4;
             v[0] = c2_add(c2_mul(gk[0], n), c2_mul(gk[1], d));
             v[1] = c2_add(c2_mul(gk[2], n), c2_mul(gk[3], d));
             c2_norm(v, 2);
         }
     }
     __syncthreads();
+    if (extra) return;
     // 3. the rows of this chunk
     f2 lx = zero, ly = zero;
     if (a.pivlim) {
-        lx = to_f2(lim.x);
-        ly = to_f2(lim.y);
+        lx = limc[0][lane];
+        ly = limc[1][lane];
     }
-    const c2 z = Z[c * 32 + lane];
+    const c2 z = Z[c * kTabBins + lane];
     f2 ix = z.re, iy = z.im;
+    const int NP = (a.nr + kProdRows<float> - 1) / kProdRows<float>;
+    cx<float> A = mk(1.f, 0.f), Q = A;
     for (int j = j0; j < j1; ++j) {
         const f2 kp = kap[j];
         const f2 by = by_of(j);
@@ -307,6 +352,20 @@ __global__ void __launch_bounds__(32 * kTabChunks) cn_table_kernel_f32_chunked(T
         const cx<float> e = a.pivlim ? mk((ix.h - lx.h) + (ix.l - lx.l), (iy.h - ly.h) + (iy.l - ly.l))
                                      : mk(ix.h + ix.l, iy.h + iy.l);
         if (on) table[FCN_IDX((size_t)j * tp + q, (size_t)a.nr * tp, 30)] = e;
+        if (a.prod) {
+            const cx<float> inv = mk(ix.h + ix.l, iy.h + iy.l);
+            const float2 f = sw[j];
+            A = cmul(cmul_i(inv, f.x), A);
+            Q = cmul(cmul_i(inv, f.y), Q);
+            if ((j % kProdRows<float>) == kProdRows<float> - 1 || j == a.nr - 1) {
+                if (on) {
+                    const int pc = j / kProdRows<float>;
+                    a.prod[FCN_IDX((size_t)pc * tp + q, (size_t)2 * NP * tp, 74)] = A;
+                    a.prod[FCN_IDX((size_t)(NP + pc) * tp + q, (size_t)2 * NP * tp, 75)] = Q;
+                }
+                A = Q = mk(1.f, 0.f);
+            }
+        }
     }
 }
 
@@ -442,291 +501,12 @@ cn_kernel(ColArgs<T> a, int C) {
     cn_body<T, L>(a, C, g, smem_raw);
 }
 
-// Batched work list: item = (pulse, column group, C); 512-thread CTAs; a
-// persistent grid pulls items from a global counter.
-template <typename T, int L>
-__global__ void __launch_bounds__(512)
-cn_batch_kernel(const ColArgs<T> *__restrict__ pulses, const int4 *__restrict__ items, int nitems,
-                unsigned *counter) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int next;
-    for (;;) {
-        if (threadIdx.x == 0) next = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int it = next;
-        __syncthreads();
-        if (it >= nitems) break;
-        const int4 w = items[it];
-        const ColArgs<T> a = pulses[w.x];
-        cn_body<T, L>(a, w.z, w.y, smem_raw);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const unsigned done = atomicAdd(counter + 1, 1u) + 1;
-        if (done == gridDim.x) {
-            counter[0] = 0;
-            counter[1] = 0;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Staged variant.  Same chunked scan, but each thread first copies its chunk
-// (rows j0-1 .. j0+L of its column, and the L pivots) into private
-// shared-memory slots with cp.async, so no registers are held by loads in
-// flight, and the per-row coefficients come from one CnCoef row instead of
-// index tests.  The first sweep turns each slot into what the later sweeps
-// need (x_j -> alpha_j, 1/piv_j -> gamma_j), so every later pass is one
-// shared-memory load and one complex multiply-add per row.  Slot k of thread
-// t sits at k * blockDim + t: consecutive lanes, consecutive words.
-// ---------------------------------------------------------------------------
-
-// One complex value global -> shared, asynchronously; valid = false writes
-// zeros without reading the source.
-template <typename T>
-__device__ __forceinline__ void cp_async_cx(cx<T> *dst, const cx<T> *src, bool valid) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const int n = valid ? int(sizeof(cx<T>)) : 0;
-    if constexpr (sizeof(cx<T>) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
-
-template <typename T>
-__device__ __forceinline__ void cp_async_cx_full(cx<T> *dst, const cx<T> *src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (sizeof(cx<T>) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
 constexpr size_t kCnStagedSmemMax = 227 * 1024;
-
-// Forward sweep, pass 1, of the register-fed staged variant: x and 1/piv
-// are read from global memory straight into registers (the compiler
-// hoists the loads of the unrolled loop), alpha_j and gamma_j go to the
-// thread's shared-memory slots.  EDGE: the chunk touches row -1 or row nr.
-template <typename T, int L, bool EDGE, int NTC>
-__device__ __forceinline__ void cn_f1_reg(const ColArgs<T> &a, int q, int qq, int j0, const CdCol<T> &cdc,
-                                          const PivLim<T> &plim, cx<T> *At,
-                                          cx<T> *Gt, int BD, cx<T> (&y)[L], cx<T> &PA, cx<T> &PB) {
-    // NTC: Nt as a compile-time constant (row strides become immediates), 0: a.nt
-    const int nt = NTC ? NTC : a.nt, nr = a.nr, nq = a.tp;
-    const cx<T> *fx = a.field + q;
-    const cx<T> *fi = a.invden + qq;
-    auto X = [&](int j) -> cx<T> {
-        if (EDGE && (j < 0 || j >= nr)) return czero<T>();
-        return ldg_cx(fx + FCN_IDX((size_t)j * nt, (size_t)nr * nt, 51));
-    };
-    cx<T> xm = X(j0 - 1), x0 = X(j0);
-#pragma unroll
-    for (int k = 0; k < L; ++k) {
-        const int j = j0 + k;
-        const cx<T> xp = X(j + 1);
-        cx<T> inv = czero<T>();
-        if (!EDGE || j < nr) inv = ldg_cx(fi + FCN_IDX((size_t)j * nq, (size_t)nr * nq, 52));
-        CnCoef<T> cf;
-        if (!EDGE || j < nr - 1) {
-            cf = a.coef[FCN_IDX(j, nr, 53)];
-        } else {
-            cf = CnCoef<T>{};
-        }
-        const cx<T> rhs = ex_rhs(ex_row(cf, j == 0, cdc), xm, x0, xp);
-        const cx<T> beta = piv_apply(rhs, inv, plim);
-        const cx<T> ivf = piv_full(inv, plim);
-        const cx<T> al = cmul_i(ivf, cf.sl);
-        At[k * BD] = al;
-        Gt[k * BD] = cmul_i(ivf, cf.sh);
-        PB = cmul(al, PB) + beta;
-        PA = cmul(al, PA);
-        y[k] = beta;
-        xm = x0;
-        x0 = xp;
-    }
-}
-
-template <typename T, int L, bool REG, int NTC = 0>
-__device__ __forceinline__ void cn_staged_body(const ColArgs<T> &a, int C, int g, unsigned char *smem_raw) {
-    const int BD = blockDim.x;
-    const int tid = threadIdx.x;
-    const int nwarp = BD >> 5;
-    cx<T> *smA = reinterpret_cast<cx<T> *>(smem_raw);
-    cx<T> *smB = smA + nwarp * C;
-    cx<T> *smC = smB + nwarp * C;
-    cx<T> *Xt = smC + nwarp * C + tid;          // slot k: Xt[k * BD]
-    // staged: L+2 x slots then L pivot slots; register-fed: L alpha slots
-    // then L gamma slots
-    cx<T> *Gt = Xt + (REG ? L : L + 2) * BD;    // slot k: Gt[k * BD], k = 0 .. L-1
-
-    const int col = tid % C;
-    const int chunk = tid / C;
-    const int q = g * C + col;
-    const int nt = NTC ? NTC : a.nt, nr = a.nr;
-    const int nq = a.tp;
-    const int qq = (q <= nt / 2) ? q : nt - q;
-    CdCol<T> cdc;
-    PivLim<T> plim;
-    col_consts<T>(a.cc, a.pivlim, a.s64, a.dk64, qq, &cdc, &plim);
-    const int j0 = chunk * L;
-
-    cx<T> y[L];
-    cx<T> PA = mk(T(1), T(0)), PB = czero<T>();
-    // slot of alpha_j: Xt[(k+1) BD] (staged: where x_j was), At[k BD] below
-    cx<T> *At = REG ? Xt : Xt + BD;
-    if constexpr (REG) {
-        if (j0 >= 1 && j0 + L < nr)
-            cn_f1_reg<T, L, false, NTC>(a, q, qq, j0, cdc, plim, At, Gt, BD, y, PA, PB);
-        else
-            cn_f1_reg<T, L, true, NTC>(a, q, qq, j0, cdc, plim, At, Gt, BD, y, PA, PB);
-    } else {
-    if (j0 >= 1 && j0 + L < nr) {
-        // interior chunk: every row j0-1 .. j0+L exists
-        const cx<T> *src = a.field + (size_t)(j0 - 1) * nt + q;
-#pragma unroll
-        for (int k = 0; k < L + 2; ++k) cp_async_cx_full(Xt + k * BD, src + (size_t)k * nt);
-        const cx<T> *pv = a.invden + (size_t)j0 * nq + qq;
-#pragma unroll
-        for (int k = 0; k < L; ++k) cp_async_cx_full(Gt + k * BD, pv + (size_t)k * nq);
-    } else {
-        // rows outside 0..nr-1 are zero-filled (the source is then not read;
-        // the base address stands in for it)
-        const cx<T> *src = a.field + (ptrdiff_t)(j0 - 1) * nt + q;
-#pragma unroll
-        for (int k = 0; k < L + 2; ++k, src += nt) {
-            const int j = j0 - 1 + k;
-            const bool ok = j >= 0 && j < nr;
-            cp_async_cx(Xt + k * BD, ok ? src : a.field, ok);
-        }
-        const cx<T> *pv = a.invden + (size_t)j0 * nq + qq;
-#pragma unroll
-        for (int k = 0; k < L; ++k, pv += nq) {
-            const bool ok = j0 + k < nr;
-            cp_async_cx(Gt + k * BD, ok ? pv : a.invden, ok);
-        }
-    }
-    cp_async_wait_all();
-
-    // forward sweep, pass 1: beta_j, alpha_j, gamma_j and the chunk map
-    cx<T> xm = Xt[0], x0 = Xt[BD];
-#pragma unroll
-    for (int k = 0; k < L; ++k) {
-        const int j = j0 + k;
-        const cx<T> xp = Xt[(k + 2) * BD];
-        const cx<T> inv = Gt[k * BD];
-        CnCoef<T> cf;
-        if (j < nr - 1) {
-            cf = a.coef[FCN_IDX(j, nr, 46)];
-        } else {
-            cf = CnCoef<T>{};
-        }
-        const cx<T> rhs = ex_rhs(ex_row(cf, j == 0, cdc), xm, x0, xp);
-        const cx<T> beta = piv_apply(rhs, inv, plim);
-        const cx<T> ivf = piv_full(inv, plim);
-        const cx<T> al = cmul_i(ivf, cf.sl);
-        Xt[(k + 1) * BD] = al;                  // x_j (slot k+1) is no longer read
-        Gt[k * BD] = cmul_i(ivf, cf.sh);
-        PB = cmul(al, PB) + beta;
-        PA = cmul(al, PA);
-        y[k] = beta;
-        xm = x0;
-        x0 = xp;
-        asm volatile("" ::: "memory");          // keep the slot loads in row order
-    }
-    }
-    // forward sweep, pass 2: exact y from the carry entering the chunk
-    {
-        cx<T> yp = chunk_scan<T, false>(PA, PB, C, col, smA, smB, smC);
-#pragma unroll
-        for (int k = 0; k < L; ++k) {
-            y[k] = cmul(At[k * BD], yp) + y[k];
-            yp = y[k];
-            asm volatile("" ::: "memory");
-        }
-    }
-    // backward sweep, pass 1: chunk map x_first = QA x_next + QB
-    cx<T> QA = mk(T(1), T(0)), QB = czero<T>();
-#pragma unroll
-    for (int k = L - 1; k >= 0; --k) {
-        const cx<T> ga = Gt[k * BD];
-        QB = cmul(ga, QB) + y[k];
-        QA = cmul(ga, QA);
-        asm volatile("" ::: "memory");
-    }
-    // backward sweep, pass 2 and store
-    cx<T> xn = chunk_scan<T, true>(QA, QB, C, col, smA, smB, smC);
-    const DispPhase<T> ph = disp_phase<T>(a.disp, qq);
-    cx<T> *fo = a.field + (size_t)j0 * nt + q;
-#pragma unroll
-    for (int k = L - 1; k >= 0; --k) {
-        const int j = j0 + k;
-        xn = cmul(Gt[k * BD], xn) + y[k];
-        if (j < nr) fo[FCN_IDX((size_t)k * nt, (size_t)(nr - j0) * nt, 47)] = disp_apply(xn, ph);
-        asm volatile("" ::: "memory");
-    }
-}
-
-// Register budget: 3 CTAs of 256 threads per SM for 16-row chunks, 2 CTAs of
-// 512 threads for 8-row chunks (the launcher keeps the CTA within this size).
-template <typename T, int L>
-constexpr int staged_threads() { return L >= 16 ? 256 : 512; }
-
-template <typename T, int L, bool REG, int NTC>
-__global__ void __launch_bounds__(staged_threads<T, L>(), L >= 16 ? 3 : 2)
-cn_staged_kernel(ColArgs<T> a, int C) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_enter();
-    const int ngroups = a.nt / C;
-    const int b = blockIdx.x;
-    const int g = (b & 1) ? (ngroups - 1 - (b >> 1)) : (b >> 1);
-    cn_staged_body<T, L, REG, NTC>(a, C, g, smem_raw);
-}
 
 template <typename T>
 __global__ void cn_coef_kernel(TableArgs a, CnCoef<T> *coef) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= a.nr) return;
-    CnCoef<T> c = CnCoef<T>{};
-    if (j < a.nr - 1) {
-        // sl, sh from their FP64 values, rounded once; the lo parts hold the
-        // rounding errors (zero in FP64)
-        const double vl = j == 0 ? 0.0 : a.s * a.lo[j];
-        const double vh = j == 0 ? 4.0 * a.s : a.s * a.hi[j];
-        c.sl = T(vl);
-        c.sh = T(vh);
-        c.sll = T(vl - double(c.sl));
-        c.shl = T(vh - double(c.sh));
-        c.c0 = T((j == 0 ? 4.0 : 2.0) * a.s);
-        c.d = T(1);
-    }
-    coef[j] = c;
-}
-
-// Chunk length L; C columns per CTA (one 32-byte sector when the column fits
-// the CTA size, fewer for tall grids, more for short ones).  Returns
-// cudaErrorInvalidConfiguration when the grid does not fit (the caller then
-// falls back to the register variant).
-template <typename T, int L, bool REG, int NTC>
-cudaError_t launch_cn_staged_l(const ColArgs<T> &a, cudaStream_t st) {
-    if (!a.coef) return cudaErrorInvalidConfiguration;
-    constexpr int CMIN = 32 / int(sizeof(cx<T>));
-    constexpr int TMAX = staged_threads<T, L>();
-    const int P = (a.nr + L - 1) / L;
-    int C = CMIN;
-    while (C > 1 && C * P > TMAX) C /= 2;                 // tall grids: fewer columns
-    while (C * 2 * P <= TMAX / 2 && C * 2 <= 32) C *= 2;  // short grids: more columns
-    if (C > a.nt) C = a.nt;
-    const int threads = ((C * P + 31) / 32) * 32;
-    if (threads > TMAX) return cudaErrorInvalidConfiguration;
-    const size_t slots = REG ? 2 * L : 2 * L + 2;
-    const size_t smem = sizeof(cx<T>) * (3 * (size_t)(threads / 32) * C + slots * threads);
-    if (smem > kCnStagedSmemMax) return cudaErrorInvalidConfiguration;
-    return launch_k(cn_staged_kernel<T, L, REG, NTC>, dim3(a.nt / C), dim3(threads), smem, st, a, C);
+    if (j < a.nr) coef[j] = cn_coef_row<T>(a, j);
 }
 
 template <typename T, int L>
@@ -913,28 +693,6 @@ cudaError_t set_pair_attr() {
     return set_col_attrs(cn_pair_kernel<T, L, NTC>);
 }
 
-// Register-fed variant with Nt as a compile-time constant for the grids of
-// 512 .. 8192 points in FP32 (every row offset an immediate), generic otherwise.
-template <typename T, int L>
-cudaError_t launch_cn_reg_nt(const ColArgs<T> &a, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        switch (a.nt) {
-            case 512: return launch_cn_staged_l<T, L, true, 512>(a, st);
-            case 1024: return launch_cn_staged_l<T, L, true, 1024>(a, st);
-            case 2048: return launch_cn_staged_l<T, L, true, 2048>(a, st);
-            case 4096: return launch_cn_staged_l<T, L, true, 4096>(a, st);
-            case 8192: return launch_cn_staged_l<T, L, true, 8192>(a, st);
-            default: break;
-        }
-    }
-    return launch_cn_staged_l<T, L, true, 0>(a, st);
-}
-
-template <typename T, int L, bool REG, int NTC>
-cudaError_t set_staged_attr() {
-    return set_col_attrs(cn_staged_kernel<T, L, REG, NTC>);
-}
-
 }  // namespace
 
 // Variants: bit 0 selects the shorter chunk (more threads, fewer registers
@@ -952,18 +710,13 @@ cudaError_t launch_cn(const ColArgs<T> &a_in, cudaStream_t st) {
         cx<T> *f = a.field;
         e = launch_cn_seq<T>(a, &f, 1, st);
         if (e != cudaErrorInvalidConfiguration) return e;
-        a.variant = kColStagedFirst + 3;            // not supported here: register-fed
+        a.variant = kColBlockFirst;                 // not supported here
     }
-    if (a.variant >= kColStagedFirst) {
-        switch (a.variant - kColStagedFirst) {
-            case 0: e = launch_cn_staged_l<T, LL, false, 0>(a, st); break;
-            case 1: e = launch_cn_staged_l<T, LS, false, 0>(a, st); break;
-            case 2: e = launch_cn_reg_nt<T, LL>(a, st); break;
-            default: e = launch_cn_reg_nt<T, LS>(a, st); break;
-        }
+    if (a.variant >= kColBlockFirst) {
+        e = launch_cn_block<T>(a, a.variant - kColBlockFirst, st);
         if (e != cudaErrorInvalidConfiguration) return e;
     }
-    if (a.variant < kColStagedFirst && (a.variant & 1)) e = launch_cn_l<T, LS>(a, target, st);
+    if (a.variant < kColBlockFirst && (a.variant & 1)) e = launch_cn_l<T, LS>(a, target, st);
     if (e == cudaErrorInvalidConfiguration) e = launch_cn_l<T, LL>(a, target, st);
     if (e == cudaErrorInvalidConfiguration) e = launch_cn_l<T, LL>(a, 256, st);
     return e;
@@ -1000,28 +753,13 @@ cudaError_t launch_cn_coef(const TableArgs &a, CnCoef<T> *coef, cudaStream_t st)
 
 template <typename T>
 cudaError_t prepare_cn() {
-    constexpr int LL = sizeof(T) == 4 ? 16 : 8, LS = LL / 2;
-    cudaError_t e = set_staged_attr<T, LL, false, 0>();
-    if (e == cudaSuccess) e = set_staged_attr<T, LS, false, 0>();
-    if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 0>();
-    if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 0>();
-    if (e == cudaSuccess) e = set_pair_attr<T, 8, 0>();
+    cudaError_t e = set_pair_attr<T, 8, 0>();
     if constexpr (sizeof(T) == 4) {
         if (e == cudaSuccess) e = set_pair_attr<T, 8, 512>();
         if (e == cudaSuccess) e = set_pair_attr<T, 8, 1024>();
         if (e == cudaSuccess) e = set_pair_attr<T, 8, 2048>();
         if (e == cudaSuccess) e = set_pair_attr<T, 8, 4096>();
         if (e == cudaSuccess) e = set_pair_attr<T, 8, 8192>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 512>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 512>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 1024>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 1024>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 2048>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 2048>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 4096>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 4096>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LL, true, 8192>();
-        if (e == cudaSuccess) e = set_staged_attr<T, LS, true, 8192>();
     }
     return e;
 }
@@ -1031,19 +769,20 @@ cudaError_t launch_cn_table(const TableArgs &a, cx<T> *table, cudaStream_t st) {
     const int nq = a.nt / 2 + 1;
     const int threads = 32;   // spread the latency-bound recurrences over many SMs
     if constexpr (sizeof(T) == 4) {
-        if (a.nr >= 128) {
+        if (cn_table_fills_all<T>(a.nr)) {
             // rows in chunks (cn_table_kernel_f32_chunked): the serial
             // recurrence down a tall column is the cost of a table
-            const size_t smem = sizeof(f2) * a.nr + sizeof(c2) * kTabChunks * 32 * 5;
+            constexpr size_t fixed = sizeof(c2) * kTabChunks * kTabBins * 5;
             static std::once_flag once;
             static cudaError_t attr = cudaSuccess;
             std::call_once(once, [] {
                 attr = cudaFuncSetAttribute(cn_table_kernel_f32_chunked, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)(sizeof(f2) * 4096 + sizeof(c2) * kTabChunks * 32 * 5));
+                                            (int)((sizeof(f2) + sizeof(float2)) * 4096 + fixed));
             });
             if (attr != cudaSuccess) return attr;
             if (a.nr > 4096) return cudaErrorInvalidValue;
-            cn_table_kernel_f32_chunked<<<(nq + 31) / 32, 32 * kTabChunks, smem, st>>>(a, table);
+            cn_table_kernel_f32_chunked<<<(nq + kTabBins - 1) / kTabBins, kTabBins * kTabChunks + 32,
+                                          (sizeof(f2) + sizeof(float2)) * a.nr + fixed, st>>>(a, table);
         } else {
             cn_table_kernel_f32<<<(nq + threads - 1) / threads, threads, sizeof(double) * a.nr, st>>>(a, table);
         }
@@ -1052,18 +791,7 @@ cudaError_t launch_cn_table(const TableArgs &a, cx<T> *table, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_cn_batch(const ColArgs<T> *pulses, const int4 *items, int nitems, unsigned *counter,
-                            int grid, cudaStream_t st) {
-    constexpr int L = sizeof(T) == 4 ? 16 : 8;
-    const size_t smem = sizeof(cx<T>) * 3 * 16 * 32;     // 16 warps x C <= 32 x 3 maps
-    cn_batch_kernel<T, L><<<grid, 512, smem, st>>>(pulses, items, nitems, counter);
-    return cudaGetLastError();
-}
-
 template cudaError_t launch_cn<float>(const ColArgs<float> &, cudaStream_t);
-template cudaError_t launch_cn_batch<float>(const ColArgs<float> *, const int4 *, int, unsigned *, int,
-                                            cudaStream_t);
 template cudaError_t launch_cn<double>(const ColArgs<double> &, cudaStream_t);
 template cudaError_t launch_cn_table<float>(const TableArgs &, cx<float> *, cudaStream_t);
 template cudaError_t launch_cn_coef<float>(const TableArgs &, CnCoef<float> *, cudaStream_t);

@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <limits>
 #include <fstream>
 #include <map>
 #include <tuple>
@@ -105,6 +106,11 @@ NLCoef<T> nl_coef(const fcn_grid &g, const fcn_params &p, double h) {
         n.hk[j] = (p.flags & FCN_KERR) ? T(h * (c.k0 / p.n0) * p.n2j[j] * isj) : T(0);
         isj *= kIs;
     }
+    // the scale is a power of two: exact unless the product leaves T's normal range
+    n.kf[0] = n.hk[0] * n.inv_is;
+    n.kf[1] = n.hk[1] * n.inv_is * n.inv_is;
+    auto exact = [](T x, T f) { return x == T(0) || std::fabs(f) >= std::numeric_limits<T>::min(); };
+    n.kerr2 = n.hk[2] == T(0) && n.hk[3] == T(0) && exact(n.hk[0], n.kf[0]) && exact(n.hk[1], n.kf[1]);
     n.hplasma = (p.flags & FCN_PLASMA) ? T(h * (c.k0 / (2.0 * p.n0 * p.n0 * c.rho_c) * p.rho_nt)) : T(0);
     n.hloss = (p.flags & FCN_MPI) ? T(h * 0.5 * c.beta_k * std::pow(kIs, p.K - 1)) : T(0);
     n.sat = (p.flags & FCN_MPI_SAT) ? T(1) : T(0);
@@ -278,6 +284,7 @@ struct Pulse {
     int *err = nullptr;        // [1] set by a kernel whose bounded wait gave up
     const void *tw = nullptr;
     const void *tw1 = nullptr;   // twiddles of FFT plan 1 (FP32, Nt >= 256), or null
+    const void *tw2 = nullptr;   // twiddles of FFT plan 2
     const void *lo = nullptr, *hi = nullptr;
     const double *lo64 = nullptr, *hi64 = nullptr;
     double z = 0.0, dz_next = 0.0;
@@ -370,11 +377,10 @@ struct fcn_ctx {
     bool batched = false;
     int2 *row_items = nullptr;
     int nrow_items = 0;
-    int4 *col_items = nullptr;
+    int2 *col_items = nullptr;
     int ncol_items = 0;
-    unsigned *counter = nullptr;
-    size_t row_smem = 0;
-    int row_grid = 0, col_grid = 0;
+    int row_th = 0;              // CTA size of the batched row kernel
+    int col_max_nr = 0;          // largest Nr of the batch
     std::map<uint64_t, std::pair<void *, void *>> batch_args;   // dz -> (RowArgs[], ColArgs[])
 };
 
@@ -420,13 +426,21 @@ size_t cc_offset(int nr, int nt) {
     const size_t b = coef_offset<T>(nr, nt) + sizeof(CnCoef<T>) * (size_t)nr;
     return (b + 255) / 256 * 256;
 }
+// then the products of the sweep factors (ColArgs::prod)
+template <typename T>
+size_t prod_offset(int nr, int nt) {
+    const size_t b = cc_offset<T>(nr, nt) + (sizeof(T) == 4 ? sizeof(ColConst) * (size_t)table_pitch(nt) : 0);
+    return (b + 255) / 256 * 256;
+}
 template <typename T>
 size_t table_bytes(int nr, int nt) {
-    return sizeof(T) == 4 ? cc_offset<T>(nr, nt) + sizeof(ColConst) * (size_t)table_pitch(nt)
-                          : coef_offset<T>(nr, nt) + sizeof(CnCoef<T>) * (size_t)nr;
+    const size_t np = (size_t)(nr + kProdRows<T> - 1) / kProdRows<T>;
+    return prod_offset<T>(nr, nt) + sizeof(cx<T>) * 2 * np * (size_t)table_pitch(nt);
 }
 
 void drop_graphs(fcn_ctx *ctx, bool all, uint64_t dz);
+template <typename T>
+ColArgs<T> col_args(Pulse &pu, void *field, const cx<T> *table, double dz);
 
 // The pivot table of (grid, dz), built on first use.  side = -1 builds it on
 // the launch stream; side = 0 or 1 builds it on a side stream (after all
@@ -505,8 +519,17 @@ int ensure_table(fcn_ctx *ctx, Pulse &pu, double dz, const cx<T> **out, int side
         CK(cudaStreamWaitEvent(bs, ctx->tbefore[side], 0), "table wait");
     }
     CnCoef<T> *coef = (CnCoef<T> *)((char *)d + coef_offset<T>(pu.g.nr, pu.g.nt));
-    CK(launch_cn_coef<T>(ta, coef, bs), "row coefficient kernel");
+    cx<T> *prod = (cx<T> *)((char *)d + prod_offset<T>(pu.g.nr, pu.g.nt));
+    const bool all = cn_table_fills_all<T>(pu.g.nr);
+    if constexpr (sizeof(T) == 4) {
+        if (all) {
+            ta.coef = coef;
+            ta.prod = prod;
+        }
+    }
+    if (!all) CK(launch_cn_coef<T>(ta, coef, bs), "row coefficient kernel");
     CK(launch_cn_table<T>(ta, (cx<T> *)d, bs), "pivot table kernel");
+    if (!all) CK(launch_cn_prod<T>(col_args<T>(pu, nullptr, (const cx<T> *)d, dz), prod, bs), "sweep product kernel");
     if (side >= 0) {
         CK(cudaEventRecord(ctx->tready[side], bs), "table event");
         if (ready) *ready = ctx->tready[side];
@@ -523,6 +546,7 @@ RowArgs<T> row_args(Pulse &pu, void *field, int ops, double dz) {
     a.field = (cx<T> *)field;
     a.tw = (const cx<T> *)pu.tw;
     a.tw1 = (const cx<T> *)pu.tw1;
+    a.tw2 = (const cx<T> *)pu.tw2;
     a.rho = (T *)pu.rho;
     a.stats = pu.stats;
     a.nr = pu.g.nr;
@@ -552,6 +576,7 @@ ColArgs<T> col_args(Pulse &pu, void *field, const cx<T> *table, double dz) {
     a.dk64 = dk;
     a.disp = disp;
     a.variant = pu.col_var;
+    a.prod = (const cx<T> *)((const char *)table + prod_offset<T>(pu.g.nr, pu.g.nt));
     a.tp = table_pitch(pu.g.nt);
     a.err = pu.err;
     a.pivlim = sizeof(T) == 4 ? 1 : 0;   // FP32 context tables hold deltas (ensure_table)
@@ -673,14 +698,12 @@ cudaError_t launch_block_batched(fcn_ctx *ctx, int kind, double dz, cudaStream_t
         if (e != cudaSuccess) return e;
         auto rows = [&](int ops, int pk) {
             return timed(ctx, pk, st, [&] {
-                return launch_rows_batch<T>(ra, ctx->row_items, ctx->nrow_items, ops, ctx->counter,
-                                            ctx->row_smem, ctx->row_grid, st);
+                return launch_rows_batch<T>(ra, ctx->row_items, ctx->nrow_items, ops, ctx->row_th, st);
             });
         };
         auto col = [&] {
             return timed(ctx, FCN_PROF_COLUMN, st, [&] {
-                return launch_cn_batch<T>(ca, ctx->col_items, ctx->ncol_items, ctx->counter,
-                                          ctx->col_grid, st);
+                return launch_cn_batch<T>(ca, ctx->col_items, ctx->ncol_items, ctx->col_max_nr, st);
             });
         };
         if (kind == 0) {
@@ -1061,7 +1084,14 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
         std::vector<float> tr(nrv, 1e30f), tc(kColVariants, 1e30f);
         for (int round = 0; round < 3; ++round) {
             for (int v = 0; v < nrv; ++v) {
-                RowArgs<T> a = row_args<T>(pu, scratch, OPS_MID, dz);
+                // on the spectrum that a middle launch meets (the pulse after
+                // its opening half step): what the nonlinear part has to do
+                // depends on the intensities
+                RowArgs<T> a = row_args<T>(pu, scratch, OPS_HEAD, dz);
+                a.variant = 0;
+                a.in = (const cx<T> *)pu.field;
+                CK(launch_rows<T>(a, pu.g.nt, ctx->st), "tuning input");
+                a = row_args<T>(pu, scratch, OPS_MID, dz);
                 a.variant = v;
                 float ms;
                 int rc = time_launches(ctx, [&] { return launch_rows<T>(a, pu.g.nt, ctx->st); }, &ms);
@@ -1713,55 +1743,47 @@ Pulse *get_pulse(fcn_ctx *ctx, int pulse) {
 }
 
 // Work lists of the batched kernels: row items (pulse, first row) with
-// 512/(Nt/16) rows each, column items (pulse, group, C) with C P <= 512 (P =
-// chunks of 16 rows); both sorted largest first.  Only when every pulse runs
-// FP32 with K = 8 and Nt >= 512 (else per-pulse launches are used).
+// row_batch_threads/(Nt/16) rows each, column items (pulse, group) of
+// cn_batch_columns columns; both sorted largest first.  Only when every pulse
+// runs FP32 with K = 8 and Nt >= 512 (else per-pulse launches are used).
 int setup_batch(fcn_ctx *ctx) {
     for (auto &pu : ctx->pulses)
         if (pu.p.K != 8 || pu.g.nt < 512) return FCN_OK;
     if (ctx->row_items) return FCN_OK;   // already built
     std::vector<std::pair<int64_t, int2>> rows;
-    std::vector<std::pair<int64_t, int4>> cols;
-    size_t smem = 0;
+    std::vector<std::pair<int64_t, int2>> cols;
+    int max_nt = 0, max_nr = 0;
+    for (auto &pu : ctx->pulses) {
+        max_nt = std::max(max_nt, (int)pu.g.nt);
+        max_nr = std::max(max_nr, (int)pu.g.nr);
+    }
+    const int th = row_batch_threads(max_nt), C = cn_batch_columns(max_nr);
     for (size_t i = 0; i < ctx->pulses.size(); ++i) {
         const Pulse &pu = ctx->pulses[i];
         const int nt = pu.g.nt, nr = pu.g.nr;
-        const int rpi = 512 / (nt / 16);
+        const int rpi = th / (nt / 16);
         for (int r0 = 0; r0 < nr; r0 += rpi) rows.push_back({(int64_t)nt, make_int2((int)i, r0)});
-        const size_t sm = row_batch_smem(nt, 8);
-        if (sm > smem) smem = sm;
-        const int P = (nr + 15) / 16;
-        int C = 4;
-        while (C * 2 * P <= 512 && C * 2 <= 32) C *= 2;
-        if (C > nt) C = nt;
         const int ng = nt / C;
         for (int b = 0; b < ng; ++b) {
             const int g = (b & 1) ? (ng - 1 - (b >> 1)) : (b >> 1);
-            cols.push_back({(int64_t)nr * C, make_int4((int)i, g, C, 0)});
+            cols.push_back({(int64_t)nr, make_int2((int)i, g)});
         }
     }
     std::stable_sort(rows.begin(), rows.end(), [](auto &x, auto &y) { return x.first > y.first; });
     std::stable_sort(cols.begin(), cols.end(), [](auto &x, auto &y) { return x.first > y.first; });
-    std::vector<int2> hr;
-    std::vector<int4> hc;
+    std::vector<int2> hr, hc;
     for (auto &x : rows) hr.push_back(x.second);
     for (auto &x : cols) hc.push_back(x.second);
     cudaError_t e = cudaMalloc(&ctx->row_items, sizeof(int2) * hr.size());
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->col_items, sizeof(int4) * hc.size());
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->counter, 2 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->col_items, sizeof(int2) * hc.size());
     if (e == cudaSuccess) e = cudaMemcpy(ctx->row_items, hr.data(), sizeof(int2) * hr.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(ctx->col_items, hc.data(), sizeof(int4) * hc.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(ctx->counter, 0, 2 * sizeof(unsigned));
-    if (e == cudaSuccess) e = prepare_rows_batch<float>(smem);
+    if (e == cudaSuccess) e = cudaMemcpy(ctx->col_items, hc.data(), sizeof(int2) * hc.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = prepare_rows_batch<float>(th);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch work lists");
     ctx->nrow_items = (int)hr.size();
     ctx->ncol_items = (int)hc.size();
-    ctx->row_smem = smem;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    ctx->row_grid = sms;          // one 512-thread CTA per SM (128 registers)
-    ctx->col_grid = 2 * sms;      // column CTAs use fewer registers
+    ctx->row_th = th;
+    ctx->col_max_nr = max_nr;
     return FCN_OK;
 }
 
@@ -1837,28 +1859,30 @@ int create_impl(int n, const fcn_grid *grids, const fcn_params *params, int prec
         cudaMemset(pu.rho, 0, rsize(prec) * np);
         cudaMemset(pu.stats, 0, sizeof(double) * NSTAT * pu.g.nr);
         if (prec == FCN_FP64) {
-            const cx<double> *tw;
+            const cx<double> *tw, *tw2;
             const double *lo, *hi;
             if ((e = get_twiddles<double>(pu.g.nt, &tw)) != cudaSuccess ||
+                (e = get_twiddles<double>(fft_tag(pu.g.nt, 2), &tw2)) != cudaSuccess ||
                 (e = get_lohi<double>(pu.g.nr, &lo, &hi, &pu.lo64, &pu.hi64)) != cudaSuccess) {
                 cuda_fail(ctx, e, "constant tables");
                 return bail(FCN_ERR_CUDA);
             }
-            pu.tw = tw; pu.lo = lo; pu.hi = hi;
+            pu.tw = tw; pu.tw2 = tw2; pu.lo = lo; pu.hi = hi;
             if ((e = prepare_rows<double>(pu.g.nt)) != cudaSuccess || (e = prepare_cn<double>()) != cudaSuccess) {
                 cuda_fail(ctx, e, "row kernel attributes");
                 return bail(FCN_ERR_CUDA);
             }
         } else {
-            const cx<float> *tw, *tw1 = nullptr;
+            const cx<float> *tw, *tw2, *tw1 = nullptr;
             const float *lo, *hi;
             if ((e = get_twiddles<float>(pu.g.nt, &tw)) != cudaSuccess ||
+                (e = get_twiddles<float>(fft_tag(pu.g.nt, 2), &tw2)) != cudaSuccess ||
                 (pu.g.nt >= 256 && (e = get_twiddles<float>(fft_tag(pu.g.nt, 1), &tw1)) != cudaSuccess) ||
                 (e = get_lohi<float>(pu.g.nr, &lo, &hi, &pu.lo64, &pu.hi64)) != cudaSuccess) {
                 cuda_fail(ctx, e, "constant tables");
                 return bail(FCN_ERR_CUDA);
             }
-            pu.tw = tw; pu.tw1 = tw1; pu.lo = lo; pu.hi = hi;
+            pu.tw = tw; pu.tw1 = tw1; pu.tw2 = tw2; pu.lo = lo; pu.hi = hi;
             if ((e = prepare_rows<float>(pu.g.nt)) != cudaSuccess || (e = prepare_cn<float>()) != cudaSuccess) {
                 cuda_fail(ctx, e, "row kernel attributes");
                 return bail(FCN_ERR_CUDA);
@@ -1922,7 +1946,6 @@ void fcn_destroy(fcn_ctx *ctx) {
     }
     cudaFree(ctx->row_items);
     cudaFree(ctx->col_items);
-    cudaFree(ctx->counter);
     if (ctx->host_red) cudaFreeHost(ctx->host_red);
     for (int b = 0; b < kMaxBranches; ++b) {
         if (ctx->bst[b]) cudaStreamDestroy(ctx->bst[b]);

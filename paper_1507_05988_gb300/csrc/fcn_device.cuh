@@ -146,19 +146,25 @@ struct NLCoef {
     T hloss;    // h loss, or 0 without MPI loss
     T sat;      // 1 with saturation of the MPI loss (factor 1 - u), else 0
     T is_root;  // sdt^(1/K) / I_s: with j = |A|^2 is_root, sdt (|A|^2/I_s)^K = j^K
+    T kf[2];    // hk[0] inv_is, hk[1] inv_is^2: phi = |A|^2 (kf0 + kf1 |A|^2)
+    int kerr2;  // 1: the Kerr phase has the n2 and n4 terms only and kf holds it exactly
     int K;
     int nkerr;  // number of leading Kerr orders in use (1..4; trailing zeros dropped)
     unsigned flags;
 };
 
 // Pass structure of the row stage's in-place FFT of Nt points and the layout
-// of its twiddle table.  Two decompositions (plans), chosen per grid by the
-// autotuner through the row variant; the last pass is radix 16 in both (a
-// thread's 16 consecutive samples then sit at one position stride):
+// of its twiddle table.  Three decompositions (plans), the first two chosen
+// per grid by the autotuner through the row variant; their last pass is
+// radix 16 (a thread's 16 consecutive samples then sit at one position
+// stride):
 //   plan 0: one radix 2/4/8 pass first for the factor left over by radix 16,
 //           then radix-16 passes (Nt = 4096: 16 16 16);
 //   plan 1 (Nt >= 256): radix-8 passes, one radix 2/4 pass first for the
-//           factor left over, then the radix-16 pass (Nt = 4096: 4 8 8 16).
+//           factor left over, then the radix-16 pass (Nt = 4096: 4 8 8 16);
+//   plan 2 (Nt >= 64, small grids): radix-4 passes after one radix-2 pass for
+//           an odd power of two; 4 values per thread, so that few rows still
+//           give every scheduler a warp.
 // Nt < 16: one pass of radix Nt.  A kernel's Nt template argument carries
 // the plan in its high bits (fft_tag); fft_nt / fft_plan decode it.
 // Twiddle table: for every pass p >= 1 (radix R_p, Ns_p = product of the
@@ -178,12 +184,14 @@ __host__ __device__ constexpr int fft_rem(int nt) { return nt >= 16 ? (1 << (fft
 // radix-8 passes and a radix 2^(m mod 3) pass first
 __host__ __device__ constexpr int fft_m8(int nt) { return fft_log2(nt) - 4; }
 __host__ __device__ constexpr bool fft_plan1(int ntp) { return fft_plan(ntp) == 1 && fft_nt(ntp) >= 256; }
+__host__ __device__ constexpr bool fft_plan2(int ntp) { return fft_plan(ntp) == 2 && fft_nt(ntp) >= 64; }
 __host__ __device__ constexpr int fft_npass(int ntp) {
-    return fft_plan1(ntp) ? (fft_m8(fft_nt(ntp)) % 3 ? 1 : 0) + fft_m8(fft_nt(ntp)) / 3 + 1
+    return fft_plan2(ntp) ? (fft_log2(fft_nt(ntp)) + 1) / 2 : fft_plan1(ntp) ? (fft_m8(fft_nt(ntp)) % 3 ? 1 : 0) + fft_m8(fft_nt(ntp)) / 3 + 1
                           : fft_n16(fft_nt(ntp)) + (fft_rem(fft_nt(ntp)) > 1 ? 1 : 0);
 }
 __host__ __device__ constexpr int fft_radix(int ntp, int p) {
     return fft_nt(ntp) < 16 ? fft_nt(ntp)
+         : fft_plan2(ntp) ? ((fft_log2(fft_nt(ntp)) % 2 && p == 0) ? 2 : 4)
          : fft_plan1(ntp)
              ? (p == fft_npass(ntp) - 1 ? 16
                 : ((fft_m8(fft_nt(ntp)) % 3 && p == 0) ? (1 << (fft_m8(fft_nt(ntp)) % 3)) : 8))
@@ -232,6 +240,7 @@ struct RowArgs {
     NLCoef<T> nl;
     int *err = nullptr;   // set nonzero by a kernel whose bounded wait gave up
     const cx<T> *tw1 = nullptr;   // twiddle table of FFT plan 1 (variants 4, 5)
+    const cx<T> *tw2 = nullptr;   // twiddle table of FFT plan 2 (small grids), or null
     const cx<T> *in = nullptr;    // rows read from here instead of field (output
                                   // still to field; may not alias it), or null
     const cx<T> *cmp = nullptr;   // OP_DIFF: the field compared against, [nr][nt]
@@ -361,16 +370,19 @@ struct ColArgs {
     double disp = 0.0;       // FCN_EXACT_DISPERSION: dk goes here instead, and the
                              // stage multiplies column q by exp(2 i disp q^2)
     int variant;             // 0..3: register chunks, long/short x CTA 256/512;
-                             // 4, 5: cp.async-staged chunks of 16 / 8 rows (FP32);
-                             // 6, 7: register-fed staged chunks of 16 / 8 rows;
+                             // 4..7: block kernel, forms 0..3 (launch_cn_block);
                              // 8: one sequential sweep per column, TMA-fed
-                             // (4..8 need coef)
+                             // (4..8 need coef, 4..7 prod)
     int tp = 0;              // row pitch of invden in complex values (>= nt/2 + 1)
     int *err = nullptr;      // set nonzero by a kernel whose bounded wait gave up
     int pivlim = 0;          // 1 (FP32 context tables): invden holds 1/pivot_j - 1/p_inf(q)
                              // (see piv_limit), applied with the limit as a two-float pair
     const ColConst *cc = nullptr;   // FP32 context tables: per-column constants (|q|)
+    const cx<T> *prod = nullptr;    // products of the sweep factors over kProdRows rows:
+                             // alpha [NP][tp], gamma [NP][tp], NP = ceil(nr / kProdRows)
 };
+template <typename T>
+constexpr int kProdRows = sizeof(T) == 4 ? 8 : 4;
 
 struct TableArgs {
     int nr, nt;
@@ -379,7 +391,14 @@ struct TableArgs {
     int tp = 0;              // row pitch of the table in complex values (0: nt/2 + 1)
     int pivlim = 0;          // FP32: store 1/pivot_j - 1/p_inf(q) (ColArgs::pivlim)
     ColConst *cc = nullptr;  // FP32: per-column constants (tp entries), or none
+    // with cn_table_fills_all also the row coefficients and the products of
+    // the sweep factors (ColArgs::coef, prod), or none
+    CnCoef<float> *coef = nullptr;
+    cx<float> *prod = nullptr;
 };
+// Whether launch_cn_table also fills TableArgs::coef and prod (tall FP32 grids).
+template <typename T>
+constexpr bool cn_table_fills_all(int nr) { return sizeof(T) == 4 && nr >= 128; }
 
 // 1/p_inf(q), the limit of 1/pivot_j for large j in column q: with lo_j,
 // hi_j -> 1 the pivot recurrence piv_j = b + s^2 lo_j hi_{j-1} / piv_{j-1}
@@ -496,7 +515,7 @@ template <typename T>
 cudaError_t launch_cn(const ColArgs<T> &a, cudaStream_t st);
 constexpr int kRowVariants = 6;
 constexpr int kColVariants = 9;
-constexpr int kColStagedFirst = 4;      // variants >= this need ColArgs::coef
+constexpr int kColBlockFirst = 4;       // variants >= this need ColArgs::coef
 constexpr int kColSeq = 8;              // the sequential TMA-fed column kernel (col_seq.cu)
 // Sequential column stage of npulse (1..8) pulses sharing the grid, the
 // coefficients and the pivot table (fields[k], blockIdx.y = k);
@@ -515,24 +534,31 @@ cudaError_t launch_cn_coef(const TableArgs &a, CnCoef<T> *coef, cudaStream_t st)
 // (a.field and field2; a's other arguments serve both).
 template <typename T>
 cudaError_t launch_cn_pair(const ColArgs<T> &a, cx<T> *field2, cudaStream_t st);
-// Sets the staged column kernels' shared-memory attribute (outside capture).
+// Column stage with all rows of a block of columns in registers
+// (col_block.cu), form 0..3; needs a.coef and a.prod.
+// cudaErrorInvalidConfiguration when the grid does not fit.
+template <typename T>
+cudaError_t launch_cn_block(const ColArgs<T> &a, int form, cudaStream_t st);
+// The products a.prod of a finished table (a.invden, a.coef, a.cc).
+template <typename T>
+cudaError_t launch_cn_prod(const ColArgs<T> &a, cx<T> *prod, cudaStream_t st);
+// Sets the paired column kernel's shared-memory attribute (outside capture).
 template <typename T>
 cudaError_t prepare_cn();
 
 // Batched work lists (pulses of uneven grids in one launch per stage).
-// Row items: (pulse, first row), 512/(Nt/16) rows each, Nt in 512..8192.
-// Column items: (pulse, column group); every pulse uses 512-thread CTAs.
-// counter: 2 unsigned, zero before the first launch (kernels reset them).
+// Row items: (pulse, first row), th/(Nt/16) rows each, Nt in 512..8192, th =
+// row_batch_threads of the largest Nt (the CTA size).  Column items: (pulse,
+// group of cn_batch_columns of the largest Nr adjacent columns).
+int row_batch_threads(int max_nt);
 template <typename T>
-cudaError_t launch_rows_batch(const RowArgs<T> *pulses, const int2 *items, int nitems, int ops,
-                              unsigned *counter, size_t smem, int grid, cudaStream_t st);
+cudaError_t launch_rows_batch(const RowArgs<T> *pulses, const int2 *items, int nitems, int ops, int th,
+                              cudaStream_t st);
 template <typename T>
-cudaError_t prepare_rows_batch(size_t smem);
+cudaError_t prepare_rows_batch(int th);
 template <typename T>
-cudaError_t launch_cn_batch(const ColArgs<T> *pulses, const int4 *items, int nitems,
-                            unsigned *counter, int grid, cudaStream_t st);
-// shared-memory bytes of the batched row kernel for rows of nt points
-size_t row_batch_smem(int nt, int bytes_per_complex);
+cudaError_t launch_cn_batch(const ColArgs<T> *pulses, const int2 *items, int nitems, int max_nr, cudaStream_t st);
+int cn_batch_columns(int max_nr);
 
 // Cartesian transverse grid (xy_kernel.cu).  One launch solves the
 // Crank-Nicolson system of every transverse line of one axis for every

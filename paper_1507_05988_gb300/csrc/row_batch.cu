@@ -1,29 +1,48 @@
 // row_batch.cu -- the batched (work-list) row stage: pulses of uneven grids
-// (Nt = 512 ... 8192) in one persistent launch per stage.  FP32 with K = 8,
-// the form the batched path runs in (see row_kernel.cuh for the row body).
+// (Nt = 512 ... 8192) in one launch per stage.  FP32 with K = 8, the form the
+// batched path runs in (see row_kernel.cuh for the row body).
 #include "row_kernel.cuh"
 
 namespace fcn {
 
-size_t row_batch_smem(int nt, int bytes_per_complex) {
-    // 512 threads hold 512 / (Nt/16) rows of Nt + Nt/16 padded values and
-    // as many real u values
-    const int tpr = nt / 16;
-    const int rpc = 512 / tpr;
-    return (size_t)(bytes_per_complex + bytes_per_complex / 2) * rpc * (nt + nt / 16) + sizeof(double) * kRowScratch;
+int row_batch_threads(int max_nt) { return max_nt <= 2048 ? 128 : max_nt <= 4096 ? 256 : 512; }
+
+namespace {
+// A CTA of th threads holds 16 th samples and one padding value per 16,
+// whatever its rows' Nt, and as many u values where they are kept.
+size_t batch_smem(int th, bool with_u) { return (size_t)17 * th * (with_u ? 12 : 8) + sizeof(double) * kRowScratch; }
+
+template <typename F>
+cudaError_t with_threads(int th, F &&f) {
+    if (th == 128) return f(std::integral_constant<int, 128>());
+    if (th == 256) return f(std::integral_constant<int, 256>());
+    return f(std::integral_constant<int, 512>());
+}
+}  // namespace
+
+template <>
+cudaError_t prepare_rows_batch<float>(int th) {
+    return with_threads(th, [&](auto n) {
+        constexpr int TH = decltype(n)::value;
+        cudaError_t e = cudaFuncSetAttribute(row_batch_kernel<float, 8, TH, ROW_PLAIN>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, false));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(row_batch_kernel<float, 8, TH, ROW_OUT>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, true));
+        return e;
+    });
 }
 
 template <>
-cudaError_t prepare_rows_batch<float>(size_t smem) {
-    return cudaFuncSetAttribute(row_batch_kernel<float, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-}
-
-template <>
-cudaError_t launch_rows_batch<float>(const RowArgs<float> *pulses, const int2 *items, int nitems, int ops,
-                                     unsigned *counter, size_t smem, int grid, cudaStream_t st) {
-    row_batch_kernel<float, 8><<<grid, 512, smem, st>>>(pulses, items, nitems, ops, counter);
-    return cudaGetLastError();
+cudaError_t launch_rows_batch<float>(const RowArgs<float> *pulses, const int2 *items, int nitems, int ops, int th,
+                                     cudaStream_t st) {
+    return with_threads(th, [&](auto n) {
+        constexpr int TH = decltype(n)::value;
+        const bool out = (ops & (OP_RHO | OP_STATS | OP_SPEC)) != 0;
+        auto k = out ? row_batch_kernel<float, 8, TH, ROW_OUT> : row_batch_kernel<float, 8, TH, ROW_PLAIN>;
+        k<<<nitems, TH, batch_smem(TH, out), st>>>(pulses, items, ops);
+        return cudaGetLastError();
+    });
 }
 
 }  // namespace fcn

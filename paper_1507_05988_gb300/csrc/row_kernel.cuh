@@ -35,10 +35,24 @@
 // scan of the warp totals.  (+) never cancels (all terms are in [0, 1]), so
 // the scan keeps the relative precision of the working type.
 #pragma once
-#include "fcn_device.cuh"
+#include <type_traits>
+
+#include "pack.cuh"
 
 namespace fcn {
 namespace {
+
+// The element of a thread from the values of its rows (x[0 .. L-1]), and back.
+template <typename V>
+__device__ __forceinline__ cx<V> pack_rows(const cx<typename Pack<V>::S> *x) {
+    if constexpr (Pack<V>::L == 2) return mk(pk2{x[0].x, x[1].x}, pk2{x[0].y, x[1].y});
+    else return x[0];
+}
+template <typename V>
+__device__ __forceinline__ cx<typename Pack<V>::S> row_of(cx<V> v, int lane) {
+    if constexpr (Pack<V>::L == 2) return lane ? mk(v.x.b, v.y.b) : mk(v.x.a, v.y.a);
+    else return v;
+}
 
 constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n / 2); }
 
@@ -52,7 +66,7 @@ template <int NT>
 struct RowCfg {
     static constexpr int N = fft_nt(NT);                    // points per row
     static constexpr int PLAN = fft_plan(NT);               // FFT decomposition
-    static constexpr int E = N < 16 ? N : 16;               // values per thread
+    static constexpr int E = PLAN == 2 ? 4 : N < 16 ? N : 16;   // values per thread
     static constexpr int TPR = N / E;                       // threads per row
     static constexpr int THREADS = TPR >= 256 ? TPR : 256;  // CTA size
     static constexpr int RPC = THREADS / TPR;               // rows per CTA
@@ -122,8 +136,10 @@ __device__ __forceinline__ void c16f_pair2(int m, float *ch, float *cl, float *s
     }
 }
 
-template <typename T, int DIR>
-__device__ __forceinline__ cx<T> rot16(cx<T> o, int m) {
+template <typename V, int DIR>
+__device__ __forceinline__ cx<V> rot16(cx<V> o, int m) {
+    using T = typename Pack<V>::S;
+    const auto K = [](T c) { return Pack<V>::splat(c); };
     m &= 15;
     if (m == 0) return o;
     if (m == 8) return mk(-o.x, -o.y);
@@ -134,19 +150,20 @@ __device__ __forceinline__ cx<T> rot16(cx<T> o, int m) {
             // odd multiples of pi/4: (c, s) = (+-1, +-1)/sqrt(2)
             constexpr float H_HI = 0.70710676908493042f;       // float(1/sqrt 2)
             constexpr float H_LO = 1.2101617485882343e-8f;     // 1/sqrt 2 - H_HI
-            const float sc = (m == 2 || m == 14) ? 1.f : -1.f;             // sign of cos
-            const float ss = float(DIR) * ((m == 2 || m == 6) ? 1.f : -1.f);  // sign of sin
-            const float re = sc * o.x - ss * o.y;
-            const float im = ss * o.x + sc * o.y;
-            return mk(T(fmaf(re, H_HI, re * H_LO)), T(fmaf(im, H_HI, im * H_LO)));
+            const bool sc = m == 2 || m == 14;                 // cos > 0
+            const bool ss = (DIR > 0) == (m == 2 || m == 6);   // sin > 0
+            const V p = o.x + o.y, d = o.x - o.y;
+            const V re = sc ? (ss ? d : p) : (ss ? -p : -d);   // +-x -+ y
+            const V im = sc ? (ss ? p : -d) : (ss ? d : -p);
+            return mk(vfma(re, K(H_HI), re * K(H_LO)), vfma(im, K(H_HI), im * K(H_LO)));
         }
         float ch, cl, sh, sl;
         c16f_pair2(m, &ch, &cl, &sh, &sl);
         if (DIR < 0) { sh = -sh; sl = -sl; }
         // (o.x + i o.y)(c + i s), the lo parts first
-        const float lre = fmaf(o.x, cl, -o.y * sl);
-        const float lim = fmaf(o.x, sl, o.y * cl);
-        return mk(T(fmaf(o.x, ch, fmaf(-o.y, sh, lre))), T(fmaf(o.x, sh, fmaf(o.y, ch, lim))));
+        const V lre = vfma(o.x, K(cl), -o.y * K(sl));
+        const V lim = vfma(o.x, K(sl), o.y * K(cl));
+        return mk(vfma(o.x, K(ch), vfma(-o.y, K(sh), lre)), vfma(o.x, K(sh), vfma(o.y, K(ch), lim)));
     } else {
         const T c = T(cos16(m));
         const T s = T(DIR) * T(cos16(m - 4));
@@ -176,6 +193,8 @@ __device__ __forceinline__ cx<float> csub2(cx<float> a, cx<float> b) {
 }
 __device__ __forceinline__ cx<double> cadd2(cx<double> a, cx<double> b) { return a + b; }
 __device__ __forceinline__ cx<double> csub2(cx<double> a, cx<double> b) { return a - b; }
+__device__ __forceinline__ cx<pk2> cadd2(cx<pk2> a, cx<pk2> b) { return a + b; }
+__device__ __forceinline__ cx<pk2> csub2(cx<pk2> a, cx<pk2> b) { return a - b; }
 
 // In-register DFT of size R (power of two <= 16), natural order in and out,
 // X_k = sum_n x_n exp(DIR 2 pi i n k / R), by radix-2 decimation in time.
@@ -203,28 +222,120 @@ struct Dft {
         }
     }
 };
+// Four-point DFT in place (no multiplications).
+template <int DIR, typename V>
+__device__ __forceinline__ void dft4(cx<V> &a, cx<V> &b, cx<V> &c, cx<V> &d) {
+    const cx<V> p = cadd2(a, c), m = csub2(a, c), q = cadd2(b, d);
+    const V rx = b.x - d.x, ry = b.y - d.y;
+    a = cadd2(p, q);
+    c = csub2(p, q);
+    // m +- DIR i (b - d)
+    b = DIR > 0 ? mk(m.x - ry, m.y + rx) : mk(m.x + ry, m.y - rx);
+    d = DIR > 0 ? mk(m.x + ry, m.y - rx) : mk(m.x - ry, m.y + rx);
+}
+// R = 16 as 4 x 4: with n = 4 n1 + n2 and k = k1 + 4 k2,
+//   X_k = sum_n2 W16^(n2 k1) (sum_n1 x_n W4^(n1 k1)) W4^(n2 k2):
+// 8 rotations (4 by odd multiples of pi/8, 4 of pi/4) against the 10 of the
+// radix-2 recursion.
+template <typename T, int DIR>
+struct Dft<T, 16, DIR> {
+    __device__ __forceinline__ static void run(cx<T> *v) {
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) dft4<DIR>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);   // v[4 k1 + n2]
+#pragma unroll
+        for (int k1 = 1; k1 < 4; ++k1)
+#pragma unroll
+            for (int n2 = 1; n2 < 4; ++n2) v[4 * k1 + n2] = rot16<T, DIR>(v[4 * k1 + n2], n2 * k1);
+        cx<T> x[16];
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            dft4<DIR>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) x[k1 + 4 * k2] = v[4 * k1 + k2];
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = x[k];
+    }
+};
 template <typename T, int DIR>
 struct Dft<T, 1, DIR> {
     __device__ __forceinline__ static void run(cx<T> *) {}
 };
 
-// v * W_e (DIR < 0) or v * conj(W_e) (DIR > 0) for twiddle entry e.  FP32
-// tables hold each twiddle as a two-float pair, 16 bytes per entry
-// (hi.x, hi.y, lo.x, lo.y); FP64 tables one complex double.
-template <typename T, int DIR>
-__device__ __forceinline__ cx<T> tw_mul(cx<T> v, const cx<T> *__restrict__ tw, int e, int entries) {
+// One twiddle as loaded: FP32 tables hold each as a two-float pair, 16 bytes
+// per entry (hi.x, hi.y, lo.x, lo.y); FP64 tables one complex double.
+template <typename T>
+struct Twiddle;
+template <>
+struct Twiddle<float> {
+    float x, y, z, w;
+};
+template <>
+struct Twiddle<double> {
+    double x, y;
+};
+__device__ __forceinline__ Twiddle<float> ld_tw(const cx<float> *__restrict__ tw, int e) {
+    Twiddle<float> r;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+                 : "l"(reinterpret_cast<const float4 *>(tw) + e));
+    return r;
+}
+__device__ __forceinline__ Twiddle<double> ld_tw(const cx<double> *__restrict__ tw, int e) {
+    Twiddle<double> r;
+    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(r.x), "=d"(r.y) : "l"(tw + e));
+    return r;
+}
+
+// v * W (DIR < 0) or v * conj(W) (DIR > 0).
+template <typename V, int DIR>
+__device__ __forceinline__ cx<V> tw_mul(cx<V> v, const Twiddle<typename Pack<V>::S> &w) {
+    using T = typename Pack<V>::S;
     if constexpr (sizeof(T) == 4) {
-        const float4 w = __ldg(reinterpret_cast<const float4 *>(tw) + FCN_IDX(e, entries, 3));
+        const auto K = [](T c) { return Pack<V>::splat(c); };
         const float hy = DIR > 0 ? -w.y : w.y;
         const float ly = DIR > 0 ? -w.w : w.w;
-        const float lre = fmaf(v.x, w.z, -v.y * ly);
-        const float lim = fmaf(v.x, ly, v.y * w.z);
-        return mk(T(fmaf(v.x, w.x, fmaf(-v.y, hy, lre))), T(fmaf(v.x, hy, fmaf(v.y, w.x, lim))));
+        const V lre = vfma(v.x, K(w.z), -v.y * K(ly));
+        const V lim = vfma(v.x, K(ly), v.y * K(w.z));
+        return mk(vfma(v.x, K(w.x), vfma(-v.y, K(hy), lre)), vfma(v.x, K(hy), vfma(v.y, K(w.x), lim)));
     } else {
-        cx<T> w = ldg_cx(&tw[FCN_IDX(e, entries, 3)]);
-        if (DIR > 0) w.y = -w.y;
-        return cmul(v, w);
+        return cmul(v, mk(w.x, DIR > 0 ? -w.y : w.y));
     }
+}
+
+// The thread's twiddles of pass P, m = 0 .. count - 1 in the order the pass
+// uses them (butterfly i, factor r).  The first kTwPre of them are loaded
+// ahead, before the barrier in front of the pass, while the sample registers
+// are free (the samples are in shared memory): their latency is then not
+// waited for behind the operands'.
+constexpr int kTwPre = 8;
+template <int NT, int P>
+struct PassTw {
+    static constexpr int R = PassCfg<NT, P>::R;
+    static constexpr int NS = PassCfg<NT, P>::NS;
+    static constexpr int COUNT = NS > 1 ? RowCfg<NT>::E / R * (R - 1) : 0;
+    static constexpr int PRE = COUNT < kTwPre ? COUNT : kTwPre;
+    __device__ __forceinline__ static int entry(int t, int m) {
+        const int i = m / (R - 1), r = m % (R - 1) + 1;
+        return tw_offset(NT, P) + (r - 1) * NS + ((t + RowCfg<NT>::TPR * i) & (NS - 1));   // P > 0
+    }
+};
+template <typename T>
+struct TwAhead {
+    Twiddle<T> w[kTwPre];
+};
+template <int NT, int P, typename T>
+__device__ __forceinline__ void tw_ahead(TwAhead<T> &a, const cx<T> *__restrict__ tw, int t) {
+    if constexpr (P >= 0 && P < RowCfg<NT>::NPASS) {
+#pragma unroll
+        for (int m = 0; m < PassTw<NT, P>::PRE; ++m)
+            a.w[m] = ld_tw(tw, FCN_IDX((PassTw<NT, P>::entry(t, m)), tw_size(NT), 3));
+    }
+}
+template <int NT, int P, typename T>
+__device__ __forceinline__ Twiddle<T> tw_get(const TwAhead<T> &a, const cx<T> *__restrict__ tw, int t, int m) {
+    if (m < PassTw<NT, P>::PRE) return a.w[m];
+    return ld_tw(tw, FCN_IDX((PassTw<NT, P>::entry(t, m)), tw_size(NT), 3));
 }
 
 // Adjoint of Dft<T, R, -1>: the same butterflies transposed, with the
@@ -255,6 +366,29 @@ struct DftAdj {
     }
 };
 template <typename T>
+struct DftAdj<T, 16> {
+    __device__ __forceinline__ static void run(cx<T> *v) {
+        // the steps of Dft<T, 16, -1> transposed, in reverse order
+        cx<T> x[16];
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) x[4 * k1 + k2] = v[k1 + 4 * k2];
+            dft4<+1>(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);                  // x[4 k1 + n2]
+        }
+#pragma unroll
+        for (int k1 = 1; k1 < 4; ++k1)
+#pragma unroll
+            for (int n2 = 1; n2 < 4; ++n2) x[4 * k1 + n2] = rot16<T, +1>(x[4 * k1 + n2], n2 * k1);
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+            dft4<+1>(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);                                // x[4 n1 + n2]
+#pragma unroll
+            for (int n1 = 0; n1 < 4; ++n1) v[4 * n1 + n2] = x[4 * n1 + n2];
+        }
+    }
+};
+template <typename T>
 struct DftAdj<T, 1> {
     __device__ __forceinline__ static void run(cx<T> *) {}
 };
@@ -263,21 +397,16 @@ struct DftAdj<T, 1> {
 // (operands already in v[i*R + r]).
 template <typename T, int NT, int P>
 __device__ __forceinline__ void pass_compute(cx<T> (&v)[RowCfg<NT>::E], int t,
-                                             const cx<T> *__restrict__ tw) {
-    using C = RowCfg<NT>;
+                                             const cx<typename Pack<T>::S> *__restrict__ tw,
+                                             const TwAhead<typename Pack<T>::S> &ahead) {
     constexpr int R = PassCfg<NT, P>::R;
-    constexpr int NS = PassCfg<NT, P>::NS;
-    constexpr int NB = C::E / R;
-    constexpr int OFF = tw_offset(NT, P);
-    static_assert(R == fft_radix(NT, P) && NS == fft_ns(NT, P), "pass structure");
+    constexpr int NB = RowCfg<NT>::E / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        const int j = t + C::TPR * i;
-        if (NS > 1) {
-            const int k = j & (NS - 1);
+        if (PassTw<NT, P>::COUNT > 0) {
 #pragma unroll
             for (int r = 1; r < R; ++r)
-                v[i * R + r] = tw_mul<T, -1>(v[i * R + r], tw, OFF + (r - 1) * NS + k, tw_size(NT));
+                v[i * R + r] = tw_mul<T, -1>(v[i * R + r], tw_get<NT, P>(ahead, tw, t, i * (R - 1) + r - 1));
         }
         Dft<T, R, -1>::run(&v[i * R]);
     }
@@ -287,27 +416,45 @@ __device__ __forceinline__ void pass_compute(cx<T> (&v)[RowCfg<NT>::E], int t,
 // twiddles.
 template <typename T, int NT, int P>
 __device__ __forceinline__ void pass_compute_adj(cx<T> (&v)[RowCfg<NT>::E], int t,
-                                                 const cx<T> *__restrict__ tw) {
-    using C = RowCfg<NT>;
+                                                 const cx<typename Pack<T>::S> *__restrict__ tw,
+                                                 const TwAhead<typename Pack<T>::S> &ahead) {
     constexpr int R = PassCfg<NT, P>::R;
-    constexpr int NS = PassCfg<NT, P>::NS;
-    constexpr int NB = C::E / R;
-    constexpr int OFF = tw_offset(NT, P);
+    constexpr int NB = RowCfg<NT>::E / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         DftAdj<T, R>::run(&v[i * R]);
-        if (NS > 1) {
-            const int k = (t + C::TPR * i) & (NS - 1);
+        if (PassTw<NT, P>::COUNT > 0) {
 #pragma unroll
             for (int r = 1; r < R; ++r)
-                v[i * R + r] = tw_mul<T, +1>(v[i * R + r], tw, OFF + (r - 1) * NS + k, tw_size(NT));
+                v[i * R + r] = tw_mul<T, +1>(v[i * R + r], tw_get<NT, P>(ahead, tw, t, i * (R - 1) + r - 1));
         }
     }
 }
 
-// Operands of forward pass P (in-place decimation in time): butterfly
-// j = t + TPR i combines the positions base + r NS (r < R), base =
-// (j / NS) NS R + j mod NS, and writes its outputs back to them.
+// Butterfly i of thread t in pass P: the thread's butterflies are adjacent in
+// pass 0 (its positions are then the contiguous E t .. E t + E - 1) and TPR
+// apart in the others.
+template <int NT, int P>
+__device__ __forceinline__ int bfly(int t, int i) {
+    if constexpr (P == 0) return RowCfg<NT>::E / PassCfg<NT, 0>::R * t + i;
+    else return t + RowCfg<NT>::TPR * i;
+}
+
+// Makes what pass P - 1 stored visible to pass P (or the reverse, in the
+// inverse transform).  In plans 0 and 2 every pass from 1 on has one butterfly of
+// radix E per thread, so both passes cover a block of NS_P E positions with
+// the same NS_P consecutive threads: up to 32 of them are one warp, and only
+// the last exchange of rows above 512 points (Nt = 4096: passes 1 and 2)
+// needs the whole CTA.  Measured on the middle launch: see RowForm.
+template <int NT, int P>
+__device__ __forceinline__ void pass_sync() {
+    if constexpr (RowCfg<NT>::PLAN != 1 && fft_ns(NT, P) <= 32) __syncwarp();
+    else __syncthreads();
+}
+
+// Operands of forward pass P (in-place decimation in time): butterfly j
+// combines the positions base + r NS (r < R), base = (j / NS) NS R + j mod NS,
+// and writes its outputs back to them.
 template <typename T, int NT, int P>
 __device__ __forceinline__ void pass_load(cx<T> (&v)[RowCfg<NT>::E], const cx<T> *S, int t) {
     using C = RowCfg<NT>;
@@ -316,7 +463,7 @@ __device__ __forceinline__ void pass_load(cx<T> (&v)[RowCfg<NT>::E], const cx<T>
     constexpr int NB = C::E / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        const int j = t + C::TPR * i;
+        const int j = bfly<NT, P>(t, i);
         const int base = (j / NS) * NS * R + (j & (NS - 1));
 #pragma unroll
         for (int r = 0; r < R; ++r) v[i * R + r] = S[FCN_IDX(pidx(base + r * NS, fft_nt(NT)), C::PADN, 1)];
@@ -331,7 +478,7 @@ __device__ __forceinline__ void pass_store(const cx<T> (&v)[RowCfg<NT>::E], cx<T
     constexpr int NB = C::E / R;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        const int j = t + C::TPR * i;
+        const int j = bfly<NT, P>(t, i);
         const int base = (j / NS) * NS * R + (j & (NS - 1));
 #pragma unroll
         for (int r = 0; r < R; ++r) S[FCN_IDX(pidx(base + r * NS, fft_nt(NT)), C::PADN, 2)] = v[i * R + r];
@@ -341,63 +488,52 @@ __device__ __forceinline__ void pass_store(const cx<T> (&v)[RowCfg<NT>::E], cx<T
 // Inverse transform: the exact adjoint of the forward transform, i.e. the
 // forward passes in reverse order, each applying the transposed butterfly
 // and the conjugate twiddles in place (input already in registers in the
-// last forward pass's order, i.e. natural frequency order; result in S in
-// the forward transform's input order, scaled by sc in its last pass).
-// Every pass reads and writes the same positions in the same thread, so one
-// barrier per pass (before other threads read them) suffices.
-template <typename T, int NT, int P, bool DONE>
-struct InvDispatch;
+// last forward pass's order, i.e. natural frequency order; the result of the
+// last pass, scaled by sc, stays in registers at the positions of forward
+// pass 0, the forward transform's input order).  Every pass reads and writes
+// the same positions in the same thread, so one synchronisation per pass
+// (before other threads read them, pass_sync) suffices.
 template <typename T, int NT, int P>
-struct InvDispatch<T, NT, P, false> {
-    // sc (the 1/Nt of the inverse transform) scales the last pass's outputs
-    __device__ __forceinline__ static void run(cx<T> (&v)[RowCfg<NT>::E], cx<T> *S, int t,
-                                               const cx<T> *tw, T sc) {
-        using C = RowCfg<NT>;
+__device__ __forceinline__ void inverse_fft(cx<T> (&v)[RowCfg<NT>::E], cx<T> *S, int t,
+                                            const cx<typename Pack<T>::S> *tw, TwAhead<typename Pack<T>::S> &ahead,
+                                            typename Pack<T>::S sc) {
+    using C = RowCfg<NT>;
+    if constexpr (P >= 0) {
         if (P + 1 < C::NPASS) pass_load<T, NT, P>(v, S, t);
-        asm volatile("" ::: "memory");
-        pass_compute_adj<T, NT, P>(v, t, tw);
-        if (P == 0) {
+        pass_compute_adj<T, NT, P>(v, t, tw, ahead);
+        if constexpr (P == 0) {
+            // sc: the 1/Nt of the inverse transform
+            const T s = Pack<T>::splat(sc);
 #pragma unroll
-            for (int e = 0; e < C::E; ++e) v[e] = mk(v[e].x * sc, v[e].y * sc);
-        }
-        pass_store<T, NT, P>(v, S, t);
-        __syncthreads();
-        InvDispatch<T, NT, P - 1, (P < 1)>::run(v, S, t, tw, sc);
-    }
-};
-template <typename T, int NT, int P>
-struct InvDispatch<T, NT, P, true> {
-    __device__ __forceinline__ static void run(cx<T> (&)[RowCfg<NT>::E], cx<T> *, int,
-                                               const cx<T> *, T) {}
-};
-
-// Forward transform in place: input in S in the digit-reversed order of
-// tpos, output of the last pass (natural frequency order, positions
-// j + r NS) left in registers for the caller.  The caller's barrier before
-// the first pass makes S complete.
-template <typename T, int NT, int P, bool LAST>
-struct FwdDispatch;
-template <typename T, int NT, int P>
-struct FwdDispatch<T, NT, P, false> {
-    __device__ __forceinline__ static void run(cx<T> (&v)[RowCfg<NT>::E], cx<T> *S, int t,
-                                               const cx<T> *tw) {
-        pass_load<T, NT, P>(v, S, t);
-        // compiler-only fence: the twiddle loads stay behind the operand
-        // loads (issuing them together costs registers the 4-CTA variant lacks)
-        asm volatile("" ::: "memory");
-        pass_compute<T, NT, P>(v, t, tw);
-        if (P + 1 < RowCfg<NT>::NPASS) {
+            for (int e = 0; e < C::E; ++e) v[e] = mk(v[e].x * s, v[e].y * s);
+        } else {
             pass_store<T, NT, P>(v, S, t);
-            __syncthreads();
+            tw_ahead<NT, P - 1>(ahead, tw, t);
+            pass_sync<NT, P>();
+            inverse_fft<T, NT, P - 1>(v, S, t, tw, ahead, sc);
         }
-        FwdDispatch<T, NT, P + 1, (P + 1 >= RowCfg<NT>::NPASS)>::run(v, S, t, tw);
     }
-};
+}
+
+// Forward transform in place: the operands of pass 0 in registers (time
+// samples in the digit-reversed order of tpos), the output of the last pass
+// (natural frequency order, positions j + r NS) left in registers.
 template <typename T, int NT, int P>
-struct FwdDispatch<T, NT, P, true> {
-    __device__ __forceinline__ static void run(cx<T> (&)[RowCfg<NT>::E], cx<T> *, int,
-                                               const cx<T> *) {}
-};
+__device__ __forceinline__ void forward_fft(cx<T> (&v)[RowCfg<NT>::E], cx<T> *S, int t,
+                                            const cx<typename Pack<T>::S> *tw,
+                                            TwAhead<typename Pack<T>::S> &ahead) {
+    using C = RowCfg<NT>;
+    if constexpr (P < C::NPASS) {
+        if constexpr (P > 0) pass_load<T, NT, P>(v, S, t);
+        pass_compute<T, NT, P>(v, t, tw, ahead);
+        if constexpr (P + 1 < C::NPASS) {
+            pass_store<T, NT, P>(v, S, t);
+            tw_ahead<NT, P + 1>(ahead, tw, t);
+            pass_sync<NT, P + 1>();
+        }
+        forward_fft<T, NT, P + 1>(v, S, t, tw, ahead);
+    }
+}
 
 // Padded shared-memory index of the e-th of the E samples a thread owns,
 // whose first sits at unpadded position p0 (tpos): when the sample stride
@@ -455,14 +591,24 @@ __device__ __forceinline__ bool row_io_chunks(const cx<T> *p) {
     else return sizeof(T) == 8 || (reinterpret_cast<uintptr_t>(p) & 15) == 0;
 }
 
+// Field values bypass L1 (each is read once; the twiddle table, read by
+// every row, then stays there).
+__device__ __forceinline__ cx<float> ld_field(const cx<float> *p) {
+    const float2 q = __ldcg(reinterpret_cast<const float2 *>(p));
+    return mk(q.x, q.y);
+}
+__device__ __forceinline__ cx<double> ld_field(const cx<double> *p) {
+    const double2 q = __ldcg(reinterpret_cast<const double2 *>(p));
+    return mk(q.x, q.y);
+}
 template <typename T>
 __device__ __forceinline__ void ld_chunk(const cx<T> *p, cx<T> *v) {
     if constexpr (sizeof(T) == 4) {
-        const float4 q = *reinterpret_cast<const float4 *>(p);
+        const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
         v[0] = mk(q.x, q.y);
         v[1] = mk(q.z, q.w);
     } else {
-        v[0] = *p;
+        v[0] = ld_field(p);
     }
 }
 
@@ -529,12 +675,12 @@ __host__ __device__ __forceinline__ void row_real_chunks(int t, F f) {
 // Nonlinear half step
 // ---------------------------------------------------------------------------
 
-template <typename T>
-__device__ __forceinline__ T ipow(T x, int k) {
-    T r = T(1);
+template <typename V>
+__device__ __forceinline__ V ipow(V x, int k) {
+    V r = Pack<V>::splat(typename Pack<V>::S(1));
     while (k) {
-        if (k & 1) r *= x;
-        x *= x;
+        if (k & 1) r = r * x;
+        x = x * x;
         k >>= 1;
     }
     return r;
@@ -542,13 +688,13 @@ __device__ __forceinline__ T ipow(T x, int k) {
 
 // x^K with K a compile-time constant when KT > 0 (squarings unrolled), the
 // runtime exponent k otherwise.
-template <int KT, typename T>
-__device__ __forceinline__ T powk(T x, int k) {
+template <int KT, typename V>
+__device__ __forceinline__ V powk(V x, int k) {
     if constexpr (KT == 8) {
-        const T x2 = x * x, x4 = x2 * x2;
+        const V x2 = x * x, x4 = x2 * x2;
         return x4 * x4;
     } else if constexpr (KT == 7) {
-        const T x2 = x * x, x4 = x2 * x2;
+        const V x2 = x * x, x4 = x2 * x2;
         return x4 * x2 * x;
     } else {
         return ipow(x, k);
@@ -564,164 +710,26 @@ __device__ __forceinline__ T uplus(T a, T b) { return a + b - a * b; }
 //   6 c = xa + 2 xm t1 + 2 xm t2 + xb t3,
 //   t1 = 1 - xa/2,  t2 = 1 - (xm/2) t1,  t3 = 1 - xm t2.
 // Returns 6 c (the caller folds the 1/6 into the (+) update).
-template <typename T>
-__device__ __forceinline__ T rk4_coef6(T xa, T xb, T xm) {
-    const T t1 = fma(T(-0.5), xa, T(1));
-    const T t2 = fma(T(-0.5) * xm, t1, T(1));
-    const T t3 = fma(-xm, t2, T(1));
-    const T acc = fma(xm + xm, t1 + t2, xa);
-    return fma(xb, t3, acc);
+template <typename V>
+__device__ __forceinline__ V rk4_coef6(V xa, V xb, V xm) {
+    const V one = Pack<V>::splat(typename Pack<V>::S(1)), mh = Pack<V>::splat(typename Pack<V>::S(-0.5));
+    const V t1 = vfma(mh, xa, one);
+    const V t2 = vfma(mh * xm, t1, one);
+    const V t3 = vfma(-xm, t2, one);
+    const V acc = vfma(xm + xm, t1 + t2, xa);
+    return vfma(xb, t3, acc);
 }
 
 // run (+) c for c = c6 / 6: run + c (1 - run)
-template <typename T>
-__device__ __forceinline__ T uplus6(T run, T c6) {
-    return fma(c6, fma(-run, T(1.0 / 6.0), T(1.0 / 6.0)), run);
+template <typename V>
+__device__ __forceinline__ V uplus6(V run, V c6) {
+    const V k = Pack<V>::splat(typename Pack<V>::S(1.0 / 6.0));
+    return vfma(c6, vfma(-run, k, k), run);
 }
 
-template <typename T>
-__device__ __forceinline__ void sincos_t(T x, T *s, T *c);
-// FP32 sine and cosine minus one of a nonlinear phase.  The factor
-// exp(i x) is applied in delta form (A + A (exp(i x) - 1)), because a float
-// cosine that rounds to 1 for small x gives |(cos, sin)|^2 = 1 + x^2 > 1 --
-// a systematic energy gain in the weak tails of the pulse.  Evaluation:
-// |x| < 1e-3: series (next terms below 5e-14);  otherwise Cody & Waite's
-// reduction x = n pi/2 + r with pi/2 split into two floats (n*PIO2_HI exact
-// inside the FMA) and Taylor polynomials of degree 9 (sin) and 10 (cos) on
-// |r| <= pi/4, truncation below 2e-9 and 1.2e-10, with cos r - 1 kept
-// without adding 1 (no cancellation); arguments beyond 1e4 rad, where the
-// two-float reduction loses digits, go to the library.
-__device__ __forceinline__ void sincos_m1_f32(float x, float *s, float *cm1) {
-    if (fabsf(x) < 1.0e-3f) {
-        const float x2 = x * x;
-        *cm1 = -0.5f * x2;
-        *s = fmaf(x * x2, -1.66666666666666666667e-1f, x);
-        return;
-    }
-    if (fabsf(x) > 1.0e4f) {
-        float c;
-        sincosf(x, s, &c);
-        *cm1 = c - 1.0f;
-        return;
-    }
-    constexpr float TWO_OVER_PI = 0.636619772367581343076f;
-    constexpr float PIO2_HI = 1.57079637050628662109f;       // float nearest pi/2
-    constexpr float PIO2_LO = -4.37113900018624283e-8f;       // pi/2 - PIO2_HI
-    const float n = rintf(x * TWO_OVER_PI);
-    float r = fmaf(-n, PIO2_HI, x);
-    r = fmaf(-n, PIO2_LO, r);
-    const float r2 = r * r;
-    // sin r = r - r^3/3! + r^5/5! - r^7/7! + r^9/9!
-    float ps = fmaf(r2, 2.75573192239858906526e-6f, -1.98412698412698412698e-4f);
-    ps = fmaf(r2, ps, 8.33333333333333333333e-3f);
-    ps = fmaf(r2, ps, -1.66666666666666666667e-1f);
-    const float sr = fmaf(r * r2, ps, r);
-    // cos r - 1 = -r^2/2! + r^4/4! - r^6/6! + r^8/8! - r^10/10!
-    float pc = fmaf(r2, -2.75573192239858906526e-7f, 2.48015873015873015873e-5f);
-    pc = fmaf(r2, pc, -1.38888888888888888889e-3f);
-    pc = fmaf(r2, pc, 4.16666666666666666667e-2f);
-    pc = fmaf(r2, pc, -0.5f);
-    const float crm1 = r2 * pc;
-    const float cr = crm1 + 1.0f;
-    switch (int(n) & 3) {
-        case 0: *s = sr; *cm1 = crm1; break;
-        case 1: *s = cr; *cm1 = -sr - 1.0f; break;
-        case 2: *s = -sr; *cm1 = -cr - 1.0f; break;
-        default: *s = -cr; *cm1 = sr - 1.0f; break;
-    }
-}
-
-// exp(x) - 1 in FP32: the loss exponent is tiny except near the peak; the
-// series x + x^2/2 is exact to float rounding there (x^3/6 < 2e-13).
-__device__ __forceinline__ float expm1_f32(float x) {
-    if (fabsf(x) < 1.0e-4f) return fmaf(0.5f * x, x, x);
-    return expm1f(x);
-}
-
-template <typename T>
-__device__ __forceinline__ void sincos_t(T x, T *s, T *c);
-template <>
-__device__ __forceinline__ void sincos_t<double>(double x, double *s, double *c) { sincos(x, s, c); }
-template <typename T>
-__device__ __forceinline__ T exp_t(T x);
-template <>
-__device__ __forceinline__ float exp_t<float>(float x) { return expf(x); }
-template <>
-__device__ __forceinline__ double exp_t<double>(double x) { return exp(x); }
-
-// A <- A exp(h N(Ihat, u)) with h folded into the coefficients:
-//   phi = Ihat (hk0 + Ihat (hk1 + Ihat (hk2 + Ihat hk3))) - hplasma u,
-//   lnamp = -hloss Ihat^(K-1) (1 - sat u),  A <- A exp(lnamp + i phi).
-// nl_terms gives (phi, lnamp); ihKm1 = Ihat^(K-1).
-template <typename T>
-__device__ __forceinline__ void nl_terms(T ih, T ihKm1, T u, const NLCoef<T> &c, T *phi, T *lnamp) {
-    T p = fma(ih, c.hk[3], c.hk[2]);
-    p = fma(ih, p, c.hk[1]);
-    p = fma(ih, p, c.hk[0]);
-    *phi = fma(-c.hplasma, u, ih * p);
-    *lnamp = -(c.hloss * fma(-c.sat, u, T(1))) * ihKm1;
-}
-
-// FP32 delta form: A + A D with D = amp exp(i phi) - 1
-//   = (em1 + cm1 + em1 cm1) + i s (1 + em1),  em1 = amp - 1.
-// A D is formed first and added to A with one rounding per component.
-// Folding the terms into A one FMA at a time (A + first-order part, then +
-// second-order part) rounds A plus the first-order part before the
-// second-order part (dre ~ -phi^2/2, a few ulps of A or less) is added, and
-// that rounding is not unbiased: it dropped part of the modulus-reducing
-// term and raised |A| by ~1e-8 of the energy per step on a Kerr-phase pulse
-// (an FP32 emulation of both orders: +9.7e-9 against -2.5e-11 per
-// application at phi up to 2e-3).
-__device__ __forceinline__ cx<float> nl_delta(cx<float> a, float sn, float cm1, float em1) {
-    const float dre = fmaf(em1, cm1, em1 + cm1);
-    const float dim = fmaf(sn, em1, sn);
-    const float dx = fmaf(a.x, dre, -(a.y * dim));
-    const float dy = fmaf(a.y, dre, a.x * dim);
-    return mk(a.x + dx, a.y + dy);
-}
-
-// Small arguments (|phi| < 1e-3, |lnamp| < 1e-4): the series of sin, cos - 1
-// and exp - 1 are exact to float rounding there (see sincos_m1_f32 and
-// expm1_f32 for the bounds).
-__device__ __forceinline__ bool nl_small(float phi, float lnamp) {
-    return fabsf(phi) < 1.0e-3f && fabsf(lnamp) < 1.0e-4f;
-}
-__device__ __forceinline__ cx<float> nl_apply_small(cx<float> a, float phi, float lnamp) {
-    const float p2 = phi * phi;
-    const float cm1 = -0.5f * p2;
-    const float sn = fmaf(phi * p2, -1.66666666666666666667e-1f, phi);
-    const float em1 = fmaf(0.5f * lnamp, lnamp, lnamp);
-    return nl_delta(a, sn, cm1, em1);
-}
-
-template <typename T>
-__device__ __forceinline__ cx<T> nl_apply_terms(cx<T> a, T phi, T lnamp);
-
-// The update of a group of points that is not all small-argument, kept out
-// of line: the unrolled nonlinear loop inlines only the common FP32
-// small-argument path (the general one is rare: the pulse's core).
-template <typename T>
-__device__ __noinline__ cx<T> nl_apply_general(cx<T> a, T phi, T lnamp) {
-    return nl_apply_terms<T>(a, phi, lnamp);
-}
-
-template <typename T>
-__device__ __forceinline__ cx<T> nl_apply_terms(cx<T> a, T phi, T lnamp) {
-    if constexpr (sizeof(T) == 4) {
-        if (nl_small(phi, lnamp)) return nl_apply_small(a, phi, lnamp);
-        float sn, cm1;
-        sincos_m1_f32(phi, &sn, &cm1);
-        return nl_delta(a, sn, cm1, expm1_f32(lnamp));
-    } else {
-        T s, co;
-        sincos_t<T>(phi, &s, &co);
-        const T amp = exp_t<T>(lnamp);
-        return cmul(a, mk(amp * co, amp * s));
-    }
-}
-
-// Exclusive (+)-scan of one value per thread across the TPR threads of a row.
-// Returns the carry entering this thread.  FP64 carries between warps.
+// Exclusive (+)-scan of one value per thread and row across the TPR threads
+// of a unit.  Returns the carry entering this thread.  FP64 carries between
+// warps.
 template <typename T, int NT>
 __device__ __forceinline__ T row_scan_exclusive(T tot, int t, double *scr, int rloc) {
     using C = RowCfg<NT>;
@@ -738,7 +746,6 @@ __device__ __forceinline__ T row_scan_exclusive(T tot, int t, double *scr, int r
     if (lane == 0) excl = T(0);
     if (C::WARPS_PER_ROW > 1) {
         const int w = t >> 5;
-        double *ws = scr + rloc * C::WARPS_PER_ROW;
         if (lane == 31) scr[FCN_IDX(rloc * C::WARPS_PER_ROW + w, 32, 14)] = double(incl);
         __syncthreads();
         if (t < 32) {
@@ -765,132 +772,368 @@ __device__ __forceinline__ T row_scan_exclusive(T tot, int t, double *scr, int r
     return excl;
 }
 
-// One nonlinear half step of this thread's E contiguous points p = E t + e
-// of the row in S (natural order, padded, already scaled), in place.  Two
-// phases: (A) the RK4 coefficients of the cells (p, p+1) -- the last one
-// needs the next thread's first point -- and the thread-local exclusive
-// (+)-scan into U, then the row scan for the carry; (B) the update
-// A <- A exp(h N), four points per iteration of a rolled loop (one copy of
-// the rare general-argument code keeps the kernel small).  STORE_U writes the
-// final u_p back to U (statistics, rho output).  Callers put a barrier
-// between two half steps (phase A reads the neighbour's point).
-template <typename T, int NT, int KT, bool STORE_U>
-__device__ __forceinline__ void nl_half_smem(cx<T> *S, T *U, int t, const NLCoef<T> &c, bool need_u,
-                                             double *scr, int rloc) {
+template <typename T>
+constexpr double u_idle();
+
+// u = rho/rho_nt along tau of the unit's rows: in, U[position] = |A|^2 of
+// every sample (positions of tpos, padded; complete for every thread); out,
+// U[position] = u.  Each thread owns E contiguous points p = E t + e: the RK4
+// coefficients of the cells (p, p+1) (the last one needs the next thread's
+// first point), the thread's own exclusive (+)-scan in registers, then the
+// row scan for the carry that enters it.  Ends with a barrier.  Out of line:
+// few rows need it in most launches (nl_plan), and inlined it would weigh on
+// the register allocation of the path that all others take.
+template <typename V, int NT, int KT, int MB>
+__device__ __noinline__ void u_rows(V *U, int t, const NLCoef<typename Pack<V>::S> *cp, double *scr, int rloc) {
     using C = RowCfg<NT>;
-    constexpr int E = C::E;
+    using T = typename Pack<V>::S;
+    constexpr int E = C::E, L = Pack<V>::L;
     constexpr int NSL = PassCfg<NT, C::NPASS - 1>::NS;
     static_assert(PassCfg<NT, C::NPASS - 1>::R == E, "a thread's samples differ in the last digit only");
+    const V isr = Pack<V>::splat(cp->is_root), half = Pack<V>::splat(T(0.5));
+    const int K = cp->K;
     // the thread's samples tau = E t + e sit at p0 + e NSL (tpos)
     const int p0 = tpos<NT>(E * t);
     const int q0 = pidx(p0, fft_nt(NT));
     const bool last_thread = (t == C::TPR - 1);
-    // |A|^2 of the thread's points and of the next thread's first point
-    T cn[E + 1];
+    // j = |A|^2 is_root: x = dtau sigma_K Ihat^K = j^K
+    V jv[E + 1];
 #pragma unroll
-    for (int e = 0; e < E; ++e) cn[e] = cnorm(S[FCN_IDX((own_idx<NT, NSL>(q0, p0, e)), C::PADN, 8)]);
-    cn[E] = last_thread ? T(0) : cnorm(S[FCN_IDX(pidx(tpos<NT>(E * (t + 1)), fft_nt(NT)), C::PADN, 8)]);
-    T cmax = T(0);
-#pragma unroll
-    for (int e = 0; e < E; ++e) cmax = fmax(cmax, cn[e]);
-    T carry = T(0), umax = T(0);
+    for (int e = 0; e < E; ++e) jv[e] = U[FCN_IDX((own_idx<NT, NSL>(q0, p0, e)), C::PADN, 8)] * isr;
+    jv[E] = last_thread ? Pack<V>::splat(T(0)) : U[FCN_IDX(pidx(tpos<NT>(E * (t + 1)), fft_nt(NT)), C::PADN, 8)] * isr;
     // the thread's exclusive local prefixes of the (+)-scan; u at point e is
-    // carry (+) lp[e] once the carry is known (registers: U exists only when
-    // the caller keeps u for rho or statistics)
-    T lp[E];
+    // carry (+) lp[e] once the carry is known
+    V lp[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) lp[e] = T(0);
-    if (need_u) {
-        T run = T(0);
-        // j = |A|^2 is_root: x = dtau sigma_K Ihat^K = j^K
-        T jv[E + 1];
+    for (int e = 0; e < E; ++e) lp[e] = Pack<V>::splat(T(0));
+    V run = Pack<V>::splat(T(0));
+    T jmax = T(0);
 #pragma unroll
-        for (int e = 0; e <= E; ++e) jv[e] = cn[e] * c.is_root;
-        T jmax = T(0);
+    for (int e = 0; e <= E; ++e) {
+        if constexpr (L == 2) jmax = fmaxf(jmax, fmaxf(jv[e].a, jv[e].b));
+        else jmax = fmax(jmax, jv[e]);
+    }
+    // Where every j^K of the thread's cells underflows to zero (the pulse's
+    // wings), every RK4 increment is exactly zero and u keeps its entering
+    // value: the arithmetic below would give the same bits.
+    if (!(KT == 8 && jmax < T(u_idle<T>()))) {
+        V ja = jv[0];
+        V xa = powk<KT>(ja, K);
 #pragma unroll
-        for (int e = 0; e <= E; ++e) jmax = fmax(jmax, jv[e]);
-        // Where every j^K of the thread's cells underflows to zero (the pulse's
-        // wings: j^8 rounds to 0 for j below 2.4e-6 in FP32, 4e-41 in FP64),
-        // every RK4 increment is exactly zero and u keeps its entering value:
-        // the arithmetic below would give the same bits.
-        const bool idle = (KT == 8) && jmax < (sizeof(T) == 4 ? T(2e-6) : T(1e-41));
-        if (!idle) {
-            T ja = jv[0];
-            T xa = powk<KT>(ja, c.K);
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                lp[e] = run;
-                if ((e + 1 < E) || !last_thread) {
-                    const T jb = jv[e + 1];
-                    const T xb = powk<KT>(jb, c.K);
-                    const T xm = powk<KT>(T(0.5) * (ja + jb), c.K);
-                    run = uplus6(run, rk4_coef6(xa, xb, xm));
-                    ja = jb;
-                    xa = xb;
-                }
+        for (int e = 0; e < E; ++e) {
+            lp[e] = run;
+            if ((e + 1 < E) || !last_thread) {
+                const V jb = jv[e + 1];
+                const V xb = powk<KT>(jb, K);
+                const V xm = powk<KT>(half * (ja + jb), K);
+                run = uplus6(run, rk4_coef6(xa, xb, xm));
+                ja = jb;
+                xa = xb;
             }
         }
+    }
+    V carry;
+    if constexpr (L == 2) {
+        carry.a = row_scan_exclusive<T, NT>(run.a, t, scr, rloc);
+        if (C::WARPS_PER_ROW > 1) __syncthreads();          // the scratch is reused
+        carry.b = row_scan_exclusive<T, NT>(run.b, t, scr, rloc);
+    } else {
         carry = row_scan_exclusive<T, NT>(run, t, scr, rloc);
-        umax = uplus(carry, run);      // u only grows along tau
     }
-    const T omc = T(1) - carry;
-    if constexpr (sizeof(T) == 4) {
-        // FP32: where |phi| and |lnamp| stay below 2^-27 at every point of the
-        // thread (the pulse's wings), exp(lnamp + i phi) - 1 is below 1/8 ulp
-        // of 1 and the update leaves A as it is to float rounding; bounds
-        // from the largest |A|^2 and the largest u (the scan's right end).
-        const T ihm = cmax * c.inv_is;
-        const T pk = fabsf(c.hk[0]) + ihm * (fabsf(c.hk[1]) + ihm * (fabsf(c.hk[2]) + ihm * fabsf(c.hk[3])));
-        const T phib = ihm * pk + fabsf(c.hplasma) * umax;
-        const T lnab = fabsf(c.hloss) * powk<(KT > 0 ? KT - 1 : 0)>(ihm, c.K - 1);
-        if (phib < T(7.450580596923828e-9) && lnab < T(7.450580596923828e-9)) {
-            if (STORE_U && need_u) {
+    const V omc = Pack<V>::splat(T(1)) - carry;
+    __syncthreads();                                        // every thread has read its neighbour's |A|^2
 #pragma unroll
-                for (int e = 0; e < E; ++e)
-                    U[FCN_IDX((own_idx<NT, NSL>(q0, p0, e)), C::PADN, 28)] = fma(lp[e], omc, carry);
+    for (int e = 0; e < E; ++e) U[FCN_IDX((own_idx<NT, NSL>(q0, p0, e)), C::PADN, 28)] = vfma(lp[e], omc, carry);
+    __syncthreads();
+}
+
+// j below which j^8 rounds to zero (j^8 < half the smallest denormal: 2.4e-6
+// in FP32, 4e-41 in FP64).
+template <typename T>
+constexpr double u_idle() { return sizeof(T) == 4 ? 2e-6 : 1e-41; }
+
+// ---- the nonlinear step of rows that ionise too little to matter ----
+// Where, over a whole row, the plasma phase and the loss exponent stay below
+// a small part of the rounding of the field (nl_plan: 2^-32 in FP32, 2^-61 in
+// FP64, against the 2^-25 and 2^-54 that rounding A itself can turn it by),
+// the half step is the Kerr rotation alone,
+//   A <- A exp(i h sum_j kerr_j |A|^(2 j + 2)),
+// pointwise: no scan along tau, so the samples can stay in the registers
+// they leave the inverse transform in and enter the forward one from.  That
+// takes 6 of 11 block barriers and 3 shared-memory round trips per point out
+// of the middle launch.  The two half steps of a middle launch stay two
+// rotations with their own roundings: a run continued from its saved field
+// (closing, then opening half step) has the same bits as one that was not
+// interrupted.
+// Only the rows through a filament's core ionise more (|A|^2 above ~2e16
+// W/m^2 for 2 mm steps); they take u_rows and nl_full.
+//
+// u at the end of the row is at most Nt max(c) with c <= max j^K (the RK4
+// increment's weights add up to 1 and every factor is in [0, 1]).
+// Returns -1: full half step; 0: nothing to do; 1..4: range of the phase
+// (nl_kerr): below 1/16 (FP32) or 2^-12 (FP64), 1/64 (FP64 only), 0.78 (no
+// reduction needed), 1e4.  Monotone in cmax.
+template <typename T, int NT, int KT>
+__device__ __forceinline__ int nl_plan(float cmax, const NLCoef<T> &c) {
+    constexpr float kNeg = sizeof(T) == 4 ? 2.3283064e-10f : 4.3368087e-19f;       // 2^-32, 2^-61
+    constexpr float kSkip = sizeof(T) == 4 ? 7.450580596923828e-9f : 6.9388939e-18f;  // 2^-27, 2^-57
+    constexpr float kSmall = sizeof(T) == 4 ? 0.0625f : 2.44140625e-4f;
+    constexpr float kMid = sizeof(T) == 4 ? 0.0f : 0.015625f;
+    const float ihm = cmax * float(c.inv_is);
+    const float pk = fabsf(float(c.hk[0])) +
+                     ihm * (fabsf(float(c.hk[1])) + ihm * (fabsf(float(c.hk[2])) + ihm * fabsf(float(c.hk[3]))));
+    const float phib = ihm * pk;
+    const float ub = float(fft_nt(NT)) * powk<KT>(cmax * float(c.is_root), c.K);
+    const float plb = fabsf(float(c.hplasma)) * ub;
+    const float lnb = fabsf(float(c.hloss)) * powk<(KT > 0 ? KT - 1 : 0)>(ihm, c.K - 1);
+    if (plb < kNeg && lnb < kNeg && phib < 1.0e4f)
+        return phib < kSkip ? 0 : phib < kSmall ? 1 : phib < kMid ? 2 : phib < 0.78f ? 3 : 4;
+    return -1;                                     // also for NaN or infinite bounds
+}
+
+// Largest part of the thread's values in modulus, as ordered unsigned bits
+// (float: its bits; double: its high word; NaN above infinity).  The largest
+// |A|^2 lies between its square and twice that.
+template <typename V, int E>
+__device__ __forceinline__ unsigned thread_max(const cx<V> (&v)[E]) {
+    if constexpr (sizeof(typename Pack<V>::S) == 8) {
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            m = max(m, max((unsigned)__double2hiint(v[e].x) & 0x7fffffffu, (unsigned)__double2hiint(v[e].y) & 0x7fffffffu));
+        return m;
+    } else {
+        float m = 0.f;
+        auto acc = [&](float x, float y) {
+            asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(fabsf(x)));
+            asm("max.NaN.f32 %0, %0, %1;" : "+f"(m) : "f"(fabsf(y)));
+        };
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if constexpr (Pack<V>::L == 2) {
+                acc(v[e].x.a, v[e].y.a);
+                acc(v[e].x.b, v[e].y.b);
+            } else {
+                acc(v[e].x, v[e].y);
             }
-            return;
         }
+        return __float_as_uint(m);
     }
-    constexpr int UN = E >= 4 ? 4 : E;
-#pragma unroll
-    for (int e0 = 0; e0 < E; e0 += UN) {
-        cx<T> x[UN];
-        T u[UN];
-#pragma unroll
-        for (int k = 0; k < UN; ++k) {
-            const int ip = own_idx<NT, NSL>(q0, p0, e0 + k);
-            x[k] = S[FCN_IDX(ip, C::PADN, 27)];
-            u[k] = need_u ? fma(lp[e0 + k], omc, carry) : T(0);
-        }
-        T phi[UN], lna[UN];
-#pragma unroll
-        for (int k = 0; k < UN; ++k) {
-            const T ih = cnorm(x[k]) * c.inv_is;
-            nl_terms(ih, powk<(KT > 0 ? KT - 1 : 0)>(ih, c.K - 1), u[k], c, &phi[k], &lna[k]);
-        }
-        bool small = false;
-        if constexpr (sizeof(T) == 4) {
-            small = true;
-#pragma unroll
-            for (int k = 0; k < UN; ++k) small = small && nl_small(phi[k], lna[k]);
-        }
-        if (small) {
-            // the common case, decided once for the group of points
-#pragma unroll
-            for (int k = 0; k < UN; ++k) {
-                if constexpr (sizeof(T) == 4)
-                    S[own_idx<NT, NSL>(q0, p0, e0 + k)] = nl_apply_small(x[k], phi[k], lna[k]);
-            }
+}
+
+// Bound of |A|^2 over the CTA's rows from the threads' thread_max, rounded
+// up to float, in every thread (NaN or an overflow reads as NaN or infinity).
+// One block barrier; two calls in a row take different halves of the scratch
+// (slot 0, 1).
+template <int TH, typename T>
+__device__ __forceinline__ float cta_bound(unsigned m, double *scr, int slot) {
+    unsigned *ws = reinterpret_cast<unsigned *>(scr) + 16 * slot;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if constexpr (TH > 32) {
+        if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = m;
+        __syncthreads();
+        m = __reduce_max_sync(0xffffffffu, ws[threadIdx.x & (TH / 32 - 1)]);
+    }
+    float f;
+    if constexpr (sizeof(T) == 8) f = __double2float_ru(__hiloint2double((int)(m + 1), 0));
+    else f = __uint_as_float(m);
+    return f * f * 2.00001f;
+}
+
+// sin(phi) = phi (1 + phi^2 ps) and cos(phi) - 1 = phi^2 pc for |phi| below
+// the tier's bound (nl_plan): Taylor polynomials, the terms left out below
+// 2^-33 (FP32) and 2^-58 (FP64) of the result's scale.
+template <int TIER, typename V>
+__device__ __forceinline__ void expi_poly(V p2, V *ps_out, V *pc_out) {
+    using T = typename Pack<V>::S;
+    const auto K = [](double c) { return Pack<V>::splat(T(c)); };
+    V ps, pc;
+    if constexpr (TIER == 1) {
+        ps = vfma(p2, K(8.33333333333333333333e-3), K(-1.66666666666666666667e-1));
+        pc = vfma(p2, K(4.16666666666666666667e-2), K(-0.5));
+    } else {
+        if constexpr (sizeof(T) == 4 || TIER == 2) {
+            ps = vfma(p2, K(2.75573192239858906526e-6), K(-1.98412698412698412698e-4));
+            pc = vfma(p2, K(-2.75573192239858906526e-7), K(2.48015873015873015873e-5));
         } else {
-#pragma unroll
-            for (int k = 0; k < UN; ++k) S[own_idx<NT, NSL>(q0, p0, e0 + k)] = nl_apply_general(x[k], phi[k], lna[k]);
+            ps = vfma(p2, K(2.81145725434552076320e-15), K(-7.64716373181981647590e-13));
+            ps = vfma(p2, ps, K(1.60590438368216145994e-10));
+            ps = vfma(p2, ps, K(-2.50521083854417187751e-8));
+            ps = vfma(p2, ps, K(2.75573192239858906526e-6));
+            ps = vfma(p2, ps, K(-1.98412698412698412698e-4));
+            pc = vfma(p2, K(4.77947733238738529743e-14), K(-1.14707455977297247139e-11));
+            pc = vfma(p2, pc, K(2.08767569878680989792e-9));
+            pc = vfma(p2, pc, K(-2.75573192239858906526e-7));
+            pc = vfma(p2, pc, K(2.48015873015873015873e-5));
         }
-        if (STORE_U) {
+        ps = vfma(p2, ps, K(8.33333333333333333333e-3));
+        ps = vfma(p2, ps, K(-1.66666666666666666667e-1));
+        pc = vfma(p2, pc, K(-1.38888888888888888889e-3));
+        pc = vfma(p2, pc, K(4.16666666666666666667e-2));
+        pc = vfma(p2, pc, K(-0.5));
+    }
+    *ps_out = ps;
+    *pc_out = pc;
+}
+
+// Quadrant n of the reduced angle: (sin r, cos r - 1) -> (sin x, cos x - 1)
+// for x = n pi/2 + r (cos - 1 kept without adding 1 where n = 0).
+template <typename T>
+__device__ __forceinline__ void expi_quadrant(int n, T &s, T &cm1) {
+    const T sr = s, cr = cm1 + T(1);
+    const T s1 = (n & 1) ? cr : sr, c1 = (n & 1) ? sr : cr;
+    s = (n & 2) ? -s1 : s1;
+    const T c = ((n + 1) & 2) ? -c1 : c1;
+    if (n & 3) cm1 = c - T(1);
+}
+
+// sin(phi) and cos(phi) - 1 for |phi| < 1e4: Cody & Waite's reduction
+// phi = n pi/2 + r with pi/2 as two words (n PIO2_HI exact inside the FMA),
+// then the polynomials for |r| < pi/4.
+template <typename V>
+__device__ __forceinline__ void expi_m1_reduced(V phi, V *s, V *cm1) {
+    using T = typename Pack<V>::S;
+    constexpr T HI = sizeof(T) == 4 ? T(1.57079637050628662109) : T(1.57079632679489655800);
+    constexpr T LO = sizeof(T) == 4 ? T(-4.37113900018624283e-8) : T(6.12323399573676603587e-17);
+    if constexpr (Pack<V>::L == 2) {
+        const pk2 n = {rintf(phi.a * 0.636619772367581343076f), rintf(phi.b * 0.636619772367581343076f)};
+        V r = vfma(-n, Pack<V>::splat(HI), phi);
+        r = vfma(-n, Pack<V>::splat(LO), r);
+        const V r2 = r * r;
+        V ps, pc;
+        expi_poly<3, V>(r2, &ps, &pc);
+        *s = vfma(r * r2, ps, r);
+        *cm1 = r2 * pc;
+        expi_quadrant<float>(int(n.a), s->a, cm1->a);
+        expi_quadrant<float>(int(n.b), s->b, cm1->b);
+    } else {
+        const T n = rint(phi * T(0.636619772367581343076));
+        V r = vfma(-n, HI, phi);
+        r = vfma(-n, LO, r);
+        const V r2 = r * r;
+        V ps, pc;
+        expi_poly<3, V>(r2, &ps, &pc);
+        *s = vfma(r * r2, ps, r);
+        *cm1 = r2 * pc;
+        expi_quadrant<T>(int(n), *s, *cm1);
+    }
+}
+
+// A <- A exp(i phi) for the thread's values, in delta form (A +
+// A (exp(i phi) - 1), one rounding per component; see nl_full).  Below pi/4
+// the common factor phi of sin and cos - 1 enters last:
+//   A + phi (A (phi pc + i (1 + phi^2 ps))).
+// With Kerr orders n2 and n4 alone (NLCoef::kerr2) phi comes from |A|^2 with
+// the intensity scale (a power of two) in the coefficients.
+template <int TIER, bool KERR2, typename V, int E, typename T = typename Pack<V>::S>
+__device__ __forceinline__ void nl_kerr_tier(cx<V> (&v)[E], const NLCoef<T> &c) {
+    const auto K = [](T x) { return Pack<V>::splat(x); };
 #pragma unroll
-            for (int k = 0; k < UN; ++k) U[FCN_IDX((own_idx<NT, NSL>(q0, p0, e0 + k)), C::PADN, 31)] = u[k];
+    for (int e = 0; e < E; ++e) {
+        const cx<V> a = v[e];
+        const V i2 = vfma(a.x, a.x, a.y * a.y);
+        V phi;
+        if constexpr (KERR2) {
+            phi = i2 * vfma(i2, K(c.kf[1]), K(c.kf[0]));
+        } else {
+            const V ih = i2 * K(c.inv_is);
+            V p = vfma(ih, K(c.hk[3]), K(c.hk[2]));
+            p = vfma(ih, p, K(c.hk[1]));
+            phi = ih * vfma(ih, p, K(c.hk[0]));
+        }
+        if constexpr (TIER == 4) {
+            V s, cm1;
+            expi_m1_reduced<V>(phi, &s, &cm1);
+            const V dx = vfma(a.x, cm1, -(a.y * s));
+            const V dy = vfma(a.y, cm1, a.x * s);
+            v[e] = mk(a.x + dx, a.y + dy);
+        } else {
+            const V p2 = phi * phi;
+            V ps, pc;
+            expi_poly<TIER, V>(p2, &ps, &pc);
+            const V s1 = vfma(p2, ps, K(T(1))), c1 = phi * pc;
+            const V tx = vfma(a.x, c1, -(a.y * s1));
+            const V ty = vfma(a.y, c1, a.x * s1);
+            v[e] = mk(vfma(phi, tx, a.x), vfma(phi, ty, a.y));
         }
     }
+}
+template <typename V, int E, typename T = typename Pack<V>::S>
+__device__ __forceinline__ void nl_kerr(cx<V> (&v)[E], const NLCoef<T> &c, int tier) {
+    if (tier <= 0) return;
+    if (!c.kerr2) return nl_kerr_tier<4, false, V, E>(v, c);      // n6, n8 terms: one form for every phase
+    if (tier == 1) nl_kerr_tier<1, true, V, E>(v, c);
+    else if (sizeof(T) == 8 && tier == 2) nl_kerr_tier<2, true, V, E>(v, c);
+    else if (tier == 3) nl_kerr_tier<3, true, V, E>(v, c);
+    else nl_kerr_tier<4, true, V, E>(v, c);
+}
+
+// exp(x) - 1: the loss exponent is tiny except near the peak, where the
+// series is exact to rounding (FP32: x^3/6 < 2e-13; FP64: x^6/720 < 2e-27).
+__device__ __forceinline__ float expm1_of(float x) {
+    if (fabsf(x) < 1.0e-4f) return fmaf(0.5f * x, x, x);
+    return expm1f(x);
+}
+__device__ __forceinline__ double expm1_of(double x) {
+    if (fabs(x) < 1.0e-4) {
+        double p = fma(x, 1.0 / 120.0, 1.0 / 24.0);
+        p = fma(x, p, 1.0 / 6.0);
+        p = fma(x, p, 0.5);
+        return fma(x * x, p, x);
+    }
+    return expm1(x);
+}
+__device__ __forceinline__ pk2 expm1_of(pk2 x) { return {expm1_of(x.a), expm1_of(x.b)}; }
+// sin and cos - 1 of any finite phase: the reduction of tier 3 where it
+// holds, the library beyond.
+template <typename V>
+__device__ __forceinline__ void expi_any(V phi, V *s, V *cm1) {
+    using T = typename Pack<V>::S;
+    expi_m1_reduced<V>(phi, s, cm1);
+    auto far = [](T x, T *sn, T *cm) {
+        if (!(fabs(x) < T(1.0e4))) {
+            T c;
+            if constexpr (sizeof(T) == 4) sincosf(x, sn, &c);
+            else sincos(x, sn, &c);
+            *cm = c - T(1);
+        }
+    };
+    if constexpr (Pack<V>::L == 2) {
+        far(phi.a, &s->a, &cm1->a);
+        far(phi.b, &s->b, &cm1->b);
+    } else {
+        far(phi, s, cm1);
+    }
+}
+
+// The full half step A <- A exp(h N(|A|^2, u)) of one value, with h and the
+// physics switches folded into the coefficients:
+//   phi = Ihat (hk0 + Ihat (hk1 + Ihat (hk2 + Ihat hk3))) - hplasma u,
+//   lnamp = -hloss Ihat^(K-1) (1 - sat u),  A <- A exp(lnamp + i phi),
+// in delta form: A D with D = amp exp(i phi) - 1 = (em1 + cm1 + em1 cm1) +
+// i s (1 + em1), em1 = amp - 1, formed first and added to A with one rounding
+// per component.  (A float cosine that rounds to 1 for small phases gives
+// |(cos, sin)|^2 = 1 + phi^2 > 1, a systematic energy gain in the pulse's
+// weak tails; and folding the terms into A one FMA at a time rounds A plus
+// the first-order part before the second-order part is added, which raised
+// |A| by ~1e-8 of the energy per step on a Kerr-phase pulse.)
+template <int KT, typename V, typename T = typename Pack<V>::S>
+__device__ __forceinline__ cx<V> nl_full(cx<V> a, V u, const NLCoef<T> &c) {
+    const auto K = [](T x) { return Pack<V>::splat(x); };
+    const V ih = vfma(a.x, a.x, a.y * a.y) * K(c.inv_is);
+    V p = vfma(ih, K(c.hk[3]), K(c.hk[2]));
+    p = vfma(ih, p, K(c.hk[1]));
+    p = vfma(ih, p, K(c.hk[0]));
+    const V phi = vfma(K(-c.hplasma), u, ih * p);
+    const V lna = -(K(c.hloss) * vfma(K(-c.sat), u, K(T(1)))) * powk<(KT > 0 ? KT - 1 : 0)>(ih, c.K - 1);
+    V s, cm1;
+    expi_any<V>(phi, &s, &cm1);
+    const V em1 = expm1_of(lna);
+    const V dre = vfma(em1, cm1, em1 + cm1);
+    const V dim = vfma(s, em1, s);
+    const V dx = vfma(a.x, dre, -(a.y * dim));
+    const V dy = vfma(a.y, dre, a.x * dim);
+    return mk(a.x + dx, a.y + dy);
 }
 
 // Reduction of NV FP64 values across the TPR threads of a row in one pass
@@ -944,6 +1187,13 @@ struct KahanF {
         c = (t2 - s) - y;
         s = t2;
     }
+    __device__ __forceinline__ double sum() const { return double(s) - double(c); }
+};
+template <typename T>
+struct PlainSum {
+    T s = T(0);
+    __device__ __forceinline__ void add(T v) { s += v; }
+    __device__ __forceinline__ double sum() const { return double(s); }
 };
 
 // MB: minimum resident CTAs per SM requested from the compiler (register cap
@@ -951,80 +1201,49 @@ struct KahanF {
 // One CTA of TH threads processes rows [row_base, row_base + TH/TPR) of one
 // pulse: TH = RowCfg<NT>::THREADS in the per-Nt kernels, 512 in the batched
 // work-list kernel.  Every thread of the CTA must call it (barriers inside).
-struct NoHook {
-    __device__ __forceinline__ void operator()() const {}
+enum : int { ROW_PLAIN = 0, ROW_OUT = 1, ROW_DIFF = 2 };
+// The buffers of one pulse (RowArgs names them).
+template <typename T>
+struct RowBufs {
+    cx<T> *field;
+    T *rho;
+    double *stats;
+    const cx<T> *in, *cmp;
+    double *diff;
 };
 
-// The time-domain store of a row (when `store`) and the step-doubling norm's
-// sums of the stored row A against cmp (diff[2 row] = sum |cmp - A|^2,
-// diff[2 row + 1] = sum |A|^2; per-thread sums in the working precision over
-// the thread's few points, FP64 from the row sum on).  Called by every
-// thread of the CTA (row_reduce has block barriers).
-template <typename T, int NT>
-__device__ __forceinline__ void row_store_diff(cx<T> *g, const cx<T> *S, const cx<T> *cmp, double *diff, int nr,
-                                               int row, int t, bool valid, bool store, double *scr, int rloc) {
+// One row stage of TH / TPR units of rows (a unit: one row, or the two
+// adjacent rows of a pair); row_base: the first unit's first row.  PF: the
+// input rows were staged in shared memory (xs: the units' rows of Nt values
+// in natural order, row_base's first) and are read from there; hook() runs
+// once every thread has finished reading them (the prefetch of the next rows
+// may then overwrite xs).
+//
+// MODE: what the kernel is compiled for -- ROW_PLAIN: neither rho nor
+// statistics (the launches of almost every z-step), ROW_OUT: also those,
+// ROW_DIFF: also the step-doubling norm's sums (OP_DIFF).  The code of the
+// outputs then does not weigh on the register allocation of the others.
+template <typename V, int NT, int KT, int TH, int MB, int MODE>
+__device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
+                                         const RowBufs<typename Pack<V>::S> &bf, int row_base, int ops,
+                                         unsigned char *smem_raw) {
+    using T = typename Pack<V>::S;
+    constexpr bool DIFFK = MODE == ROW_DIFF;
     using C = RowCfg<NT>;
     constexpr int E = C::E;
-    T d2 = T(0), b2 = T(0);
-    const cx<T> *gc = cmp ? cmp + (size_t)(valid ? row : 0) * C::N : nullptr;
-    auto acc = [&](cx<T> x, cx<T> y) {             // x: stored value, y: compared value
-        const T dx = y.x - x.x, dy = y.y - x.y;
-        d2 = fma(dx, dx, fma(dy, dy, d2));
-        b2 = fma(x.x, x.x, fma(x.y, x.y, b2));
-    };
-    if (store && valid) {
-        if (row_io_chunks<T, NT>(g) && (!gc || row_io_chunks<T, NT>(gc))) {
-            using IO = RowIo<T, NT>;
-            row_chunks<T, NT>(t, [&](int tau, int cq0, int cp0) {
-                cx<T> cv[IO::CPC];
-#pragma unroll
-                for (int m = 0; m < IO::CPC; ++m)
-                    cv[m] = S[FCN_IDX((own_idx<NT, IO::NSL>(cq0, cp0, (tau & 15) + m)), C::PADN, 11)];
-                st_chunk<T>(g + FCN_IDX(tau, IO::N - IO::CPC + 1, 10), cv);
-                if (gc) {
-                    cx<T> yv[IO::CPC];
-                    ld_chunk<T>(gc + FCN_IDX(tau, IO::N - IO::CPC + 1, 32), yv);
-#pragma unroll
-                    for (int m = 0; m < IO::CPC; ++m) acc(cv[m], yv[m]);
-                }
-            });
-        } else {
-#pragma unroll
-            for (int i = 0; i < E; ++i) {
-                const int idx = t + C::TPR * i;
-                const cx<T> x = S[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 11)];
-                g[FCN_IDX(idx, fft_nt(NT), 10)] = x;
-                if (gc) acc(x, gc[FCN_IDX(idx, fft_nt(NT), 32)]);
-            }
-        }
-    }
-    double v2[2] = {double(d2), double(b2)};
-    const bool sk[2] = {false, false};
-    row_reduce<NT, 2>(v2, sk, t, scr, rloc);
-    if (t == 0 && valid && diff) {
-        diff[FCN_IDX((size_t)2 * row, (size_t)2 * nr, 33)] = v2[0];
-        diff[FCN_IDX((size_t)2 * row + 1, (size_t)2 * nr, 34)] = v2[1];
-    }
-    __syncthreads();                               // the scratch is reused
-}
-
-// One row stage of RPC rows.  PF: the input rows were staged in shared memory
-// (xs: RPC rows of Nt values in natural order, row_base's first) and are read
-// from there; hook() runs once every thread has finished reading them (the
-// prefetch of the next rows may then overwrite xs).
-template <typename T, int NT, int KT, int TH, bool PF = false, typename Hook = NoHook, bool DIFFK = false>
-__device__ __forceinline__ void row_body(const RowArgs<T> &a, int row_base, int ops,
-                                         unsigned char *smem_raw, const cx<T> *xs = nullptr,
-                                         Hook hook = Hook(), const RowMultiArgs<T> *mp = nullptr) {
-    using C = RowCfg<NT>;
-    constexpr int E = C::E;
+    constexpr int L = Pack<V>::L;
     constexpr int RPC = TH / C::TPR;
+    constexpr int PL = C::NPASS - 1;
+    constexpr int RL = PassCfg<NT, PL>::R;
+    constexpr int NSL = PassCfg<NT, PL>::NS;
     static_assert(RPC * C::TPR == TH, "CTA size must hold whole rows");
     // shared memory: the rows S, the FP64 scratch, then the u rows U, which
     // only launches with rho or statistics output allocate
-    cx<T> *S_all = reinterpret_cast<cx<T> *>(smem_raw);
+    cx<V> *S_all = reinterpret_cast<cx<V> *>(smem_raw);
     double *scr = reinterpret_cast<double *>(S_all + RPC * C::PADN);
-    T *U_all = reinterpret_cast<T *>(scr + kRowScratch);
+    // u rows: behind the scratch where they are kept for an output, else in
+    // the storage of S (the samples are then in registers)
+    V *U_all = MODE == ROW_PLAIN ? reinterpret_cast<V *>(smem_raw) : reinterpret_cast<V *>(scr + kRowScratch);
 
 #ifdef FCN_CHECKED
     {
@@ -1032,146 +1251,196 @@ __device__ __forceinline__ void row_body(const RowArgs<T> &a, int row_base, int 
         asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
         const bool with_u = (ops & (OP_RHO | OP_STATS)) != 0;
         if (threadIdx.x == 0)
-            FCN_IDX((sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * RPC * C::PADN + sizeof(double) * kRowScratch - 1,
+            FCN_IDX((sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * L * RPC * C::PADN + sizeof(double) * kRowScratch - 1,
                     dsm, 25);
     }
 #endif
     const int tid = threadIdx.x;
     const int rloc = tid / C::TPR;
     const int t = tid - rloc * C::TPR;
-    const int row = row_base + rloc;
+    const int row = row_base + rloc * L;             // the unit's first row
     const bool valid = row < a.nr;
-    cx<T> *S = S_all + rloc * C::PADN;
-    T *U = U_all + rloc * C::PADN;
-    cx<T> *g = a.field + (size_t)(valid ? row : 0) * C::N;
-    // the row's input: the field itself, or a separate source (out of place)
-    const cx<T> *gin = a.in ? a.in + (size_t)(valid ? row : 0) * C::N : g;
+    // rows of the unit that exist (a pair's second row is missing at the end
+    // of an odd Nr: it then computes on a copy of the first and stores nothing)
+    const int nrow = min(L, a.nr - row);
+    cx<V> *S = S_all + rloc * C::PADN;
+    V *U = U_all + rloc * C::PADN;
+    cx<T> *g[L];
+    const cx<T> *src[L];                             // the rows' input: the field itself, or a separate source
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        const size_t r = valid ? row + (k < nrow ? k : 0) : 0;
+        g[k] = bf.field + r * C::N;
+        src[k] = bf.in ? bf.in + r * C::N : g[k];
+    }
 
-    cx<T> v[E];
+    cx<V> v[E];
+    bool in_regs = false;                            // v holds the time samples at the positions of pass 0
     if (ops & OP_IFFT) {
         // the inverse's first pass (the adjoint of the last forward pass) takes
         // its operands straight from HBM: X[j + r*NS], j = t + TPR*i, coalesced
-        constexpr int PL = C::NPASS - 1;
-        constexpr int RL = PassCfg<NT, PL>::R;
-        constexpr int NSL = PassCfg<NT, PL>::NS;
-        const cx<T> *src = PF ? xs + rloc * C::N : gin;
 #pragma unroll
         for (int i = 0; i < E / RL; ++i) {
             const int j = t + C::TPR * i;
 #pragma unroll
-            for (int r = 0; r < RL; ++r)
-                v[i * RL + r] = valid ? src[FCN_IDX(j + r * NSL, fft_nt(NT), 4)] : mk(T(0), T(0));
+            for (int r = 0; r < RL; ++r) {
+                cx<T> x[L];
+#pragma unroll
+                for (int k = 0; k < L; ++k)
+                    x[k] = valid ? ld_field(&src[k][FCN_IDX(j + r * NSL, fft_nt(NT), 4)]) : mk(T(0), T(0));
+                v[i * RL + r] = pack_rows<V>(x);
+            }
         }
-        InvDispatch<T, NT, PL, (PL < 0)>::run(v, S, t, C::PLAN ? a.tw1 : a.tw, a.nl.inv_nt);
-        hook();
+        TwAhead<T> ahead;
+        tw_ahead<NT, PL>(ahead, C::PLAN == 2 ? a.tw2 : C::PLAN ? a.tw1 : a.tw, t);
+        inverse_fft<V, NT, PL>(v, S, t, C::PLAN == 2 ? a.tw2 : C::PLAN ? a.tw1 : a.tw, ahead, a.nl.inv_nt);
+        in_regs = true;
     } else {
-        const cx<T> *src = PF ? xs + rloc * C::N : gin;
-        if (!PF && row_io_chunks<T, NT>(src)) {
+        bool chunks = true;
+#pragma unroll
+        for (int k = 0; k < L; ++k) chunks = chunks && row_io_chunks<T, NT>(src[k]);
+        if (chunks) {
             using IO = RowIo<T, NT>;
             row_chunks<T, NT>(t, [&](int tau, int cq0, int cp0) {
-                cx<T> cv[IO::CPC];
-                if (valid) {
-                    ld_chunk<T>(src + FCN_IDX(tau, IO::N - IO::CPC + 1, 6), cv);
-                } else {
+                cx<T> cv[L][IO::CPC];
 #pragma unroll
-                    for (int m = 0; m < IO::CPC; ++m) cv[m] = mk(T(0), T(0));
+                for (int k = 0; k < L; ++k) {
+                    if (valid) {
+                        ld_chunk<T>(src[k] + FCN_IDX(tau, IO::N - IO::CPC + 1, 6), cv[k]);
+                    } else {
+#pragma unroll
+                        for (int m = 0; m < IO::CPC; ++m) cv[k][m] = mk(T(0), T(0));
+                    }
                 }
 #pragma unroll
-                for (int m = 0; m < IO::CPC; ++m)
-                    S[FCN_IDX((own_idx<NT, IO::NSL>(cq0, cp0, (tau & 15) + m)), C::PADN, 5)] = cv[m];
+                for (int m = 0; m < IO::CPC; ++m) {
+                    cx<T> x[L];
+#pragma unroll
+                    for (int k = 0; k < L; ++k) x[k] = cv[k][m];
+                    S[FCN_IDX((own_idx<NT, IO::NSL>(cq0, cp0, (tau & 15) + m)), C::PADN, 5)] = pack_rows<V>(x);
+                }
             });
         } else {
 #pragma unroll
             for (int i = 0; i < E; ++i) {
                 const int idx = t + C::TPR * i;
-                S[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 5)] = valid ? src[FCN_IDX(idx, fft_nt(NT), 6)] : mk(T(0), T(0));
+                cx<T> x[L];
+#pragma unroll
+                for (int k = 0; k < L; ++k) x[k] = valid ? ld_field(&src[k][FCN_IDX(idx, fft_nt(NT), 6)]) : mk(T(0), T(0));
+                S[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 5)] = pack_rows<V>(x);
             }
         }
         __syncthreads();
-        hook();
     }
-
-    // the time-domain stage runs whenever the row passes through tau space
-    // (nonlinear step, statistics, rho output) or the 1/Nt of an inverse
-    // transform has to be applied; it works in place on S
-    const bool time_work = (ops & (OP_NL | OP_STATS | OP_RHO | OP_IFFT)) != 0;
-    if (time_work) {
-        const bool need_u = (a.nl.flags & (PH_PLASMA | PH_MPI_SAT)) || (ops & (OP_RHO | OP_STATS));
-        const bool keep_u = (ops & (OP_RHO | OP_STATS)) != 0;
-        bool have_u = false;
-        const int nhalf = ((ops & OP_NL) ? 1 : 0) + ((ops & OP_NL2) ? 1 : 0);
-        for (int hs = 0; hs < nhalf; ++hs) {
-            if (keep_u && hs + 1 == nhalf)
-                nl_half_smem<T, NT, KT, true>(S, U, t, a.nl, need_u, scr, rloc);
-            else
-                nl_half_smem<T, NT, KT, false>(S, U, t, a.nl, need_u, scr, rloc);
-            have_u = need_u;
+    // the samples to shared memory (complete for every thread), where the
+    // row is needed along tau
+    auto to_smem = [&] {
+        if (in_regs) {
+            pass_store<V, NT, 0>(v, S, t);
             __syncthreads();
+            in_regs = false;
         }
-        // statistics of the final row; rho is written below, coalesced
-        if (ops & (OP_STATS | OP_RHO)) {
-            // v = {sum |A|^2, max |A|^2, max u, count of non-finite |A|^2}
-            double v4[4] = {0.0, 0.0, 0.0, 0.0};
-            if (ops & OP_STATS) {
-                if constexpr (sizeof(T) == 4) {
-                    KahanF ks;
-                    float mxf = 0.f, muf = 0.f, badf = 0.f;
-#pragma unroll 4
-                    for (int e = 0; e < E; ++e) {
-                        const int ip = own_idx<NT, PassCfg<NT, C::NPASS - 1>::NS>(pidx(tpos<NT>(E * t), fft_nt(NT)),
-                                                                                  tpos<NT>(E * t), e);
-                        const cx<T> x = S[FCN_IDX(ip, C::PADN, 29)];
-                        const float i2 = fmaf(x.x, x.x, x.y * x.y);
-                        if (!isfinite(i2)) badf += 1.f;
-                        ks.add(i2);
-                        mxf = fmaxf(mxf, i2);
-                        if (have_u) muf = fmaxf(muf, U[ip]);
-                    }
-                    v4[0] = double(ks.s) - double(ks.c);
-                    v4[1] = mxf;
-                    v4[2] = muf;
-                    v4[3] = badf;
-                } else {
-#pragma unroll 4
-                    for (int e = 0; e < E; ++e) {
-                        const int ip = own_idx<NT, PassCfg<NT, C::NPASS - 1>::NS>(pidx(tpos<NT>(E * t), fft_nt(NT)),
-                                                                                  tpos<NT>(E * t), e);
-                        const cx<T> x = S[FCN_IDX(ip, C::PADN, 29)];
-                        const double i2 = double(x.x) * double(x.x) + double(x.y) * double(x.y);
-                        if (!isfinite(i2)) v4[3] += 1.0;
-                        v4[0] += i2;
-                        v4[1] = fmax(v4[1], i2);
-                        if (have_u) v4[2] = fmax(v4[2], double(U[ip]));
+    };
+
+    const bool keep_u = MODE != ROW_PLAIN && (ops & (OP_RHO | OP_STATS)) != 0;
+    const bool need_u = (a.nl.flags & (PH_PLASMA | PH_MPI_SAT)) || keep_u;
+    const int nhalf = ((ops & OP_NL) ? 1 : 0) + ((ops & OP_NL2) ? 1 : 0);
+    int plan = -1;
+    bool known = false;
+#pragma unroll 1
+    for (int hs = 0; hs < nhalf; ++hs) {
+        if (!in_regs) {
+            pass_load<V, NT, 0>(v, S, t);
+            in_regs = true;
+        }
+        float m = 0.f;
+        if (!known) {
+            m = cta_bound<TH, T>(thread_max<V, E>(v), scr, hs);
+            plan = nl_plan<T, NT, KT>(m, a.nl);
+            // a rotation leaves |A| to a rounding or two, and so the bound
+            // within a factor of 2: unless a tier ends in that range, the
+            // second half step's plan is the same
+            known = !keep_u && plan >= 0 && plan == nl_plan<T, NT, KT>(m * 0.499f, a.nl) &&
+                    plan == nl_plan<T, NT, KT>(m * 2.002f, a.nl);
+        }
+        const bool out_u = MODE != ROW_PLAIN && keep_u && hs + 1 == nhalf;
+        if (plan < 0 || out_u) {
+            // u of every sample into U: through the scan along tau, unless
+            // every increment of the CTA's rows is exactly zero
+            const bool idle = KT == 8 && m * float(a.nl.is_root) < float(u_idle<T>()) && sizeof(T) == 4;
+            auto at = [&](int e) { return FCN_IDX(pidx(E * t + e, fft_nt(NT)), C::PADN, 7); };   // pass 0's positions
+            if (MODE == ROW_PLAIN) __syncthreads();      // U is the storage of S here
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                U[at(e)] = idle ? Pack<V>::splat(T(0)) : vfma(v[e].x, v[e].x, v[e].y * v[e].y);
+            __syncthreads();
+            if (!idle) u_rows<V, NT, KT, MB>(U, t, &a.nl, scr, rloc);
+            if (plan < 0) {
+                const bool with_u = need_u;
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    v[e] = nl_full<KT, V>(v[e], with_u ? U[at(e)] : Pack<V>::splat(T(0)), a.nl);
+            }
+            if (MODE == ROW_PLAIN) __syncthreads();
+        }
+        nl_kerr<V, E>(v, a.nl, plan);
+    }
+    const bool have_u = nhalf > 0;
+    if (keep_u) {
+        if (!in_regs) pass_load<V, NT, 0>(v, S, t);
+        // statistics of the final rows; rho is written below, coalesced
+        if ((ops & OP_STATS) && bf.stats) {
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                // v4 = {sum |A|^2, max |A|^2, max u, count of non-finite |A|^2}
+                double v4[4] = {0.0, 0.0, 0.0, 0.0};
+                std::conditional_t<sizeof(T) == 4, KahanF, PlainSum<T>> ks;
+                T mx = T(0), mu = T(0), bad = T(0);
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const cx<T> x = row_of<V>(v[e], k);
+                    const T i2 = vfma(x.x, x.x, x.y * x.y);
+                    if (!isfinite(i2)) bad += T(1);
+                    ks.add(i2);
+                    mx = fmax(mx, i2);
+                    if (have_u) {
+                        const V u = U[FCN_IDX(pidx(E * t + e, fft_nt(NT)), C::PADN, 7)];
+                        mu = fmax(mu, row_of<V>(mk(u, u), k).x);
                     }
                 }
-            }
-            if ((ops & OP_STATS) && a.stats) {
+                v4[0] = ks.sum();
+                v4[1] = mx;
+                v4[2] = mu;
+                v4[3] = bad;
                 const bool mxk[4] = {false, true, true, false};
                 row_reduce<NT, 4>(v4, mxk, t, scr, rloc);
-                if (t == 0 && valid) {
-                    double *st = a.stats + FCN_IDX((size_t)row * NSTAT, (size_t)a.nr * NSTAT, 23);
+                if (t == 0 && valid && k < nrow) {
+                    double *st = bf.stats + FCN_IDX((size_t)(row + k) * NSTAT, (size_t)a.nr * NSTAT, 23);
                     st[ST_SUM_I] = v4[0];
                     st[ST_MAX_I] = v4[1];
                     if (ops & (OP_NL | OP_NL2)) st[ST_MAX_U] = v4[2];
                     st[ST_NONFINITE] = v4[3];
                 }
             }
-            __syncthreads();
-            if ((ops & OP_RHO) && valid && a.rho) {
-                T *rr = a.rho + (size_t)row * C::N;
+        }
+        if ((ops & OP_RHO) && valid && bf.rho) {
+            auto u_of = [&](int q, int k) {
+                const V u = U[FCN_IDX(q, C::PADN, 30)];
+                return have_u ? row_of<V>(mk(u, u), k).x * a.nl.rho_nt : T(0);
+            };
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                if (k >= nrow) break;
+                T *rr = bf.rho + (size_t)(row + k) * C::N;
                 if (row_io_real_chunks<T, NT>(rr)) {
                     // 16-byte chunks in the sector-wise order of the field rows
                     using IO = RowIoReal<T, NT>;
-                    constexpr int NSL = PassCfg<NT, C::NPASS - 1>::NS;
                     row_real_chunks<T, NT>(t, [&](int tau) {
                         const int cp0 = tpos<NT>(tau & ~15);
                         const int cq0 = pidx(cp0, fft_nt(NT));
                         T w[IO::RC];
 #pragma unroll
-                        for (int m = 0; m < IO::RC; ++m)
-                            w[m] = have_u ? U[FCN_IDX((own_idx<NT, NSL>(cq0, cp0, (tau & 15) + m)), C::PADN, 30)] *
-                                                a.nl.rho_nt
-                                          : T(0);
+                        for (int m = 0; m < IO::RC; ++m) w[m] = u_of(own_idx<NT, NSL>(cq0, cp0, (tau & 15) + m), k);
                         T *dst = rr + FCN_IDX(tau, IO::N - IO::RC + 1, 12);
                         if constexpr (sizeof(T) == 4) *reinterpret_cast<float4 *>(dst) = make_float4(w[0], w[1], w[2], w[3]);
                         else *reinterpret_cast<double2 *>(dst) = make_double2(w[0], w[1]);
@@ -1181,260 +1450,227 @@ __device__ __forceinline__ void row_body(const RowArgs<T> &a, int row_base, int 
 #pragma unroll
                     for (int i = 0; i < E; ++i) {
                         const int idx = t + C::TPR * i;
-                        rr[FCN_IDX(idx, fft_nt(NT), 12)] =
-                            have_u ? U[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 30)] * a.nl.rho_nt : T(0);
+                        rr[FCN_IDX(idx, fft_nt(NT), 12)] = u_of(pidx(tpos<NT>(idx), fft_nt(NT)), k);
                     }
                 }
             }
         }
-        if constexpr (DIFFK) {
-            // the kernels of launches with OP_DIFF: the store and the norm sums
-            // (a multi-pulse launch's per-pulse pointers from its parameters)
-            const bool store = (!(ops & OP_FFT) || (ops & OP_SPEC_OF_TIME)) && !(ops & OP_NOSTORE);
-            const cx<T> *cmp = mp ? mp->cmp[blockIdx.y] : a.cmp;
-            double *diff = mp ? mp->diff[blockIdx.y] : a.diff;
-            row_store_diff<T, NT>(g, S, cmp, diff, a.nr, row, t, valid, store, scr, rloc);
-        } else if ((!(ops & OP_FFT) || (ops & OP_SPEC_OF_TIME)) && !(ops & OP_NOSTORE) && valid) {
-            if (row_io_chunks<T, NT>(g)) {
+    }
+    // the time-domain rows to HBM; DIFFK (the kernels of launches with
+    // OP_DIFF): also the step-doubling norm's sums of each stored row A
+    // against cmp, diff[2 row] = sum |cmp - A|^2, diff[2 row + 1] =
+    // sum |A|^2 (per-thread sums in the working precision over the thread's
+    // few points, FP64 from the row sum on)
+    const bool store = (!(ops & OP_FFT) || (ops & OP_SPEC_OF_TIME)) && !(ops & OP_NOSTORE);
+    T d2[L] = {}, b2[L] = {};
+    const cx<T> *gc[L] = {};
+    double *diff = nullptr;
+    if constexpr (DIFFK) {
+        const cx<T> *cmp = bf.cmp;
+        diff = bf.diff;
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            gc[k] = cmp ? cmp + (size_t)(valid ? row + (k < nrow ? k : 0) : 0) * C::N : nullptr;
+        }
+    }
+    if (store) {
+        to_smem();
+        auto acc = [&](int k, cx<T> x, cx<T> y) {          // x: stored value, y: compared value
+            const T dx = y.x - x.x, dy = y.y - x.y;
+            d2[k] = fma(dx, dx, fma(dy, dy, d2[k]));
+            b2[k] = fma(x.x, x.x, fma(x.y, x.y, b2[k]));
+        };
+        if (valid) {
+            bool chunks = true;
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                chunks = chunks && row_io_chunks<T, NT>(g[k]);
+                if constexpr (DIFFK) chunks = chunks && (!gc[k] || row_io_chunks<T, NT>(gc[k]));
+            }
+            if (chunks) {
                 using IO = RowIo<T, NT>;
                 row_chunks<T, NT>(t, [&](int tau, int cq0, int cp0) {
-                    cx<T> cv[IO::CPC];
+                    cx<V> cv[IO::CPC];
 #pragma unroll
                     for (int m = 0; m < IO::CPC; ++m)
                         cv[m] = S[FCN_IDX((own_idx<NT, IO::NSL>(cq0, cp0, (tau & 15) + m)), C::PADN, 11)];
-                    st_chunk<T>(g + FCN_IDX(tau, IO::N - IO::CPC + 1, 10), cv);
+#pragma unroll
+                    for (int k = 0; k < L; ++k) {
+                        cx<T> x[IO::CPC];
+#pragma unroll
+                        for (int m = 0; m < IO::CPC; ++m) x[m] = row_of<V>(cv[m], k);
+                        if (k < nrow) st_chunk<T>(g[k] + FCN_IDX(tau, IO::N - IO::CPC + 1, 10), x);
+                        if constexpr (DIFFK) {
+                            if (gc[k]) {
+                                cx<T> yv[IO::CPC];
+                                ld_chunk<T>(gc[k] + FCN_IDX(tau, IO::N - IO::CPC + 1, 32), yv);
+#pragma unroll
+                                for (int m = 0; m < IO::CPC; ++m) acc(k, x[m], yv[m]);
+                            }
+                        }
+                    }
                 });
             } else {
 #pragma unroll
                 for (int i = 0; i < E; ++i) {
                     const int idx = t + C::TPR * i;
-                    g[FCN_IDX(idx, fft_nt(NT), 10)] = S[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 11)];
+                    const cx<V> xv = S[FCN_IDX(pidx(tpos<NT>(idx), fft_nt(NT)), C::PADN, 11)];
+#pragma unroll
+                    for (int k = 0; k < L; ++k) {
+                        const cx<T> x = row_of<V>(xv, k);
+                        if (k < nrow) g[k][FCN_IDX(idx, fft_nt(NT), 10)] = x;
+                        if constexpr (DIFFK) {
+                            if (gc[k]) acc(k, x, gc[k][FCN_IDX(idx, fft_nt(NT), 32)]);
+                        }
+                    }
                 }
             }
         }
-        // the in-place transform below overwrites S: every thread's store first
-        if (ops & OP_SPEC_OF_TIME) __syncthreads();
+    }
+    if constexpr (DIFFK) {
+        double v2[2 * L];
+        bool sk[2 * L];
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            v2[2 * k] = double(d2[k]);
+            v2[2 * k + 1] = double(b2[k]);
+            sk[2 * k] = sk[2 * k + 1] = false;
+        }
+        row_reduce<NT, 2 * L>(v2, sk, t, scr, rloc);
+        if (t == 0 && valid && diff) {
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                if (k < nrow) {
+                    diff[FCN_IDX((size_t)2 * (row + k), (size_t)2 * a.nr, 33)] = v2[2 * k];
+                    diff[FCN_IDX((size_t)2 * (row + k) + 1, (size_t)2 * a.nr, 34)] = v2[2 * k + 1];
+                }
+            }
+        }
     }
 
     if (ops & OP_FFT) {
-        FwdDispatch<T, NT, 0, (C::NPASS <= 0)>::run(v, S, t, C::PLAN ? a.tw1 : a.tw);
+        // the in-place transform overwrites S: every thread's reads of it first
+        if (store || keep_u) __syncthreads();
+        if (!in_regs) pass_load<V, NT, 0>(v, S, t);
+        TwAhead<T> ahead;
+        tw_ahead<NT, 0>(ahead, C::PLAN == 2 ? a.tw2 : C::PLAN ? a.tw1 : a.tw, t);
+        forward_fft<V, NT, 0>(v, S, t, C::PLAN == 2 ? a.tw2 : C::PLAN ? a.tw1 : a.tw, ahead);
         // last-pass outputs: index j + r*NS, j = t + TPR*i
-        constexpr int PL = C::NPASS - 1;
-        constexpr int R = PassCfg<NT, PL>::R;
-        constexpr int NS = PassCfg<NT, PL>::NS;
-        constexpr int NB = E / R;
+        constexpr int NB = E / RL;
         if (!(ops & (OP_NOSTORE | OP_SPEC_OF_TIME)) && valid) {
 #pragma unroll
             for (int i = 0; i < NB; ++i) {
                 const int j = t + C::TPR * i;
 #pragma unroll
-                for (int r = 0; r < R; ++r) g[FCN_IDX(j + r * NS, fft_nt(NT), 13)] = v[i * R + r];
-            }
-        }
-        if ((ops & OP_SPEC) && a.stats) {
-            // spectral moments sum_q w^k |A_q|^2, w = signed bin, k = 0, 1, 2
-            double m3[3] = {0.0, 0.0, 0.0};
-            if constexpr (sizeof(T) == 4) {
-                KahanF k0, k1, k2;
+                for (int r = 0; r < RL; ++r) {
 #pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int j = t + C::TPR * i;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int q = j + r * NS;
-                        const float w = float(q < C::N / 2 ? q : q - C::N);
-                        const cx<T> x = v[i * R + r];
-                        const float p2 = fmaf(x.x, x.x, x.y * x.y);
-                        k0.add(p2);
-                        k1.add(w * p2);
-                        k2.add(w * w * p2);
-                    }
-                }
-                m3[0] = double(k0.s) - double(k0.c);
-                m3[1] = double(k1.s) - double(k1.c);
-                m3[2] = double(k2.s) - double(k2.c);
-            } else {
-#pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    const int j = t + C::TPR * i;
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const int q = j + r * NS;
-                        const double w = double(q < C::N / 2 ? q : q - C::N);
-                        const cx<T> x = v[i * R + r];
-                        const double p2 = double(x.x) * double(x.x) + double(x.y) * double(x.y);
-                        m3[0] += p2;
-                        m3[1] += w * p2;
-                        m3[2] += w * w * p2;
-                    }
+                    for (int k = 0; k < L; ++k)
+                        if (k < nrow) g[k][FCN_IDX(j + r * NSL, fft_nt(NT), 13)] = row_of<V>(v[i * RL + r], k);
                 }
             }
-            const bool mxk[3] = {false, false, false};
-            row_reduce<NT, 3>(m3, mxk, t, scr, rloc);
-            if (t == 0 && valid) {
-                double *st = a.stats + FCN_IDX((size_t)row * NSTAT, (size_t)a.nr * NSTAT, 24);
-                st[ST_S0] = m3[0];
-                st[ST_S1] = m3[1];
-                st[ST_S2] = m3[2];
+        }
+        if (MODE != ROW_PLAIN && (ops & OP_SPEC) && bf.stats) {
+#pragma unroll
+            for (int k = 0; k < L; ++k) {
+                // spectral moments sum_q w^k |A_q|^2, w = signed bin, k = 0, 1, 2
+                double m3[3] = {0.0, 0.0, 0.0};
+                if constexpr (sizeof(T) == 4) {
+                    KahanF k0, k1, k2;
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const int j = t + C::TPR * i;
+#pragma unroll
+                        for (int r = 0; r < RL; ++r) {
+                            const int q = j + r * NSL;
+                            const float w = float(q < C::N / 2 ? q : q - C::N);
+                            const cx<T> x = row_of<V>(v[i * RL + r], k);
+                            const float p2 = fmaf(x.x, x.x, x.y * x.y);
+                            k0.add(p2);
+                            k1.add(w * p2);
+                            k2.add(w * w * p2);
+                        }
+                    }
+                    m3[0] = double(k0.s) - double(k0.c);
+                    m3[1] = double(k1.s) - double(k1.c);
+                    m3[2] = double(k2.s) - double(k2.c);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const int j = t + C::TPR * i;
+#pragma unroll
+                        for (int r = 0; r < RL; ++r) {
+                            const int q = j + r * NSL;
+                            const double w = double(q < C::N / 2 ? q : q - C::N);
+                            const cx<T> x = row_of<V>(v[i * RL + r], k);
+                            const double p2 = double(x.x) * double(x.x) + double(x.y) * double(x.y);
+                            m3[0] += p2;
+                            m3[1] += w * p2;
+                            m3[2] += w * w * p2;
+                        }
+                    }
+                }
+                const bool mxk[3] = {false, false, false};
+                row_reduce<NT, 3>(m3, mxk, t, scr, rloc);
+                if (t == 0 && valid && k < nrow) {
+                    double *st = bf.stats + FCN_IDX((size_t)(row + k) * NSTAT, (size_t)a.nr * NSTAT, 24);
+                    st[ST_S0] = m3[0];
+                    st[ST_S1] = m3[1];
+                    st[ST_S2] = m3[2];
+                }
             }
         }
     }
 }
 
-// DIFFK: the kernels for launches with OP_DIFF (the closing launch of a
-// step-doubling attempt); the others are compiled without that code, so
-// that it does not weigh on the register allocation of the launch that runs
-// at almost every z-step.
-template <typename T, int NT, int KT, int MB, bool DIFFK = false>
-__global__ void __launch_bounds__(RowCfg<NT>::THREADS, MB)
-row_kernel(RowArgs<T> a) {
+// Up to kRowMulti pulses of one grid and one set of coefficients in one
+// launch: blockIdx.y selects the pulse (its buffers; all else is shared).
+// One launch over all pulses fills the waves that a launch per pulse leaves
+// part-empty.  TH: CTA size; V = pk2: pairs of rows.
+template <typename V, int NT, int KT, int TH, int MB, int MODE>
+__global__ void __launch_bounds__(TH, MB)
+row_kernel(const __grid_constant__ RowMultiArgs<typename Pack<V>::S> m) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int ROWS = TH / RowCfg<NT>::TPR * Pack<V>::L;
     pdl_enter();
-    if constexpr (DIFFK)
-        row_body<T, NT, KT, RowCfg<NT>::THREADS, false, NoHook, true>(a, blockIdx.x * RowCfg<NT>::RPC, a.ops,
-                                                                       smem_raw);
-    else
-        row_body<T, NT, KT, RowCfg<NT>::THREADS>(a, blockIdx.x * RowCfg<NT>::RPC, a.ops, smem_raw);
-}
-
-// Several pulses of one grid and one set of coefficients in one launch:
-// blockIdx.y selects the pulse (its field, rho and statistics pointers; all
-// else is shared).  One launch over all pulses fills the waves that a launch
-// per pulse leaves part-empty.
-template <typename T, int NT, int KT, int MB, bool DIFFK = false>
-__global__ void __launch_bounds__(RowCfg<NT>::THREADS, MB)
-row_kernel_multi(const __grid_constant__ RowMultiArgs<T> m) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    pdl_enter();
-    RowArgs<T> a = m.a;
-    a.field = m.field[blockIdx.y];
-    a.rho = m.rho[blockIdx.y];
-    a.stats = m.stats[blockIdx.y];
-    a.in = m.in[blockIdx.y];
-    if constexpr (DIFFK)
-        row_body<T, NT, KT, RowCfg<NT>::THREADS, false, NoHook, true>(a, blockIdx.x * RowCfg<NT>::RPC, a.ops,
-                                                                       smem_raw, nullptr, NoHook(), &m);
-    else
-        row_body<T, NT, KT, RowCfg<NT>::THREADS>(a, blockIdx.x * RowCfg<NT>::RPC, a.ops, smem_raw);
-}
-
-// Persistent row stage with the next rows prefetched: each CTA walks the
-// units (RPC consecutive rows of one pulse) u = blockIdx.x, + gridDim.x, ...
-// of the launch's pulses; while it transforms and steps one unit, one bulk
-// copy (cp.async.bulk, completion on an mbarrier) brings the next unit's
-// rows from HBM into a staging buffer, so no thread waits on a global load
-// when a unit starts.  The wait on the mbarrier is bounded (~1 s): after it
-// the CTA records an error code, waits (bounded) for its copy in flight and
-// returns.
-constexpr long long kRowWaitCycles = 1ll << 31;
-
-__device__ __forceinline__ bool row_mbar_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok = 0;
-    const long long t0 = clock64();
-    for (;;) {
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > kRowWaitCycles) return false;
-    }
-}
-
-// Byte offset of the staging buffer: after the rows, the FP64 scratch and
-// (launches with rho or statistics) the u rows, 128-byte aligned.
-template <typename T, int NT>
-__host__ __device__ constexpr size_t pf_stage_offset(bool with_u) {
-    using C = RowCfg<NT>;
-    return ((sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * C::RPC * C::PADN + sizeof(double) * kRowScratch +
-            127) / 128 * 128;
-}
-
-template <typename T, int NT, int KT, int MB>
-__global__ void __launch_bounds__(RowCfg<NT>::THREADS, MB)
-row_kernel_pf(const __grid_constant__ RowMultiArgs<T> m, int npulse, int *err) {
-    using C = RowCfg<NT>;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    pdl_enter();
-    const RowArgs<T> &a0 = m.a;
-    const int upp = (a0.nr + C::RPC - 1) / C::RPC;      // units per pulse
-    const int units = upp * npulse;
-    if ((int)blockIdx.x >= units) return;
-    const bool with_u = (a0.ops & (OP_RHO | OP_STATS)) != 0;
-    cx<T> *xs = reinterpret_cast<cx<T> *>(smem_raw + pf_stage_offset<T, NT>(with_u));
-    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(xs + C::RPC * C::N);
-    auto issue = [&](int u) {                           // thread 0 only
-        const int pulse = u / upp, row0 = (u - pulse * upp) * C::RPC;
-        const int rows = min(C::RPC, a0.nr - row0);
-        const uint32_t bytes = (uint32_t)(rows * C::N * sizeof(cx<T>));
-        const cx<T> *src = (m.in[pulse] ? m.in[pulse] : m.field[pulse]) + (size_t)row0 * C::N;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-            ::"r"((uint32_t)__cvta_generic_to_shared(xs)), "l"(src), "r"(bytes), "r"(bar)
-            : "memory");
-    };
+    const int y = blockIdx.y;
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        issue(blockIdx.x);
-    }
-    __syncthreads();
-    uint32_t parity = 0;
-    for (int u = blockIdx.x; u < units; u += gridDim.x, parity ^= 1u) {
-        if (!row_mbar_wait(bar, parity)) {
-            if (threadIdx.x == 0 && err) atomicExch(err, 2);
-            row_mbar_wait(bar, parity);                 // the copy in flight, bounded
-            return;
+        // the rows of the CTA that takes this one's place, into L2: CTAs
+        // start in order, about kResident after one another
+        constexpr int kResident = 152 * (MB > 1 ? MB : 2);
+        const unsigned n = blockIdx.x + kResident, yn = y + n / gridDim.x, xn = n % gridDim.x;
+        const int row0 = (int)xn * ROWS, rows = min(ROWS, m.a.nr - row0);
+        if (yn < gridDim.y) {
+            const cx<typename Pack<V>::S> *f = (m.in[yn] ? m.in[yn] : m.field[yn]) + (size_t)row0 * fft_nt(NT);
+            const unsigned bytes = (unsigned)(rows * fft_nt(NT) * (int)sizeof(*f)) & ~15u;
+            if (bytes && (reinterpret_cast<uintptr_t>(f) & 15) == 0)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(f), "r"(bytes) : "memory");
         }
-        const int pulse = u / upp, row0 = (u - pulse * upp) * C::RPC;
-        RowArgs<T> a = a0;
-        a.field = m.field[pulse];
-        a.rho = m.rho[pulse];
-        a.stats = m.stats[pulse];
-        const int next = u + gridDim.x;
-        row_body<T, NT, KT, C::THREADS, true>(a, row0, a.ops, smem_raw, xs, [&] {
-            if (threadIdx.x == 0 && next < units) issue(next);
-        });
-        __syncthreads();                                // S and the scratch are reused
     }
+    const RowBufs<typename Pack<V>::S> bf = {m.field[y], m.rho[y], m.stats[y], m.in[y], m.cmp[y], m.diff[y]};
+    row_body<V, NT, KT, TH, MB, MODE>(m.a, bf, blockIdx.x * ROWS, m.a.ops, smem_raw);
 }
 
-// Batched work list: each item (pulse, first row) covers 512 / (Nt/16) rows of
-// one pulse; pulses may have different Nr and Nt (Nt = 512 ... 8192).  A
-// persistent grid pulls items from a global counter, largest rows first.
-template <typename T, int KT>
-__global__ void __launch_bounds__(512, 1)
-row_batch_kernel(const RowArgs<T> *__restrict__ pulses, const int2 *__restrict__ items, int nitems,
-                 int ops, unsigned *counter) {
+// Work list of rows: each CTA takes the item (pulse, first row) of its index,
+// the next TH / (Nt/16) rows of that pulse; pulses may have different Nr and
+// Nt (Nt = 512 ... 16 TH).  TH is the smallest CTA that holds a row of the
+// list's largest Nt: 16 uneven pulses (Nr 64-256, Nt 512 and 1024) run their
+// middle stage in one launch of 128-thread CTAs, five per SM, handed out by
+// the hardware as slots free up (as persistent 512-thread CTAs pulling items
+// from a counter: one per SM, every stage of a row waiting on 16 warps).
+template <typename T, int KT, int TH, int MODE>
+__global__ void __launch_bounds__(TH, TH >= 512 ? 1 : 640 / TH)
+row_batch_kernel(const RowArgs<T> *__restrict__ pulses, const int2 *__restrict__ items, int ops) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int next;
-    for (;;) {
-        if (threadIdx.x == 0) next = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int it = next;
-        __syncthreads();
-        if (it >= nitems) break;
-        const int2 w = items[it];
-        const RowArgs<T> a = pulses[w.x];
-        switch (a.nt) {
-            case 512: row_body<T, 512, KT, 512>(a, w.y, ops, smem_raw); break;
-            case 1024: row_body<T, 1024, KT, 512>(a, w.y, ops, smem_raw); break;
-            case 2048: row_body<T, 2048, KT, 512>(a, w.y, ops, smem_raw); break;
-            case 4096: row_body<T, 4096, KT, 512>(a, w.y, ops, smem_raw); break;
-            default: row_body<T, 8192, KT, 512>(a, w.y, ops, smem_raw); break;
-        }
-        __syncthreads();
-    }
-    // the last CTA out resets the counter for the next launch
-    if (threadIdx.x == 0) {
-        const unsigned done = atomicAdd(counter + 1, 1u) + 1;
-        if (done == gridDim.x) {
-            counter[0] = 0;
-            counter[1] = 0;
-        }
+    constexpr int MB = TH >= 512 ? 1 : 640 / TH;
+    const int2 w = items[blockIdx.x];
+    const RowArgs<T> &a = pulses[w.x];
+    const RowBufs<T> bf = {a.field, a.rho, a.stats, a.in, nullptr, nullptr};
+    if (a.nt == 512) row_body<T, 512, KT, TH, MB, MODE>(a, bf, w.y, ops, smem_raw);
+    else if (a.nt == 1024) row_body<T, 1024, KT, TH, MB, MODE>(a, bf, w.y, ops, smem_raw);
+    else if (a.nt == 2048) row_body<T, 2048, KT, TH, MB, MODE>(a, bf, w.y, ops, smem_raw);
+    else if constexpr (TH >= 256) {
+        if (TH == 256 || a.nt == 4096) row_body<T, 4096, KT, TH, MB, MODE>(a, bf, w.y, ops, smem_raw);
+        else if constexpr (TH >= 512) row_body<T, 8192, KT, TH, MB, MODE>(a, bf, w.y, ops, smem_raw);
     }
 }
 }  // namespace
@@ -1442,165 +1678,163 @@ row_batch_kernel(const RowArgs<T> *__restrict__ pulses, const int2 *__restrict__
 namespace rowimpl {
 
 // Rows S and the FP64 scratch, plus the u rows when the launch outputs rho
-// or statistics.
-template <typename T, int NT>
+// or statistics, of a CTA of TH threads.
+template <typename V, int NT, int TH>
 size_t smem_bytes(bool with_u = true) {
     using C = RowCfg<NT>;
-    return (sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * C::RPC * C::PADN + sizeof(double) * kRowScratch;
+    using T = typename Pack<V>::S;
+    return (sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * Pack<V>::L * (TH / C::TPR) * C::PADN +
+           sizeof(double) * kRowScratch;
 }
 
-// Sets the dynamic shared-memory limit of the kernel; must run before any
-// launch of it (and outside stream capture).
-// Occupancy variants: v = 0 is the compiler's natural allocation; v = 1, 2
-// ask for 3 and 4 CTAs of 256 threads per SM (80 and 64 registers), or 2 CTAs
-// of 512 threads for Nt = 8192.  Only FP32 with K = 8 and Nt >= 256 has
-// variants (smaller rows are cheap; their variants map to v = 0).
-template <int NT>
-constexpr int mb_of(int v) {
-    return RowCfg<NT>::THREADS >= 512 ? (v == 0 ? 1 : 2) : (v == 0 ? 1 : (v == 1 ? 3 : 4));
-}
-
-template <typename T, int NT, int KT, int MB>
-cudaError_t set_smem_attr() {
-    cudaError_t e = cudaSuccess;
-    for (int d = 0; d < 2 && e == cudaSuccess; ++d) {
-        e = cudaFuncSetAttribute(d ? row_kernel<T, NT, KT, MB, true> : row_kernel<T, NT, KT, MB, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<T, NT>());
+// One compiled row kernel: value type, CTA size, minimum CTAs per SM.
+template <typename V_, int NT_, int KT_, int TH_, int MB_>
+struct RowForm {
+    using V = V_;
+    using T = typename Pack<V>::S;
+    static constexpr int NT = NT_, TH = TH_;
+    static constexpr int ROWS = TH / RowCfg<NT>::TPR * Pack<V>::L;       // rows per CTA
+    template <int MODE>
+    static constexpr auto kernel() { return row_kernel<V, NT, KT_, TH, MB_, MODE>; }
+    // Sets the dynamic shared-memory limit; must run before any launch (and
+    // outside stream capture).
+    static cudaError_t prepare() {
+        const int smem = (int)smem_bytes<V, NT, TH>();
+        cudaError_t e = cudaFuncSetAttribute(kernel<ROW_PLAIN>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(d ? row_kernel_multi<T, NT, KT, MB, true> : row_kernel_multi<T, NT, KT, MB, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<T, NT>());
+            e = cudaFuncSetAttribute(kernel<ROW_OUT>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel<ROW_DIFF>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return e;
     }
-    return e;
+    static cudaError_t launch(const RowMultiArgs<T> &m, int npulse, cudaStream_t st) {
+        const bool out = (m.a.ops & (OP_RHO | OP_STATS)) != 0;
+        const size_t smem = smem_bytes<V, NT, TH>(out);
+        const dim3 grid((m.a.nr + ROWS - 1) / ROWS, npulse);
+        auto k = (m.a.ops & OP_DIFF) ? kernel<ROW_DIFF>()
+                 : (out || (m.a.ops & OP_SPEC)) ? kernel<ROW_OUT>() : kernel<ROW_PLAIN>();
+        return launch_k(k, grid, dim3(TH), smem, st, m);
+    }
+};
+
+// The kernels of the row variants (0..5; RowArgs::variant).  CTAs are small
+// (a row's threads, at least 64 or 128): with the same warps per SM, more and
+// smaller CTAs wait less on each other's barriers and leave a shorter last
+// wave (middle launch of 8 x 2048 rows of 2048 points: 182 us in CTAs of 128
+// threads, 193 us in CTAs of 256; one 1350 x 1024 pulse: 12.4 against
+// 16.3 us).  Register caps: about 100 hold a thread's samples and the
+// twiddles in flight (102: 182 us, 64 with twice the warps: 193 us).
+//   0: one row per unit; the only form of FP64, K != 8 and Nt < 256;
+//   1: pairs of rows in packed arithmetic, 128 registers (177 us);
+//   2: one row per unit, 64 registers;
+//   3: the pairs in CTAs of 64 threads (Nt <= 1024) or with more registers
+//      (2048), single rows at 85 registers (4096); 8192: as 0;
+//   4, 5: FFT plan 1 at 3 and 4 CTAs of 256 threads.
+// Which is fastest depends on the number of rows; the autotuner picks.
+template <int NT, int MIN>
+constexpr int th_of() { return RowCfg<NT>::TPR < MIN ? MIN : RowCfg<NT>::TPR; }
+constexpr int at_least_1(int n) { return n < 1 ? 1 : n; }
+
+template <typename T, int NT, int KT>
+using FormNat = RowForm<T, NT, KT, th_of<NT, 64>(), at_least_1((sizeof(T) == 4 ? 640 : 512) / th_of<NT, 64>())>;
+template <int NT>
+using FormPair = RowForm<pk2, NT, 8, th_of<NT, 128>(), at_least_1(512 / th_of<NT, 128>())>;
+template <int NT>
+using FormOcc = RowForm<float, NT, 8, th_of<NT, 128>(), 1024 / th_of<NT, 128>()>;
+template <int NT>
+using FormAlt = std::conditional_t<
+    (RowCfg<NT>::TPR <= 64), RowForm<pk2, NT, 8, th_of<NT, 64>(), 8>,
+    std::conditional_t<(RowCfg<NT>::TPR == 128), RowForm<pk2, NT, 8, th_of<NT, 128>(), 3>,
+                       std::conditional_t<(RowCfg<NT>::TPR == 256), RowForm<float, NT, 8, th_of<NT, 256>(), 3>,
+                                          FormNat<float, NT, 8>>>>;
+template <int NT1>
+using FormPlan1 = RowForm<float, NT1, 8, RowCfg<NT1>::THREADS, (RowCfg<NT1>::THREADS >= 512 ? 1 : 3)>;
+template <int NT1>
+using FormPlan1Occ = RowForm<float, NT1, 8, RowCfg<NT1>::THREADS, 1024 / RowCfg<NT1>::THREADS>;
+
+// Small grids: FFT plan 2, 4 values per thread.  A launch of few rows is
+// latency-bound, and in FP64 each of an SM's four schedulers has a quarter of
+// its FP64 rate: a grid needs a warp on every one of the 608, and 128 x 256
+// points in 16 values per thread are 64 warps (51 us in FP64, 6.2 us in FP32;
+// with plan 2 16.5 and 4.3 us).  thin_rows: rows (of one pulse, so that
+// launches of one and of several pulses agree) below which plan 2 serves
+// variant 0; where the two meet, FP64: 512 x 1024 points (131 us both),
+// 512 x 256 still 31 against 54 us; FP32: 512 x 512 6.3 against 8.3 us, 512 x
+// 256 6.2 us both, 1024 and more points never ahead.
+template <typename T, int NT, int KT>
+using FormThin = RowForm<T, fft_tag(NT, 2), KT, th_of<fft_tag(NT, 2), 64>(), 1>;
+template <typename T, int NT>
+constexpr int thin_rows() {
+    return fft_nt(NT) < 64 || fft_nt(NT) > (sizeof(T) == 8 ? 1024 : 512) ? 0
+           : (sizeof(T) == 8 ? 400000 : 270000) / fft_nt(NT);
 }
 
-// The prefetching persistent variant (3): FP32, K = 8, Nt >= 512; 3 CTAs of
-// 256 threads per SM (the staging buffer leaves no room for a fourth), or
-// 1 CTA of 512 threads for Nt = 8192.
-template <int NT>
-constexpr int mb_pf() { return RowCfg<NT>::THREADS >= 512 ? 1 : 3; }
 template <typename T, int NT>
-constexpr bool has_pf() { return sizeof(T) == 4 && fft_nt(NT) >= 512 && fft_plan(NT) == 0; }
-template <typename T, int NT>
-size_t pf_smem_bytes(bool with_u) {
-    return pf_stage_offset<T, NT>(with_u) + sizeof(cx<T>) * RowCfg<NT>::RPC * RowCfg<NT>::N + 16;
-}
+constexpr bool has_forms() { return sizeof(T) == 4 && fft_nt(NT) >= 256; }
 
 template <typename T, int NT>
 cudaError_t prepare_nt() {
-    cudaError_t e = set_smem_attr<T, NT, 0, 1>();
-    if (e == cudaSuccess) e = set_smem_attr<T, NT, 8, 1>();
-    if constexpr (sizeof(T) == 4 && fft_nt(NT) >= 256) {
-        constexpr int NT1 = fft_tag(NT, 1);
-        if (e == cudaSuccess) e = set_smem_attr<T, NT, 8, mb_of<NT>(1)>();
-        if (e == cudaSuccess) e = set_smem_attr<T, NT, 8, mb_of<NT>(2)>();
-        if (e == cudaSuccess) e = set_smem_attr<T, NT1, 8, mb_of<NT1>(1)>();
-        if (e == cudaSuccess) e = set_smem_attr<T, NT1, 8, mb_of<NT1>(2)>();
+    cudaError_t e = FormNat<T, NT, 0>::prepare();
+    if (e == cudaSuccess) e = FormNat<T, NT, 8>::prepare();
+    if constexpr (thin_rows<T, NT>() > 0) {
+        if (e == cudaSuccess) e = FormThin<T, NT, 0>::prepare();
+        if (e == cudaSuccess) e = FormThin<T, NT, 8>::prepare();
     }
-    if constexpr (has_pf<T, NT>()) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(row_kernel_pf<T, NT, 8, mb_pf<NT>()>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pf_smem_bytes<T, NT>(true));
+    if constexpr (has_forms<T, NT>()) {
+        constexpr int NT1 = fft_tag(NT, 1);
+        if (e == cudaSuccess) e = FormPair<NT>::prepare();
+        if (e == cudaSuccess) e = FormOcc<NT>::prepare();
+        if (e == cudaSuccess) e = FormAlt<NT>::prepare();
+        if (e == cudaSuccess) e = FormPlan1<NT1>::prepare();
+        if (e == cudaSuccess) e = FormPlan1Occ<NT1>::prepare();
     }
     return e;
 }
 
-// Launch of the prefetching variant over npulse pulses: one CTA per SM slot
-// (occupancy queried once), each walking units of RPC rows.
-template <typename T, int NT>
-cudaError_t launch_nt_pf(const RowMultiArgs<T> &m, int npulse, cudaStream_t st) {
-    using C = RowCfg<NT>;
-    if constexpr (!has_pf<T, NT>()) {
-        return cudaErrorInvalidConfiguration;
-    } else {
-        const RowArgs<T> &a = m.a;
-        const bool with_u = (a.ops & (OP_RHO | OP_STATS)) != 0;
-        const size_t smem = pf_smem_bytes<T, NT>(with_u);
-        const int units = (a.nr + C::RPC - 1) / C::RPC * npulse;
-        if (units <= 0) return cudaSuccess;
-        auto k = row_kernel_pf<T, NT, 8, mb_pf<NT>()>;
-        static int slots[2] = {0, 0};
-        int &sl = slots[with_u ? 1 : 0];
-        if (!sl) {
-            int dev = 0, sms = 0, occ = 0;
-            cudaError_t e = cudaGetDevice(&dev);
-            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, C::THREADS, smem);
-            if (e != cudaSuccess) return e;
-            sl = sms * (occ > 0 ? occ : 1);
+// Calls f with the form of the launch's variant (K = 8, the photon number of
+// 800 nm in air: unrolled powers; other K: the generic kernel).
+template <typename T, int NT, typename F>
+cudaError_t with_form(const RowArgs<T> &a, F &&f) {
+    if constexpr (has_forms<T, NT>()) {
+        if (a.nl.K == 8) {
+            constexpr int NT1 = fft_tag(NT, 1);
+            if (a.variant == 1) return f(FormPair<NT>());
+            if (a.variant == 2) return f(FormOcc<NT>());
+            if (a.variant == 3) return f(FormAlt<NT>());
+            if (a.variant == 4 && a.tw1) return f(FormPlan1<NT1>());
+            if (a.variant == 5 && a.tw1) return f(FormPlan1Occ<NT1>());
         }
-        const int grid = units < sl ? units : sl;
-        return launch_k(k, dim3(grid), dim3(C::THREADS), smem, st, m, npulse, a.err);
     }
-}
-
-// The kernel of the launch's variant (K = 8: unrolled powers; other K: the
-// generic kernel), compiled with the norm sums (DIFFK) or without.
-template <typename T, int NT, bool DIFFK>
-auto multi_kernel_for(const RowArgs<T> &a) -> void (*)(const RowMultiArgs<T>) {
-    if (a.nl.K != 8) return row_kernel_multi<T, NT, 0, 1, DIFFK>;
-    void (*k)(const RowMultiArgs<T>) = row_kernel_multi<T, NT, 8, 1, DIFFK>;
-    if constexpr (sizeof(T) == 4 && fft_nt(NT) >= 256) {
-        constexpr int NT1 = fft_tag(NT, 1);
-        if (a.variant == 1) k = row_kernel_multi<T, NT, 8, mb_of<NT>(1), DIFFK>;
-        else if (a.variant == 2) k = row_kernel_multi<T, NT, 8, mb_of<NT>(2), DIFFK>;
-        else if (a.variant == 4 && a.tw1) k = row_kernel_multi<T, NT1, 8, mb_of<NT1>(1), DIFFK>;
-        else if (a.variant == 5 && a.tw1) k = row_kernel_multi<T, NT1, 8, mb_of<NT1>(2), DIFFK>;
+    if constexpr (thin_rows<T, NT>() > 0) {
+        if (a.tw2 && a.nr < thin_rows<T, NT>()) {
+            if (a.nl.K == 8) return f(FormThin<T, NT, 8>());
+            return f(FormThin<T, NT, 0>());
+        }
     }
-    return k;
-}
-
-template <typename T, int NT, bool DIFFK>
-auto kernel_for(const RowArgs<T> &a) -> void (*)(RowArgs<T>) {
-    if (a.nl.K != 8) return row_kernel<T, NT, 0, 1, DIFFK>;
-    void (*k)(RowArgs<T>) = row_kernel<T, NT, 8, 1, DIFFK>;
-    if constexpr (sizeof(T) == 4 && fft_nt(NT) >= 256) {
-        constexpr int NT1 = fft_tag(NT, 1);
-        if (a.variant == 1) k = row_kernel<T, NT, 8, mb_of<NT>(1), DIFFK>;
-        else if (a.variant == 2) k = row_kernel<T, NT, 8, mb_of<NT>(2), DIFFK>;
-        else if (a.variant == 4 && a.tw1) k = row_kernel<T, NT1, 8, mb_of<NT1>(1), DIFFK>;
-        else if (a.variant == 5 && a.tw1) k = row_kernel<T, NT1, 8, mb_of<NT1>(2), DIFFK>;
-    }
-    return k;
+    if (a.nl.K == 8) return f(FormNat<T, NT, 8>());
+    return f(FormNat<T, NT, 0>());
 }
 
 template <typename T, int NT>
 cudaError_t launch_nt_multi(const RowMultiArgs<T> &m, int npulse, cudaStream_t st) {
-    using C = RowCfg<NT>;
-    const RowArgs<T> &a = m.a;
-    const size_t smem = smem_bytes<T, NT>((a.ops & (OP_RHO | OP_STATS)) != 0);
-    const dim3 grid((a.nr + C::RPC - 1) / C::RPC, npulse);
-    if (grid.x == 0 || npulse <= 0) return cudaSuccess;
+    if (m.a.nr <= 0 || npulse <= 0) return cudaSuccess;
     if (npulse > kRowMulti) return cudaErrorInvalidValue;
-    const bool dk = (a.ops & OP_DIFF) != 0;
-    if constexpr (has_pf<T, NT>())
-        if (a.variant == 3 && a.nl.K == 8 && !dk) return launch_nt_pf<T, NT>(m, npulse, st);
-    void (*k)(const RowMultiArgs<T>) = dk ? multi_kernel_for<T, NT, true>(a) : multi_kernel_for<T, NT, false>(a);
-    return launch_k(k, grid, dim3(C::THREADS), smem, st, m);
+    return with_form<T, NT>(m.a, [&](auto form) { return decltype(form)::launch(m, npulse, st); });
 }
 
 template <typename T, int NT>
 cudaError_t launch_nt(const RowArgs<T> &a, cudaStream_t st) {
-    using C = RowCfg<NT>;
-    const size_t smem = smem_bytes<T, NT>((a.ops & (OP_RHO | OP_STATS)) != 0);
-    const int grid = (a.nr + C::RPC - 1) / C::RPC;
-    if (grid == 0) return cudaSuccess;
-    const bool dk = (a.ops & OP_DIFF) != 0;
-    if constexpr (has_pf<T, NT>()) {
-        if (a.variant == 3 && a.nl.K == 8 && !dk) {
-            RowMultiArgs<T> m;
-            m.a = a;
-            for (int c = 0; c < kRowMulti; ++c) {
-                m.field[c] = a.field;
-                m.rho[c] = a.rho;
-                m.stats[c] = a.stats;
-                m.in[c] = a.in;
-            }
-            return launch_nt_pf<T, NT>(m, 1, st);
-        }
+    RowMultiArgs<T> m;
+    m.a = a;
+    for (int c = 0; c < kRowMulti; ++c) {
+        m.field[c] = a.field;
+        m.rho[c] = a.rho;
+        m.stats[c] = a.stats;
+        m.in[c] = a.in;
+        m.cmp[c] = a.cmp;
+        m.diff[c] = a.diff;
     }
-    // K = 8 (the photon number of 800 nm in air) gets unrolled powers
-    void (*k)(RowArgs<T>) = dk ? kernel_for<T, NT, true>(a) : kernel_for<T, NT, false>(a);
-    return launch_k(k, dim3(grid), dim3(C::THREADS), smem, st, a);
+    return launch_nt_multi<T, NT>(m, 1, st);
 }
 
 }  // namespace rowimpl

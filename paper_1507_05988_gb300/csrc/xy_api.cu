@@ -38,6 +38,7 @@ struct fcn_xy_ctx {
     double *host_red = nullptr;     // pinned [16]
     const void *tw = nullptr;
     const void *tw1 = nullptr;   // twiddles of FFT plan 1 (FP32, Nt >= 256), or null
+    const void *tw2 = nullptr;   // twiddles of FFT plan 2
     // pivot tables of the current dz: x lines (no dispersion), y lines
     uint64_t tab_dz = 0;
     void *tab_x = nullptr, *tab_y = nullptr;
@@ -112,6 +113,7 @@ RowArgs<T> row_args(fcn_xy_ctx *ctx, void *field, int ops, double dz) {
     a.field = (cx<T> *)field;
     a.tw = (const cx<T> *)ctx->tw;
     a.tw1 = (const cx<T> *)ctx->tw1;
+    a.tw2 = (const cx<T> *)ctx->tw2;
     a.rho = (T *)ctx->rho;
     a.stats = ctx->stats;
     a.nr = (int)ctx->rows();
@@ -257,7 +259,13 @@ int ensure_tuned(fcn_xy_ctx *ctx, double dz) {
         std::vector<float> tr(nrv, 1e30f), tl(kXYVariants, 1e30f);
         for (int round = 0; round < 3; ++round) {
             for (int v = 0; v < nrv; ++v) {
-                RowArgs<T> a = row_args<T>(ctx, scratch, OPS_MID, dz);
+                // on the spectrum that a middle launch meets: what the
+                // nonlinear part has to do depends on the intensities
+                RowArgs<T> a = row_args<T>(ctx, scratch, OPS_HEAD, dz);
+                a.variant = 0;
+                a.in = (const cx<T> *)ctx->field;
+                CK(launch_rows<T>(a, ctx->g.nt, ctx->st), "tuning input");
+                a = row_args<T>(ctx, scratch, OPS_MID, dz);
                 a.variant = v;
                 float ms;
                 int rc = time_launches(ctx, [&] { return launch_rows<T>(a, ctx->g.nt, ctx->st); }, &ms);
@@ -449,6 +457,8 @@ int fcn_xy_create(const fcn_grid_xy *grid, const fcn_params *params, int32_t pre
             const cx<double> *tw;
             e = hostx::twiddles<double>(grid->nt, &tw);
             ctx->tw = tw;
+            if (e == cudaSuccess) e = hostx::twiddles<double>(fft_tag(grid->nt, 2), &tw);
+            ctx->tw2 = tw;
             if (e == cudaSuccess) e = prepare_rows<double>(grid->nt);
         } else {
             const cx<float> *tw, *tw1 = nullptr;
@@ -456,6 +466,8 @@ int fcn_xy_create(const fcn_grid_xy *grid, const fcn_params *params, int32_t pre
             if (e == cudaSuccess && grid->nt >= 256) e = hostx::twiddles<float>(fft_tag(grid->nt, 1), &tw1);
             ctx->tw = tw;
             ctx->tw1 = tw1;
+            if (e == cudaSuccess) e = hostx::twiddles<float>(fft_tag(grid->nt, 2), &tw);
+            ctx->tw2 = tw;
             if (e == cudaSuccess) e = prepare_rows<float>(grid->nt);
         }
     }
