@@ -43,97 +43,26 @@ struct alignas(16) CoRow<double> {
     double sl, sh;
 };
 
-__device__ __forceinline__ float tfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double tfma(double a, double b, double c) { return fma(a, b, c); }
-// m y + b for the complex factor m of a sweep: in the chunks' maps.
-template <typename T>
-__device__ __forceinline__ cx<T> cfma(cx<T> m, cx<T> y, cx<T> b) {
-    return mk(tfma(y.x, m.x, tfma(-y.y, m.y, b.x)), tfma(y.x, m.y, tfma(y.y, m.x, b.y)));
-}
-// The same in the sweeps themselves: in FP32 the product first, then one
+// m y + b in a sweep: in FP32 the product first, then one
 // rounding at the size of the sum.  (Folded into two FMAs the sum is rounded
 // twice, and every later row inherits both.)
 template <typename T>
 __device__ __forceinline__ cx<T> sweep(cx<T> m, cx<T> y, cx<T> b) {
     if constexpr (sizeof(T) == 4)
-        return mk(tfma(y.x, m.x, -(y.y * m.y)) + b.x, tfma(y.x, m.y, y.y * m.x) + b.y);
+        return mk(vfma(y.x, m.x, -(y.y * m.y)) + b.x, vfma(y.x, m.y, y.y * m.x) + b.y);
     else
         return cfma(m, y, b);
 }
-template <typename T>
-__device__ __forceinline__ cx<T> cshfl(cx<T> v, int src, int width) {
-    return mk(__shfl_sync(0xffffffffu, v.x, src, width), __shfl_sync(0xffffffffu, v.y, src, width));
-}
-
-// Value entering this thread's chunk, the chunks of a column mapping x -> A x
-// + B, composed in chunk order (REV: in reverse).  Lanes of one column sit C
-// apart; the totals of the nw warps are scanned for all columns in parallel,
-// one lane per (column, warp).  sA, sB, sC: one value per (warp, column).
-template <typename T, bool REV, int C>
-__device__ __forceinline__ cx<T> block_scan(cx<T> A, cx<T> B, int nw, cx<T> *sA, cx<T> *sB, cx<T> *sC) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    constexpr int cpw = 32 / C;
-    const int ciw = lane / C, col = lane % C;
-#pragma unroll
-    for (int d = 1; d < cpw; d <<= 1) {
-        const int src = REV ? lane + d * C : lane - d * C;
-        const cx<T> Ao = cshfl(A, src & 31, 32);
-        const cx<T> Bo = cshfl(B, src & 31, 32);
-        if (REV ? (ciw + d < cpw) : (ciw >= d)) {
-            B = cfma(A, Bo, B);
-            A = cfma(A, Ao, czero<T>());
-        }
-    }
-    cx<T> Ae = cshfl(A, (REV ? lane + C : lane - C) & 31, 32);
-    cx<T> Be = cshfl(B, (REV ? lane + C : lane - C) & 31, 32);
-    if (REV ? (ciw == cpw - 1) : (ciw == 0)) {
-        Ae = mk(T(1), T(0));
-        Be = czero<T>();
-    }
-    if (nw == 1) {
-        __syncwarp();
-        return Be;
-    }
-    if (REV ? (ciw == 0) : (ciw == cpw - 1)) {
-        sA[FCN_IDX(w * C + col, nw * C, 38)] = A;
-        sB[FCN_IDX(w * C + col, nw * C, 39)] = B;
-    }
-    __syncthreads();
-    constexpr int NW = 16;                       // warps of a CTA at most
-    for (int base = w * 32; base < NW * C; base += nw * 32) {
-        const int i = base + lane, c0 = i / NW, kw = i & (NW - 1);
-        const bool on = kw < nw && c0 < C;
-        cx<T> A2 = mk(T(1), T(0)), B2 = czero<T>();
-        if (on) {
-            A2 = sA[FCN_IDX(kw * C + c0, nw * C, 48)];
-            B2 = sB[FCN_IDX(kw * C + c0, nw * C, 49)];
-        }
-#pragma unroll
-        for (int d = 1; d < NW; d <<= 1) {
-            const int src = (REV ? kw + d : kw - d) & (NW - 1);
-            const cx<T> Ao = cshfl(A2, src, NW);
-            const cx<T> Bo = cshfl(B2, src, NW);
-            if (REV ? (kw + d < NW) : (kw >= d)) {
-                B2 = cfma(A2, Bo, B2);
-                A2 = cfma(A2, Ao, czero<T>());
-            }
-        }
-        cx<T> ex = cshfl(B2, (REV ? kw + 1 : kw - 1) & (NW - 1), NW);
-        if (REV ? (kw >= nw - 1) : (kw == 0)) ex = czero<T>();
-        if (on) sC[FCN_IDX(kw * C + c0, nw * C, 50)] = ex;
-    }
-    __syncthreads();
-    return cfma(Ae, sC[FCN_IDX(w * C + col, nw * C, 43)], Be);
-}
-
 // Shared-memory index of row j's coefficients: one padding entry per chunk,
 // so that the chunks of a warp read different banks.
 template <int L>
 __host__ __device__ __forceinline__ int co_idx(int j) { return j + j / L; }
 
 // Right-hand sides over pivots, the rounded pivots for the sweep factors and
-// the forward map's B of one chunk.  EDGE: the chunk touches row -1 or nr-1.
-template <typename T, int L, bool EDGE>
+// the forward map's B of one chunk.  Chunks at the ends of the column run the
+// same code with predicates (in a path of their own they would diverge from
+// the other chunks of their warp, and the CTA wait for them).
+template <typename T, int L>
 __device__ __forceinline__ cx<T> block_load(const ColArgs<T> &a, int q, int qq, int j0, const CdCol<T> &cd,
                                             const PivLim<T> &lim, const CoRow<T> *co, cx<T> (&y)[L], cx<T> (&iv)[L]) {
     const int nr = a.nr, nt = a.nt;
@@ -143,17 +72,18 @@ __device__ __forceinline__ cx<T> block_load(const ColArgs<T> &a, int q, int qq, 
     unsigned o = (unsigned)((j0 - 1) * nt + q);
 #pragma unroll
     for (int k = 0; k < L + 2; ++k, o += nt) {
-        const int j = j0 - 1 + k;
-        x[k] = (EDGE && (j < 0 || j >= nr)) ? czero<T>() : a.field[FCN_IDX(o, (size_t)nr * nt, 66)];
+        x[k] = czero<T>();
+        if ((k > 0 || j0 > 0) && j0 - 1 + k < nr) x[k] = a.field[FCN_IDX(o, (size_t)nr * nt, 66)];
     }
     o = (unsigned)(j0 * a.tp + qq);
 #pragma unroll
-    for (int k = 0; k < L; ++k, o += a.tp)
-        iv[k] = (!EDGE || j0 + k < nr) ? ldg_cx(a.invden + FCN_IDX(o, (size_t)nr * a.tp, 67)) : czero<T>();
+    for (int k = 0; k < L; ++k, o += a.tp) {
+        iv[k] = czero<T>();
+        if (j0 + k < nr) iv[k] = ldg_cx(a.invden + FCN_IDX(o, (size_t)nr * a.tp, 67));
+    }
     cx<T> B = czero<T>();
 #pragma unroll
     for (int k = 0; k < L; ++k) {
-        const int j = j0 + k;
         const CoRow<T> c = co[k];
         // rhs = x_j + i (sl x_{j-1} + sh x_{j+1} - (c0 - delta) x_j); the
         // axis row has its own c0, the last row (A = 0) and the rows past it
@@ -162,15 +92,16 @@ __device__ __forceinline__ cx<T> block_load(const ColArgs<T> &a, int q, int qq, 
         e.sl = c.sl;
         e.sh = c.sh;
         e.d = T(1);
-        e.cd = (EDGE && j == 0) ? cd.ah : cd.ih;
+        e.cd = (k == 0 && j0 == 0) ? cd.ah : cd.ih;
         if constexpr (sizeof(T) == 4) {
             e.sll = c.sll;
             e.shl = c.shl;
-            e.cdl = (EDGE && j == 0) ? cd.al : cd.il;
+            e.cdl = (k == 0 && j0 == 0) ? cd.al : cd.il;
         }
-        const bool dead = EDGE && j >= nr - 1;
-        y[k] = dead ? czero<T>() : piv_apply(ex_rhs(e, x[k], x[k + 1], x[k + 2]), iv[k], lim);
-        iv[k] = dead ? czero<T>() : piv_full(iv[k], lim);
+        const bool dead = j0 + k >= nr - 1;
+        y[k] = piv_apply(ex_rhs(e, x[k], x[k + 1], x[k + 2]), iv[k], lim);
+        iv[k] = piv_full(iv[k], lim);           // sl = sh = 0 in the dead rows: any finite value does
+        if (dead) y[k] = czero<T>();
         B = cfma(cmul_i(iv[k], c.sl), B, y[k]);
     }
     return B;
@@ -186,7 +117,7 @@ __host__ __device__ constexpr size_t block_smem(int threads) {
 
 // Columns [g C, g C + C) of one field.  Threads past block_threads(nr) return
 // (whole warps, before any barrier); chunks past the last row hold zero maps.
-template <typename T, int L, int C>
+template <typename T, int L, int C, int MAXT>
 __device__ __forceinline__ void block_body(const ColArgs<T> &a, int g, unsigned char *smem_raw) {
     const int nr = a.nr, nt = a.nt, tp = a.tp;
     const int nthr = block_threads<L, C>(nr);
@@ -235,10 +166,9 @@ __device__ __forceinline__ void block_body(const ColArgs<T> &a, int g, unsigned 
     const CoRow<T> *cr = co + co_idx<L>(j0);
     cx<T> y[L], iv[L];
     cx<T> B;
-    if (j0 >= 1 && j0 + L < nr) B = block_load<T, L, false>(a, q, qq, j0, cd, lim, cr, y, iv);
-    else B = block_load<T, L, true>(a, q, qq, j0, cd, lim, cr, y, iv);
+    B = block_load<T, L>(a, q, qq, j0, cd, lim, cr, y, iv);
     // exact y from the value entering the chunk
-    cx<T> v = block_scan<T, false, C>(PA, B, nw, sA, sB, sC);
+    cx<T> v = block_scan<T, T, false, C, MAXT / 32>(PA, B, nw, sA, sB, sC);
 #pragma unroll
     for (int k = 0; k < L; ++k) {
         v = sweep(cmul_i(iv[k], cr[k].sl), v, y[k]);
@@ -248,7 +178,7 @@ __device__ __forceinline__ void block_body(const ColArgs<T> &a, int g, unsigned 
     B = czero<T>();
 #pragma unroll
     for (int k = L - 1; k >= 0; --k) B = cfma(cmul_i(iv[k], cr[k].sh), B, y[k]);
-    v = block_scan<T, true, C>(QA, B, nw, sA, sB, sC);
+    v = block_scan<T, T, true, C, MAXT / 32>(QA, B, nw, sA, sB, sC);
     unsigned o = (unsigned)((j0 + L - 1) * nt + q);
     if (a.disp == 0.0) {
 #pragma unroll
@@ -272,7 +202,7 @@ __global__ void __launch_bounds__(MAXT, MB) cn_block_kernel(const __grid_constan
     pdl_enter();
     // groups g and ngroups - 1 - g share their pivot columns: adjacent CTAs
     const int ngroups = a.nt / C, b = blockIdx.x;
-    block_body<T, L, C>(a, (b & 1) ? (ngroups - 1 - (b >> 1)) : (b >> 1), smem_raw);
+    block_body<T, L, C, MAXT>(a, (b & 1) ? (ngroups - 1 - (b >> 1)) : (b >> 1), smem_raw);
 }
 
 // Work list of columns: each CTA takes the item (pulse, column group) of its
@@ -282,7 +212,7 @@ __global__ void __launch_bounds__(MAXT, MB)
 cn_block_list_kernel(const ColArgs<T> *__restrict__ pulses, const int2 *__restrict__ items) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int2 w = items[blockIdx.x];
-    block_body<T, L, C>(pulses[w.x], w.y, smem_raw);
+    block_body<T, L, C, MAXT>(pulses[w.x], w.y, smem_raw);
 }
 
 // Products of alpha_j (first NP rows of prod) and gamma_j (next NP rows) over

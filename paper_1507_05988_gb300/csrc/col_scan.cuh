@@ -5,7 +5,7 @@
 // exact dispersion factor of one frequency column.
 #pragma once
 
-#include "fcn_device.cuh"
+#include "pack.cuh"
 
 namespace fcn {
 namespace colscan {
@@ -144,6 +144,99 @@ __device__ __forceinline__ cx<T> disp_apply(cx<T> x, const DispPhase<T> &p) {
     } else {
         return cmul(x, p.hi);
     }
+}
+
+// m y + b, the factor m of type W (a pair's lines share it: W scalar, V packed).
+template <typename V, typename W>
+__device__ __forceinline__ cx<V> cfma(cx<W> m, cx<V> y, cx<V> b) {
+    V mx, my;
+    if constexpr (sizeof(V) == sizeof(W)) {
+        mx = m.x;
+        my = m.y;
+    } else {
+        mx = Pack<V>::splat(m.x);
+        my = Pack<V>::splat(m.y);
+    }
+    return mk(vfma(y.x, mx, vfma(-y.y, my, b.x)), vfma(y.x, my, vfma(y.y, mx, b.y)));
+}
+template <typename V>
+__device__ __forceinline__ V vshfl(V v, int src, int width) {
+    if constexpr (Pack<V>::L == 2)
+        return pk2{__shfl_sync(0xffffffffu, v.a, src, width), __shfl_sync(0xffffffffu, v.b, src, width)};
+    else
+        return __shfl_sync(0xffffffffu, v, src, width);
+}
+template <typename V>
+__device__ __forceinline__ cx<V> cshfl(cx<V> v, int src, int width) {
+    return mk(vshfl(v.x, src, width), vshfl(v.y, src, width));
+}
+template <typename V>
+__device__ __forceinline__ cx<V> vzero() {
+    const V z = Pack<V>::splat(typename Pack<V>::S(0));
+    return mk(z, z);
+}
+
+// Value entering this thread's chunk, the chunks of a column mapping x -> A x
+// + B, composed in chunk order (REV: in reverse).  Lanes of one column sit C
+// apart; the totals of the nw (<= NW) warps are scanned for all columns in
+// parallel, one lane per (column, warp).  sA, sB, sC: one value per (warp,
+// column).  Every thread of the nw warps calls it.
+template <typename V, typename W, bool REV, int C, int NW>
+__device__ __forceinline__ cx<V> block_scan(cx<W> A, cx<V> B, int nw, cx<W> *sA, cx<V> *sB, cx<V> *sC) {
+    using T = typename Pack<V>::S;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int cpw = 32 / C;
+    const int ciw = lane / C, col = lane % C;
+#pragma unroll
+    for (int d = 1; d < cpw; d <<= 1) {
+        const int src = REV ? lane + d * C : lane - d * C;
+        const cx<W> Ao = cshfl(A, src & 31, 32);
+        const cx<V> Bo = cshfl(B, src & 31, 32);
+        if (REV ? (ciw + d < cpw) : (ciw >= d)) {
+            B = cfma(A, Bo, B);
+            A = cfma(A, Ao, vzero<W>());
+        }
+    }
+    cx<W> Ae = cshfl(A, (REV ? lane + C : lane - C) & 31, 32);
+    cx<V> Be = cshfl(B, (REV ? lane + C : lane - C) & 31, 32);
+    if (REV ? (ciw == cpw - 1) : (ciw == 0)) {
+        Ae = mk(W(T(1)), W(T(0)));
+        Be = vzero<V>();
+    }
+    if (NW == 1 || nw == 1) {
+        __syncwarp();
+        return Be;
+    }
+    if (REV ? (ciw == 0) : (ciw == cpw - 1)) {
+        sA[FCN_IDX(w * C + col, nw * C, 38)] = A;
+        sB[FCN_IDX(w * C + col, nw * C, 39)] = B;
+    }
+    __syncthreads();
+    for (int base = w * 32; base < NW * C; base += nw * 32) {
+        const int i = base + lane, c0 = i / NW, kw = i & (NW - 1);
+        const bool on = kw < nw && c0 < C;
+        cx<W> A2 = mk(W(T(1)), W(T(0)));
+        cx<V> B2 = vzero<V>();
+        if (on) {
+            A2 = sA[FCN_IDX(kw * C + c0, nw * C, 48)];
+            B2 = sB[FCN_IDX(kw * C + c0, nw * C, 49)];
+        }
+#pragma unroll
+        for (int d = 1; d < NW; d <<= 1) {
+            const int src = (REV ? kw + d : kw - d) & (NW - 1);
+            const cx<W> Ao = cshfl(A2, src, NW);
+            const cx<V> Bo = cshfl(B2, src, NW);
+            if (REV ? (kw + d < NW) : (kw >= d)) {
+                B2 = cfma(A2, Bo, B2);
+                A2 = cfma(A2, Ao, vzero<W>());
+            }
+        }
+        cx<V> ex = cshfl(B2, (REV ? kw + 1 : kw - 1) & (NW - 1), NW);
+        if (REV ? (kw >= nw - 1) : (kw == 0)) ex = vzero<V>();
+        if (on) sC[FCN_IDX(kw * C + c0, nw * C, 50)] = ex;
+    }
+    __syncthreads();
+    return cfma(Ae, sC[FCN_IDX(w * C + col, nw * C, 43)], Be);
 }
 
 // chunk_scan for NP right-hand sides sharing one A: returns the value entering

@@ -571,7 +571,7 @@ int cn_batch_columns(int max_nr);
 template <typename T>
 struct XYLine {
     cx<T> *field;
-    const cx<T> *invden;     // [n][nt/2+1]: 1/pivot_j per |q|
+    const cx<T> *invden;     // table of launch_xy_table (xy_table_entries)
     int n, nt, width, batch;
     long long pitch, bstride;
     long long total;         // elements of the field buffer
@@ -579,12 +579,13 @@ struct XYLine {
     T dk;                    // delta_q = dk q^2 (0 in a line without dispersion)
     double s64, dk64;        // s and dk in FP64 (two-float explicit side in FP32)
     double disp;             // exact dispersion factor exp(2 i disp q^2), 0: none
-    // chunk length L (long: 16 nodes in FP32, 8 in FP64; short: half),
-    // lines per thread NP and CTA size: 0 long/1/512, 1 short/1/512,
-    // 2 short/2/512, 3 short/2/256, 4 long/1/256, 5 short/1/256,
-    // 6 short/2/256 compiled for three CTAs per SM, 7 short/1/256 for four
+    // chunk length, columns per CTA and CTA size (launch_xy_line)
     int variant;
 };
+// Nodes per product of the sweep factors in the table, and its entries (16
+// bytes each in both precisions).
+constexpr int kXYProd = 4;
+size_t xy_table_entries(int n, int nt);
 template <typename T>
 cudaError_t launch_xy_table(int n, int nt, double s, double dk, cx<T> *table, cudaStream_t st);
 template <typename T>

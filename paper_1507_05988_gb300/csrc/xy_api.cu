@@ -201,11 +201,9 @@ int ensure_tables(fcn_xy_ctx *ctx, double dz) {
         for (auto &kv : ctx->graphs) cudaGraphExecDestroy(kv.second);
         ctx->graphs.clear();
     }
-    const int nq = ctx->g.nt / 2 + 1;
     if (!ctx->tab_x) {
-        const size_t per = sizeof(cx<T>) * (sizeof(T) == 4 ? 2 : 1);   // FP32: two-float entries
-        CK(cudaMalloc(&ctx->tab_x, per * (size_t)ctx->g.nx * nq), "x pivot table");
-        CK(cudaMalloc(&ctx->tab_y, per * (size_t)ctx->g.ny * nq), "y pivot table");
+        CK(cudaMalloc(&ctx->tab_x, 16 * xy_table_entries(ctx->g.nx, ctx->g.nt)), "x pivot table");
+        CK(cudaMalloc(&ctx->tab_y, 16 * xy_table_entries(ctx->g.ny, ctx->g.nt)), "y pivot table");
     }
     double s, dk, disp;
     line_coefs(ctx, dz, dx_of(ctx), &s, &dk, &disp);
