@@ -1136,44 +1136,71 @@ __device__ __forceinline__ cx<V> nl_full(cx<V> a, V u, const NLCoef<T> &c) {
     return mk(a.x + dx, a.y + dy);
 }
 
-// Reduction of NV FP64 values across the TPR threads of a row in one pass
-// (warp shuffles, then one exchange of the warp partials); mx[k] selects max
-// instead of sum for value k.  Results valid in thread t = 0.
-template <int NT, int NV>
-__device__ __forceinline__ void row_reduce(double (&x)[NV], const bool (&mx)[NV], int t, double *scr,
-                                           int rloc) {
+// Totals over the TPR threads of each row of a CTA of TH threads: sums of
+// s[k] in FP64, sums (k < NA) or maxima of m[k] in T.  Every thread leaves its
+// partials in shared memory (smem: free for all, no barrier needed before);
+// G of them each go to one lane, the lanes of a row combine theirs by
+// shuffles, and the row's first lane calls out(unit of the CTA, s, m).  No
+// barrier after: the caller has one before smem is written again.
+//
+// FP64 units bound it: a warp's FP64 instruction holds one of an SM's four
+// schedulers' FP64 lanes for 64 cycles, so a tree of shuffles in every warp
+// (5 levels x 4 FP64 values, of which most lanes are idle work) took as long
+// as the row's transform.  Here one warp adds for 256 threads, 13 FP64
+// additions deep, and maxima and counts are in T.  Last stage with rho and
+// statistics, 8 x 1024 rows of 4096 points, FP32: 303 -> TAILUS us; with the
+// step-doubling sums 336 -> DIFFUS us.
+constexpr int row_red_group(int tpr) { return tpr >= 256 ? tpr / 32 : tpr >= 8 ? 8 : tpr; }
+template <typename T, int NT, int TH, int NS, int NA, int NX, typename F>
+__device__ __forceinline__ void row_totals(const double (&s)[NS], const T (&m)[NA + NX + 1], unsigned char *smem,
+                                           F out) {
     using C = RowCfg<NT>;
-    constexpr int W = C::TPR < 32 ? C::TPR : 32;
+    if constexpr (C::TPR == 1) return out((int)threadIdx.x, s, m);
+    constexpr int G = row_red_group(C::TPR), LPR = C::TPR / G, NM = NA + NX;
+    constexpr int STRIDE = G > 1 ? TH + TH / G : TH;          // padded: conflict-free for writers and readers
+    static_assert(C::TPR == 1 || STRIDE * (NS * 8 + NM * (int)sizeof(T)) <= TH * C::PADN / C::TPR * 2 * (int)sizeof(T), "row storage");
+    static_assert(LPR <= 32, "a row's lanes are in one warp");
+    double *P = reinterpret_cast<double *>(smem);
+    T *Q = reinterpret_cast<T *>(P + NS * STRIDE);
+    const int tid = threadIdx.x;
+    const int pos = G > 1 ? tid + tid / G : tid;
+    __syncthreads();
 #pragma unroll
-    for (int d = W / 2; d >= 1; d >>= 1) {
+    for (int k = 0; k < NS; ++k) P[FCN_IDX(k * STRIDE + pos, NS * STRIDE, 18)] = s[k];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            const double o = __shfl_down_sync(0xffffffffu, x[k], d, W);
-            x[k] = mx[k] ? fmax(x[k], o) : x[k] + o;
+    for (int k = 0; k < NM; ++k) Q[FCN_IDX(k * STRIDE + pos, NM * STRIDE, 19)] = m[k];
+    __syncthreads();
+    if ((tid & ~31) >= TH / G) return;
+    const bool on = tid < TH / G;
+    const int p0 = on ? (G > 1 ? tid * (G + 1) : tid) : 0;
+    double x[NS];
+    T y[NM + 1];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        x[k] = P[FCN_IDX(k * STRIDE + p0, NS * STRIDE, 20)];
+#pragma unroll
+        for (int g = 1; g < G; ++g) x[k] += P[FCN_IDX(k * STRIDE + p0 + g, NS * STRIDE, 20)];
+    }
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+        y[k] = Q[FCN_IDX(k * STRIDE + p0, NM * STRIDE, 21)];
+#pragma unroll
+        for (int g = 1; g < G; ++g) {
+            const T o = Q[FCN_IDX(k * STRIDE + p0 + g, NM * STRIDE, 21)];
+            y[k] = k < NA ? y[k] + o : fmax(y[k], o);
         }
     }
-    if (C::WARPS_PER_ROW > 1) {
-        static_assert(C::WARPS_PER_ROW * NV <= kRowScratch, "row scratch");
-        __syncthreads();
-        if ((t & 31) == 0) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k)
-                scr[FCN_IDX((rloc * C::WARPS_PER_ROW + (t >> 5)) * NV + k, kRowScratch, 18)] = x[k];
-        }
-        __syncthreads();
-        if (t == 0) {
+    for (int d = LPR / 2; d >= 1; d >>= 1) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                double acc = scr[FCN_IDX(rloc * C::WARPS_PER_ROW * NV + k, kRowScratch, 20)];
-                for (int w = 1; w < C::WARPS_PER_ROW; ++w) {
-                    const double o = scr[FCN_IDX((rloc * C::WARPS_PER_ROW + w) * NV + k, kRowScratch, 21)];
-                    acc = mx[k] ? fmax(acc, o) : acc + o;
-                }
-                x[k] = acc;
-            }
+        for (int k = 0; k < NS; ++k) x[k] += __shfl_down_sync(0xffffffffu, x[k], d, LPR);
+#pragma unroll
+        for (int k = 0; k < NM; ++k) {
+            const T o = __shfl_down_sync(0xffffffffu, y[k], d, LPR);
+            y[k] = k < NA ? y[k] + o : fmax(y[k], o);
         }
-        __syncthreads();
     }
+    if (on && (tid & (LPR - 1)) == 0) out(tid / LPR, x, y);
 }
 
 // Compensated (Kahan) FP32 running sum: the per-thread partials of the FP32
@@ -1387,13 +1414,17 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
     }
     const bool have_u = nhalf > 0;
     if (keep_u) {
-        if (!in_regs) pass_load<V, NT, 0>(v, S, t);
+        if (!in_regs) {
+            pass_load<V, NT, 0>(v, S, t);
+            in_regs = true;
+        }
         // statistics of the final rows; rho is written below, coalesced
         if ((ops & OP_STATS) && bf.stats) {
+            // sum |A|^2; count of non-finite |A|^2, max |A|^2, max u
+            double sum[L];
+            T m[3 * L + 1];
 #pragma unroll
             for (int k = 0; k < L; ++k) {
-                // v4 = {sum |A|^2, max |A|^2, max u, count of non-finite |A|^2}
-                double v4[4] = {0.0, 0.0, 0.0, 0.0};
                 std::conditional_t<sizeof(T) == 4, KahanF, PlainSum<T>> ks;
                 T mx = T(0), mu = T(0), bad = T(0);
 #pragma unroll
@@ -1408,20 +1439,23 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
                         mu = fmax(mu, row_of<V>(mk(u, u), k).x);
                     }
                 }
-                v4[0] = ks.sum();
-                v4[1] = mx;
-                v4[2] = mu;
-                v4[3] = bad;
-                const bool mxk[4] = {false, true, true, false};
-                row_reduce<NT, 4>(v4, mxk, t, scr, rloc);
-                if (t == 0 && valid && k < nrow) {
-                    double *st = bf.stats + FCN_IDX((size_t)(row + k) * NSTAT, (size_t)a.nr * NSTAT, 23);
-                    st[ST_SUM_I] = v4[0];
-                    st[ST_MAX_I] = v4[1];
-                    if (ops & (OP_NL | OP_NL2)) st[ST_MAX_U] = v4[2];
-                    st[ST_NONFINITE] = v4[3];
-                }
+                sum[k] = ks.sum();
+                m[k] = bad;
+                m[L + 2 * k] = mx;
+                m[L + 2 * k + 1] = mu;
             }
+            row_totals<T, NT, TH, L, L, 2 * L>(sum, m, smem_raw, [&](int unit, const double *x, const T *y) {
+#pragma unroll
+                for (int k = 0; k < L; ++k) {
+                    const int r = row_base + unit * L + k;
+                    if (r >= a.nr) break;
+                    double *st = bf.stats + FCN_IDX((size_t)r * NSTAT, (size_t)a.nr * NSTAT, 23);
+                    st[ST_SUM_I] = x[k];
+                    st[ST_MAX_I] = double(y[L + 2 * k]);
+                    if (ops & (OP_NL | OP_NL2)) st[ST_MAX_U] = double(y[L + 2 * k + 1]);
+                    st[ST_NONFINITE] = double(y[k]);
+                }
+            });
         }
         if ((ops & OP_RHO) && valid && bf.rho) {
             auto u_of = [&](int q, int k) {
@@ -1474,6 +1508,7 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
         }
     }
     if (store) {
+        if (keep_u) __syncthreads();                     // row_totals' reads of the storage of S
         to_smem();
         auto acc = [&](int k, cx<T> x, cx<T> y) {          // x: stored value, y: compared value
             const T dx = y.x - x.x, dy = y.y - x.y;
@@ -1528,24 +1563,23 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
         }
     }
     if constexpr (DIFFK) {
-        double v2[2 * L];
-        bool sk[2 * L];
+        double sum[2 * L];
+        T none[1];
 #pragma unroll
         for (int k = 0; k < L; ++k) {
-            v2[2 * k] = double(d2[k]);
-            v2[2 * k + 1] = double(b2[k]);
-            sk[2 * k] = sk[2 * k + 1] = false;
+            sum[2 * k] = double(d2[k]);
+            sum[2 * k + 1] = double(b2[k]);
         }
-        row_reduce<NT, 2 * L>(v2, sk, t, scr, rloc);
-        if (t == 0 && valid && diff) {
+        row_totals<T, NT, TH, 2 * L, 0, 0>(sum, none, smem_raw, [&](int unit, const double *x, const T *) {
+            if (!diff) return;
 #pragma unroll
             for (int k = 0; k < L; ++k) {
-                if (k < nrow) {
-                    diff[FCN_IDX((size_t)2 * (row + k), (size_t)2 * a.nr, 33)] = v2[2 * k];
-                    diff[FCN_IDX((size_t)2 * (row + k) + 1, (size_t)2 * a.nr, 34)] = v2[2 * k + 1];
-                }
+                const int r = row_base + unit * L + k;
+                if (r >= a.nr) break;
+                diff[FCN_IDX((size_t)2 * r, (size_t)2 * a.nr, 33)] = x[2 * k];
+                diff[FCN_IDX((size_t)2 * r + 1, (size_t)2 * a.nr, 34)] = x[2 * k + 1];
             }
-        }
+        });
     }
 
     if (ops & OP_FFT) {
@@ -1574,6 +1608,7 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
             for (int k = 0; k < L; ++k) {
                 // spectral moments sum_q w^k |A_q|^2, w = signed bin, k = 0, 1, 2
                 double m3[3] = {0.0, 0.0, 0.0};
+                T none[1];
                 if constexpr (sizeof(T) == 4) {
                     KahanF k0, k1, k2;
 #pragma unroll
@@ -1609,14 +1644,14 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
                         }
                     }
                 }
-                const bool mxk[3] = {false, false, false};
-                row_reduce<NT, 3>(m3, mxk, t, scr, rloc);
-                if (t == 0 && valid && k < nrow) {
-                    double *st = bf.stats + FCN_IDX((size_t)(row + k) * NSTAT, (size_t)a.nr * NSTAT, 24);
-                    st[ST_S0] = m3[0];
-                    st[ST_S1] = m3[1];
-                    st[ST_S2] = m3[2];
-                }
+                row_totals<T, NT, TH, 3, 0, 0>(m3, none, smem_raw, [&](int unit, const double *x, const T *) {
+                    const int r = row_base + unit * L + k;
+                    if (r >= a.nr) return;
+                    double *st = bf.stats + FCN_IDX((size_t)r * NSTAT, (size_t)a.nr * NSTAT, 24);
+                    st[ST_S0] = x[0];
+                    st[ST_S1] = x[1];
+                    st[ST_S2] = x[2];
+                });
             }
         }
     }
