@@ -203,15 +203,17 @@ __global__ void cn_table_kernel_f32(TableArgs a, cx<float> *table) {
 //   1. warp c composes its chunk's matrices, G_c = F_{j1-1} ... F_{j0}
 //      (double-float complex entries, rescaled by powers of two now and
 //      then: z is a ratio, so the common scale is free);
-//   2. warp 0 walks the chunks from (num, den) = (0, 1) (1/piv_{-1} = 0),
-//      giving each chunk the z that enters it;
-//   3. warp c runs the recurrence of cn_table_kernel_f32 over its rows from
-//      that z and stores the table.
+//   2. two warps, four lanes per bin, walk the chunks from (num, den) = (0, 1)
+//      (1/piv_{-1} = 0), giving each chunk the pair that enters it: the only
+//      serial part, one product and two sums deep per chunk;
+//   3. warp c forms z from its pair, runs the recurrence of
+//      cn_table_kernel_f32 over its rows from it and stores the table.
 // The entering z comes from the matrix products instead of the recurrence
 // itself, so the two kernels agree to double-float precision (~1e-14), not
 // bit for bit.  A CTA has 16 bins x 32 chunks: a table is ~230 double-float
 // instructions per entry, and the 129 CTAs of Nt = 4096 spread them over
-// nearly all SMs (32 bins x 16 chunks: 65 SMs, 72 us for Nr = 1024).
+// nearly all SMs (Nr = 1024: 42 us; 49 us with step 2 on one lane per bin, 8
+// bins x 64 chunks 52 us, 32 bins x 16 chunks on 65 SMs 72 us).
 // The kernel also leaves the row coefficients (a.coef) and the products of
 // the sweep factors over kProdRows rows (a.prod): the rows and pivots are at
 // hand here, and an adaptive run builds two tables per attempt.
@@ -237,6 +239,10 @@ __device__ __forceinline__ int c2_exp(c2 a) {
     frexpf(fmaxf(fabsf(a.re.h), fabsf(a.im.h)), &e);
     return e;
 }
+__device__ __forceinline__ c2 c2_xor(c2 a, int m) {                  // the value of lane ^ m
+    auto x = [&](float f) { return __shfl_xor_sync(0xffffffffu, f, m); };
+    return {{x(a.re.h), x(a.re.l)}, {x(a.im.h), x(a.im.l)}};
+}
 // rescales the entries by a common power of two so that the largest is O(1)
 __device__ __forceinline__ void c2_norm(c2 *v, int n) {
     int e = -1000;
@@ -252,7 +258,6 @@ __global__ void __launch_bounds__(kTabBins * kTabChunks + 32) cn_table_kernel_f3
     f2 *kap = reinterpret_cast<f2 *>(sh_tab);                         // [nr]
     float2 *sw = reinterpret_cast<float2 *>(kap + a.nr);              // [nr]: (sl, sh) as the sweeps use them
     c2 *G = reinterpret_cast<c2 *>(sw + a.nr);                       // [kTabChunks][kTabBins][4]
-    c2 *Z = G + kTabChunks * kTabBins * 4;                           // [kTabChunks][kTabBins]
     __shared__ f2 byc[2][kTabBins], limc[2][kTabBins];               // per bin: by0, by1; the pivots' limit
     const double s2 = a.s * a.s;
     for (int j = threadIdx.x; j < a.nr; j += blockDim.x) {
@@ -260,9 +265,11 @@ __global__ void __launch_bounds__(kTabBins * kTabChunks + 32) cn_table_kernel_f3
         if (j == 1) k = s2 * a.lo[FCN_IDX(1, a.nr, 31)] * 4.0;
         else if (j >= 2 && j < a.nr - 1) k = s2 * a.lo[FCN_IDX(j, a.nr, 31)] * a.hi[FCN_IDX(j - 1, a.nr, 32)];
         kap[j] = to_f2(k);
-        const CnCoef<float> f = cn_coef_row<float>(a, j);
-        sw[j] = make_float2(f.sl, f.sh);
-        if (a.coef && blockIdx.x == 0) a.coef[FCN_IDX(j, a.nr, 76)] = f;
+        // the rounded sl, sh of cn_coef_row
+        const bool on_j = j < a.nr - 1;
+        sw[j] = make_float2(on_j && j > 0 ? float(a.s * a.lo[FCN_IDX(j, a.nr, 31)]) : 0.f,
+                            !on_j ? 0.f : j == 0 ? float(4.0 * a.s) : float(a.s * a.hi[FCN_IDX(j, a.nr, 32)]));
+        if (a.coef && blockIdx.x == 0) a.coef[FCN_IDX(j, a.nr, 76)] = cn_coef_row<float>(a, j);
     }
     const int lane = threadIdx.x % kTabBins, c = threadIdx.x / kTabBins;
     const int nq = a.nt / 2 + 1;
@@ -314,18 +321,26 @@ __global__ void __launch_bounds__(kTabBins * kTabChunks + 32) cn_table_kernel_f3
         for (int k = 0; k < 4; ++k) G[(c * kTabBins + lane) * 4 + k] = g[k];
     }
     __syncthreads();
-    if (c == 0) {
-        // 2. the z entering every chunk
-        c2 v[2] = {{zero, zero}, {one, zero}};                                // (num, den)
+    if (threadIdx.x < 4 * kTabBins) {
+        // 2. (num, den) entering every chunk, over the entries g00, g01 of its
+        // matrix.  Four lanes per bin: lane r forms the product of entry r,
+        // lanes r and r ^ 1 add theirs.
+        const int b = threadIdx.x >> 2, r = threadIdx.x & 3;
+        c2 v = {r & 1 ? one : zero, zero};                        // num (r even), den (r odd)
+        c2 g = G[b * 4 + r];
         for (int k = 0; k < kTabChunks; ++k) {
-            const c2 n = v[0], d = v[1];
-            const f2 rn = df_recip(df_add(df_mul(d.re, d.re), df_mul(d.im, d.im)));
-            const c2 z = c2_mul(n, c2{d.re, df_neg(d.im)});
-            Z[k * kTabBins + lane] = c2{df_mul(z.re, rn), df_mul(z.im, rn)};
-            const c2 *gk = G + (k * kTabBins + lane) * 4;
-            v[0] = c2_add(c2_mul(gk[0], n), c2_mul(gk[1], d));
-            v[1] = c2_add(c2_mul(gk[2], n), c2_mul(gk[3], d));
-            c2_norm(v, 2);
+            const c2 gk = g;
+            if (k + 1 < kTabChunks) g = G[((k + 1) * kTabBins + b) * 4 + r];
+            __syncwarp();                                         // every lane has read its entry
+            if (r < 2) G[(k * kTabBins + b) * 4 + r] = v;
+            const c2 m = c2_mul(gk, v);
+            c2 w = c2_add(m, c2_xor(m, 1));                       // num' (r < 2), den'
+            // the common power of two of c2_norm
+            int e = w.re.h != 0.f || w.im.h != 0.f ? c2_exp(w) : -1000;
+            e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+            if (e != -1000) w = c2_scale(w, ldexpf(1.f, -e));
+            const c2 o = c2_xor(w, 2);
+            v = (r & 1) == (r >> 1) ? w : o;
         }
     }
     __syncthreads();
@@ -336,8 +351,11 @@ __global__ void __launch_bounds__(kTabBins * kTabChunks + 32) cn_table_kernel_f3
         lx = limc[0][lane];
         ly = limc[1][lane];
     }
-    const c2 z = Z[c * kTabBins + lane];
-    f2 ix = z.re, iy = z.im;
+    // z = num / den entering the chunk
+    const c2 num = G[(c * kTabBins + lane) * 4], den = G[(c * kTabBins + lane) * 4 + 1];
+    const f2 rd = df_recip(df_add(df_mul(den.re, den.re), df_mul(den.im, den.im)));
+    const c2 z = c2_mul(num, c2{den.re, df_neg(den.im)});
+    f2 ix = df_mul(z.re, rd), iy = df_mul(z.im, rd);
     const int NP = (a.nr + kProdRows<float> - 1) / kProdRows<float>;
     cx<float> A = mk(1.f, 0.f), Q = A;
     for (int j = j0; j < j1; ++j) {
@@ -772,7 +790,7 @@ cudaError_t launch_cn_table(const TableArgs &a, cx<T> *table, cudaStream_t st) {
         if (cn_table_fills_all<T>(a.nr)) {
             // rows in chunks (cn_table_kernel_f32_chunked): the serial
             // recurrence down a tall column is the cost of a table
-            constexpr size_t fixed = sizeof(c2) * kTabChunks * kTabBins * 5;
+            constexpr size_t fixed = sizeof(c2) * kTabChunks * kTabBins * 4;
             static std::once_flag once;
             static cudaError_t attr = cudaSuccess;
             std::call_once(once, [] {
