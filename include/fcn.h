@@ -219,17 +219,19 @@ int fcn_get_state(fcn_ctx *ctx, int32_t pulse, double state[4]);
 int fcn_set_state(fcn_ctx *ctx, int32_t pulse, const double state[4]);
 
 /* ======================= kernel variants (autotuner) ======================= */
-/* The row stage has 6 variants (FP32, K = 8): 0-2 one CTA per row (group)
- * with the compiler's register allocation, or 3 or 4 CTAs per SM; 3 a
- * persistent kernel that prefetches each CTA's next rows into shared memory
- * by bulk copies (Nt >= 512); 4, 5 the occupancy of 1, 2 with the other FFT
- * decomposition: radix-8 passes before the final radix-16 one (Nt = 4096:
- * 4 8 8 16) instead of radix-16 passes after one radix 2/4/8 pass (16 16 16)
- * (Nt >= 256; smaller rows run variant 0).  The column stage has 9:
+/* The row stage has 6 variants (FP32, K = 8, Nt >= 256; other launches run
+ * variant 0): 0 one row per group of Nt/16 threads (few rows of few points:
+ * Nt/4 threads), 1 two adjacent rows per group in packed arithmetic, 2 as 0
+ * with 64 registers per thread, 3 packed pairs in smaller CTAs or with more
+ * registers, or single rows with a register cap between those of 0 and 2,
+ * by Nt; 4, 5 the other FFT decomposition: radix-8 passes before the final
+ * radix-16 one (Nt = 4096: 4 8 8 16) instead of radix-16 passes after one
+ * radix 2/4/8 pass (16 16 16), at 3 and 4 CTAs of 256 threads per SM.  The
+ * column stage has 9:
  *   0-3  chunked affine-map scans of the two Thomas sweeps, chunks in
  *        registers (chunk length x CTA size);
- *   4-7  the same with chunks staged in shared memory (cp.async) or fed to
- *        registers, row coefficients from a per-dz table;
+ *   4-7  the same with the chunk products and row coefficients from the
+ *        per-dz table, in four shapes (rows per thread x columns per CTA);
  *   8    one sequential Thomas sweep per column, 32 columns per warp, rows
  *        streamed through a shared-memory ring by TMA (Nt a multiple of 64;
  *        other grids fall back to variant 7).
@@ -243,8 +245,8 @@ int fcn_set_state(fcn_ctx *ctx, int32_t pulse, const double state[4]);
 int fcn_set_variants(fcn_ctx *ctx, int32_t row_variant, int32_t col_variant);
 
 /* Batched work lists for multi-pulse FP32 contexts (every pulse K = 8,
- * Nt >= 512): mode 1 runs each stage of all pulses as one persistent launch
- * over (pulse, rows) and (pulse, column group) items; 0 launches each pulse
+ * Nt >= 512): mode 1 runs each stage of all pulses as one launch over a list
+ * of (pulse, rows) and (pulse, column group) items; 0 launches each pulse
  * separately (tuned per-Nt kernels, all inside one CUDA graph); -1 (the
  * default) uses the work lists when the grids differ and most points lie in
  * pulses too small to fill the GPU with a launch of their own.  Drops the
@@ -520,10 +522,9 @@ int  fcn_xy_step_nograph(fcn_xy_ctx *ctx, double dz, int64_t n);
 /* FP64 diagnostics of the current field (synchronises the stream).
  * Returns FCN_ERR_NONFINITE if the field holds NaN or Inf. */
 int  fcn_xy_get_diag(fcn_xy_ctx *ctx, fcn_diag *out);
-/* Forces the row-stage variant (0..5, as fcn_set_variants; 3 runs as 0
- * here) and the line variant (0..7: the chunk
- * of nodes a thread owns, 16 or 8 in FP32 and 8 or 4 in FP64, one or two
- * lines per thread, CTAs of up to 512 or 256 threads); -1 returns to
+/* Forces the row-stage variant (0..5, as fcn_set_variants) and the line
+ * variant (0..7: the chunk of nodes a thread owns, 16 or 8 in FP32 and 8 or 4
+ * in FP64, one or, in FP32, two lines per thread, CTA shapes); -1 returns to
  * timing.  Every variant computes the same step (up to rounding order). */
 int  fcn_xy_set_variants(fcn_xy_ctx *ctx, int32_t row_variant, int32_t line_variant);
 int  fcn_xy_get_variants(const fcn_xy_ctx *ctx, int32_t out[2]);

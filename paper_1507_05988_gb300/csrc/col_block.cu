@@ -14,13 +14,14 @@
 // Shared memory holds the row coefficients (one broadcast load per row) and
 // the warps' scan totals only.
 //
-// What bounds it: one 1024 x 4096 FP32 pulse takes 33 us with the field in L2
-// (45 us when x, alpha and gamma went through shared memory and every launch
-// formed the chunk products).  Measured with parts left out: arithmetic alone
-// 20 us, the scans 4, the loads 6, the stores 6 -- two CTAs of 8 warps per SM
-// overlap them only in part.  Column segments of 16, 32 or 64 bytes per row
-// make no difference; two adjacent columns per thread in packed arithmetic is
-// slower (39 us: the shuffles and shared-memory values double).
+// What bounds it: one 1024 x 4096 FP32 pulse takes 29-31 us with the field in
+// L2 (45 us when x, alpha and gamma went through shared memory and every
+// launch formed the chunk products).  Issue is 36 % of the cycles; half of a
+// warp's time goes to global loads, which two CTAs of 8 warps per SM (128
+// registers a thread) overlap in part.  At 33 us, column segments of 16, 32 or
+// 64 bytes per row made no difference, two adjacent columns per thread in
+// packed arithmetic took 39 us (the shuffles and shared-memory values double)
+// and issuing the loads before the coefficients' 34.
 #include <type_traits>
 
 #include "col_scan.cuh"
@@ -249,14 +250,15 @@ cudaError_t launch_form(const ColArgs<T> &a, cudaStream_t st) {
 
 // FP32 forms (chunk rows L, columns C), FP64 in brackets:
 //   0: L 16, C 4 in CTAs of up to 256 threads, 128 registers [8, 2]; taller
-//      grids as 2 (1350 x 1024: 16.5 us, 28.5 us before);
-//   1: L 8, C 4, 512 threads at 64 registers [8, 4 at 128] (1024 x 4096: 34.9
-//      against 32.9 us for 0, but 128 x 256: 6.3 against 8.2 us);
+//      grids as 2 (1024 x 4096: 29-32 us, 45 before; 1350 x 1024: 14.5-17 us,
+//      28.5 before);
+//   1: L 8, C 4, 512 threads at 64 registers [8, 4 at 128] (1024 x 4096: 35 us,
+//      but 128 x 256: 6.3 against 8.2 us);
 //   2: L 16, C 8, up to 512 threads at 128 registers, C 4 when taller
-//      [8, 4, then 8, 2] (2048 x 8192: 152 us, 219 us in one sequential sweep
-//      per column);
+//      [8, 4, then 8, 2] (1024 x 4096: 31 us; 2048 x 8192: 140 us, 219 us in
+//      one sequential sweep per column);
 //   3: small grids: L 8, C 2 [4, 1], CTAs of up to 256 threads (FP64 128 x
-//      256: 14.5 us, 28.8 us before).
+//      256: 12.4-15 us against 20 us for 0, 28.8 us before).
 template <typename T>
 cudaError_t launch_cn_block(const ColArgs<T> &a, int form, cudaStream_t st) {
     constexpr bool F = sizeof(T) == 4;

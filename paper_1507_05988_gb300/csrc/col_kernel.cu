@@ -519,7 +519,7 @@ cn_kernel(ColArgs<T> a, int C) {
     cn_body<T, L>(a, C, g, smem_raw);
 }
 
-constexpr size_t kCnStagedSmemMax = 227 * 1024;
+constexpr size_t kCnSmemMax = 227 * 1024;
 
 template <typename T>
 __global__ void cn_coef_kernel(TableArgs a, CnCoef<T> *coef) {
@@ -694,7 +694,7 @@ cudaError_t launch_cn_pair_l(const ColArgs<T> &a, cx<T> *field2, cudaStream_t st
     const int threads = ((C * P + 31) / 32) * 32;
     if (threads > TMAX) return cudaErrorInvalidConfiguration;
     const size_t smem = sizeof(cx<T>) * (5 * (size_t)(threads / 32) * C + 2 * (size_t)L * threads);
-    if (smem > kCnStagedSmemMax) return cudaErrorInvalidConfiguration;
+    if (smem > kCnSmemMax) return cudaErrorInvalidConfiguration;
     return launch_k(cn_pair_kernel<T, L, NTC>, dim3(a.nt / C), dim3(threads), smem, st, a, field2, C);
 }
 
@@ -703,7 +703,7 @@ cudaError_t launch_cn_pair_l(const ColArgs<T> &a, cx<T> *field2, cudaStream_t st
 // stage's loads lean on L1.
 template <typename Kern>
 cudaError_t set_col_attrs(Kern k) {
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCnStagedSmemMax);
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCnSmemMax);
 }
 
 template <typename T, int L, int NTC>
@@ -713,8 +713,9 @@ cudaError_t set_pair_attr() {
 
 }  // namespace
 
-// Variants: bit 0 selects the shorter chunk (more threads, fewer registers
-// per thread), bit 1 a target CTA size of 512 instead of 256 threads.  A
+// Variants below kColBlockFirst: bit 0 selects the shorter chunk (more
+// threads, fewer registers per thread), bit 1 a target CTA size of 512
+// instead of 256 threads.  A
 // variant that does not fit (more than 512 threads) falls back to variant 0.
 template <typename T>
 cudaError_t launch_cn(const ColArgs<T> &a_in, cudaStream_t st) {

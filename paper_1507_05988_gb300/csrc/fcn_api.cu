@@ -97,9 +97,6 @@ NLCoef<T> nl_coef(const fcn_grid &g, const fcn_params &p, double h) {
     n.inv_nt = T(1.0 / double(g.nt));
     n.rho_nt = T(p.rho_nt);
     n.K = p.K;
-    n.nkerr = 1;
-    for (int j = 0; j < 4; ++j)
-        if (p.n2j[j] != 0.0) n.nkerr = j + 1;
     n.flags = p.flags;
     isj = kIs;
     for (int j = 0; j < 4; ++j) {
@@ -414,7 +411,7 @@ uint64_t dz_key(double dz) {
 // per pulse.  Least-recently used tables beyond 2 per pulse + 8 are freed,
 // together with the graphs and batch arguments captured with them.
 // A context table allocation holds the pivots ([nr][nt/2+1] complex) and,
-// from this byte offset on, the nr CnCoef rows of the staged column kernels.
+// from this byte offset on, the nr CnCoef rows.
 template <typename T>
 size_t coef_offset(int nr, int nt) {
     const size_t b = sizeof(cx<T>) * (size_t)nr * (size_t)table_pitch(nt);
@@ -554,7 +551,6 @@ RowArgs<T> row_args(Pulse &pu, void *field, int ops, double dz) {
     a.ops = ops;
     a.variant = pu.row_var;
     a.nl = nl_coef<T>(pu.g, pu.p, 0.5 * dz);
-    a.err = pu.err;
     return a;
 }
 
@@ -741,7 +737,7 @@ bool same_row_launch(const RowArgs<T> &a, const RowArgs<T> &b) {
                 x.h == y.h && x.plasma == y.plasma && x.loss == y.loss && x.sdt == y.sdt &&
                 x.inv_is == y.inv_is && x.inv_nt == y.inv_nt && x.rho_nt == y.rho_nt &&
                 x.hplasma == y.hplasma && x.hloss == y.hloss && x.sat == y.sat && x.is_root == y.is_root &&
-                x.K == y.K && x.nkerr == y.nkerr && x.flags == y.flags;
+                x.K == y.K && x.flags == y.flags;
     for (int j = 0; j < 4; ++j) same = same && x.kerr[j] == y.kerr[j] && x.hk[j] == y.hk[j];
     return same;
 }
@@ -1079,11 +1075,12 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
         } guard{scratch};
         CK(cudaMemcpyAsync(scratch, pu.field, bytes, cudaMemcpyDeviceToDevice, ctx->st), "tuning copy");
         // three interleaved rounds over the variants, each variant's best
-        // round counts (a burst of noise on the GPU then decides nothing)
+        // round counts (a burst of noise on the GPU then decides nothing);
+        // FP64 and other K have one row form
         const int nrv = (sizeof(T) == 4 && pu.p.K == 8) ? kRowVariants : 1;
         std::vector<float> tr(nrv, 1e30f), tc(kColVariants, 1e30f);
         for (int round = 0; round < 3; ++round) {
-            for (int v = 0; v < nrv; ++v) {
+            for (int v = 0; nrv > 1 && v < nrv; ++v) {
                 // on the spectrum that a middle launch meets (the pulse after
                 // its opening half step): what the nonlinear part has to do
                 // depends on the intensities
@@ -1093,8 +1090,18 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
                 CK(launch_rows<T>(a, pu.g.nt, ctx->st), "tuning input");
                 a = row_args<T>(pu, scratch, OPS_MID, dz);
                 a.variant = v;
+                // each with a column launch behind it, as in the z-loop: row
+                // launches back to back find the field in L2 in the order
+                // they left it (six processes each, us per step: 1024 x 4096
+                // 54.2-56.2 as row launches alone chose, 54.2 in all now;
+                // 512 x 2048 16.5-17.6 and 16.5-16.9)
+                ColArgs<T> ca = col_args<T>(pu, scratch, tab, dz);
+                ca.variant = kColBlockFirst;
                 float ms;
-                int rc = time_launches(ctx, [&] { return launch_rows<T>(a, pu.g.nt, ctx->st); }, &ms);
+                int rc = time_launches(ctx, [&] {
+                    const cudaError_t e = launch_rows<T>(a, pu.g.nt, ctx->st);
+                    return e == cudaSuccess ? launch_cn<T>(ca, ctx->st) : e;
+                }, &ms);
                 if (rc) return rc;
                 tr[v] = std::min(tr[v], ms);
             }

@@ -149,7 +149,6 @@ struct NLCoef {
     T kf[2];    // hk[0] inv_is, hk[1] inv_is^2: phi = |A|^2 (kf0 + kf1 |A|^2)
     int kerr2;  // 1: the Kerr phase has the n2 and n4 terms only and kf holds it exactly
     int K;
-    int nkerr;  // number of leading Kerr orders in use (1..4; trailing zeros dropped)
     unsigned flags;
 };
 
@@ -232,13 +231,10 @@ struct RowArgs {
     int nr;
     int nt;
     int ops;
-    int variant;          // 0..2: occupancy variants; 3: persistent, next rows
-                          // prefetched by bulk copies (FP32, K = 8, Nt >= 512);
-                          // 4, 5: FFT plan 1 (radix-8 passes) with the
-                          // occupancy of variants 1, 2 (FP32, K = 8, Nt >= 256);
-                          // chosen by the autotuner
+    int variant;          // form of the kernel (FP32, K = 8, Nt >= 256; else 0):
+                          // 0, 2: one row per unit, 1: pairs, 3: by Nt, 4, 5:
+                          // FFT plan 1 (radix-8 passes); chosen by the autotuner
     NLCoef<T> nl;
-    int *err = nullptr;   // set nonzero by a kernel whose bounded wait gave up
     const cx<T> *tw1 = nullptr;   // twiddle table of FFT plan 1 (variants 4, 5)
     const cx<T> *tw2 = nullptr;   // twiddle table of FFT plan 2 (small grids), or null
     const cx<T> *in = nullptr;    // rows read from here instead of field (output
@@ -362,7 +358,7 @@ struct ColArgs {
     const cx<T> *invden;     // [nr][tp]: 1/pivot_j per |q| = 0..nt/2
     const T *lo;             // [nr]: 1 - 1/(2j) (j >= 1), 0 at j = 0
     const T *hi;             // [nr]: 1 + 1/(2j) (j >= 1), 0 at j = 0
-    const CnCoef<T> *coef = nullptr;   // [nr] row coefficients (staged variants)
+    const CnCoef<T> *coef = nullptr;   // [nr] row coefficients (variants 4..8)
     int nr, nt;
     T s;                     // dz / (4 k0 dr^2), 0 without diffraction
     T dk;                    // k'' dz/4 domega^2, 0 without dispersion: delta_q = dk q^2
@@ -527,7 +523,7 @@ template <typename T>
 bool cn_seq_supported(const ColArgs<T> &a);
 template <typename T>
 cudaError_t launch_cn_table(const TableArgs &a, cx<T> *table, cudaStream_t st);
-// Row coefficients for the staged column variants (nr rows).
+// Row coefficients for the column variants that take a table's (nr rows).
 template <typename T>
 cudaError_t launch_cn_coef(const TableArgs &a, CnCoef<T> *coef, cudaStream_t st);
 // Column stage of two pulses with the same grid and pivot table in one launch

@@ -4,10 +4,10 @@
 // Sec. 4 where the nonlinear part and the transforms share the radial
 // decomposition).
 //
-// One row (fixed radial index m) is one independent unit of work.  Rows of
-// Nt <= 4096 points run on 256 threads (several rows per CTA for Nt < 4096);
-// Nt = 8192 runs on 512 threads.  Each thread owns E = 16 complex values
-// (E = Nt when Nt < 16).
+// One row (fixed radial index m) is one independent unit of work, on Nt/16
+// threads with E = 16 complex values each (E = Nt when Nt < 16; E = 4 on
+// grids of few rows), or two adjacent rows on as many threads in packed
+// arithmetic.
 //
 // Transform: in-place decimation-in-time FFT (one radix 2/4/8 pass for the
 // factor left by radix 16, then radix-16 passes) in one padded shared-memory
@@ -1148,8 +1148,8 @@ __device__ __forceinline__ cx<V> nl_full(cx<V> a, V u, const NLCoef<T> &c) {
 // (5 levels x 4 FP64 values, of which most lanes are idle work) took as long
 // as the row's transform.  Here one warp adds for 256 threads, 13 FP64
 // additions deep, and maxima and counts are in T.  Last stage with rho and
-// statistics, 8 x 1024 rows of 4096 points, FP32: 303 -> TAILUS us; with the
-// step-doubling sums 336 -> DIFFUS us.
+// statistics, 8 x 1024 rows of 4096 points, FP32: 303 -> 209-215 us; with the
+// step-doubling sums 336-353 -> 264-285 us.
 constexpr int row_red_group(int tpr) { return tpr >= 256 ? tpr / 32 : tpr >= 8 ? 8 : tpr; }
 template <typename T, int NT, int TH, int NS, int NA, int NX, typename F>
 __device__ __forceinline__ void row_totals(const double (&s)[NS], const T (&m)[NA + NX + 1], unsigned char *smem,
@@ -1240,11 +1240,7 @@ struct RowBufs {
 };
 
 // One row stage of TH / TPR units of rows (a unit: one row, or the two
-// adjacent rows of a pair); row_base: the first unit's first row.  PF: the
-// input rows were staged in shared memory (xs: the units' rows of Nt values
-// in natural order, row_base's first) and are read from there; hook() runs
-// once every thread has finished reading them (the prefetch of the next rows
-// may then overwrite xs).
+// adjacent rows of a pair); row_base: the first unit's first row.
 //
 // MODE: what the kernel is compiled for -- ROW_PLAIN: neither rho nor
 // statistics (the launches of almost every z-step), ROW_OUT: also those,
