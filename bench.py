@@ -674,9 +674,9 @@ def run_ours(args):
     s64.close()
     # the FP64 path is bound by FP64 arithmetic: flops per point-step from the
     # ncu instruction counts of its row and column kernels (2 DFMA + DADD +
-    # DMUL: 346 + 96 per point, profiles/fp64_kernels_cfg2.md) against the
+    # DMUL: 152 + 76 per point, profiles/fp64_kernels_cfg2.md) against the
     # FP64 FMA rate measured here by the library's microkernel
-    fp64_flops_per_point_step = 442.0
+    fp64_flops_per_point_step = 228.0
     fp64_peak = fcn.alu_peak(0)
     fp64_roof = {"bound": "alu", "achieved": fp64_flops_per_point_step * v64 / world / 1e12,
                  "peak": fp64_peak / 1e12, "unit": "TFLOP/s",
