@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(MAXT, MINB) xy_line_kernel(const __grid_consta
     using V = typename LineV<T>::V;
     constexpr int NP = Pack<V>::L;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_enter();                             // the row or line launch before this one stores the same field
     const int nw = blockDim.x >> 5;
     cx<V> *sB = reinterpret_cast<cx<V> *>(smem_raw);
     cx<V> *sC = sB + nw * C;

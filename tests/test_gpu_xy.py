@@ -6,13 +6,17 @@ Tolerances (relative L2 over the compared array):
   FP64 path: 1e-10 on the field and rho;
   FP32-mixed path: 1e-4 on the field and 1e-5 on the energy.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
 
 import oracle
 from paper_1507_05988_gb300 import workloads as W
-from tests.conftest import rel_l2
+from tests.conftest import ROOT, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -157,3 +161,37 @@ def test_c64_host_calls_and_state_errors(fcn):
     with pytest.raises(fcn.FcnError):
         s.step(-1.0, 1)
     s.close()
+
+
+_PDL_RUN = """
+import sys
+import numpy as np
+from paper_1507_05988_gb300 import fcn, workloads as W
+out = {}
+for prec in (0, 1):
+    for i, (nx, ny, nt) in enumerate([(37, 29, 64), (130, 65, 256), (9, 200, 1024)]):
+        wl = W.small_xy(nx, ny, nt, p_over_pcr=3.0, noise_seed=5, dz=1e-2)
+        s = fcn.SolverXY(wl.grid(), wl.physics(), precision=prec)
+        s.set_variants(0, 3)
+        for graph in (False, True):
+            s.set_field(wl.field())
+            s.step(wl.dz, 19, graph=graph)
+            out[f"{prec}_{i}_{graph}"] = s.get_field()
+        s.close()
+np.savez(sys.argv[1], **out)
+"""
+
+
+def test_programmatic_dependent_launch_gives_the_same_bits(fcn, tmp_path):
+    """FCN_PDL=1 lets a launch start before its predecessor has ended; every
+    kernel then waits before its first access, so nothing changes.  The switch
+    is read once per process: one process per setting."""
+    res = []
+    for pdl in ("0", "1"):
+        path = tmp_path / f"pdl{pdl}.npz"
+        subprocess.run([sys.executable, "-c", _PDL_RUN, str(path)], check=True, cwd=ROOT,
+                       env=dict(os.environ, FCN_PDL=pdl), timeout=300)
+        res.append(np.load(path))
+    assert len(res[0].files) == 12
+    for k in res[0].files:
+        assert np.array_equal(res[0][k], res[1][k]), k
