@@ -9,8 +9,10 @@ int row_batch_threads(int max_nt) { return max_nt <= 2048 ? 128 : max_nt <= 4096
 
 namespace {
 // A CTA of th threads holds 16 th samples and one padding value per 16,
-// whatever its rows' Nt, and as many u values where they are kept.
-size_t batch_smem(int th, bool with_u) { return (size_t)17 * th * (with_u ? 12 : 8) + sizeof(double) * kRowScratch; }
+// whatever its rows' Nt, and as many u values in the modes that keep them.
+size_t batch_smem(int th, int mode) {
+    return (size_t)17 * th * (row_keeps_u(mode) ? 12 : 8) + sizeof(double) * kRowScratch;
+}
 
 template <typename F>
 cudaError_t with_threads(int th, F &&f) {
@@ -25,10 +27,10 @@ cudaError_t prepare_rows_batch<float>(int th) {
     return with_threads(th, [&](auto n) {
         constexpr int TH = decltype(n)::value;
         cudaError_t e = cudaFuncSetAttribute(row_batch_kernel<float, 8, TH, ROW_PLAIN>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, false));
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, ROW_PLAIN));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(row_batch_kernel<float, 8, TH, ROW_OUT>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, true));
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)batch_smem(TH, ROW_OUT));
         return e;
     });
 }
@@ -38,9 +40,9 @@ cudaError_t launch_rows_batch<float>(const RowArgs<float> *pulses, const int2 *i
                                      cudaStream_t st) {
     return with_threads(th, [&](auto n) {
         constexpr int TH = decltype(n)::value;
-        const bool out = (ops & (OP_RHO | OP_STATS | OP_SPEC)) != 0;
-        auto k = out ? row_batch_kernel<float, 8, TH, ROW_OUT> : row_batch_kernel<float, 8, TH, ROW_PLAIN>;
-        k<<<nitems, TH, batch_smem(TH, out), st>>>(pulses, items, ops);
+        const int mode = row_mode(ops) == ROW_PLAIN ? ROW_PLAIN : ROW_OUT;
+        auto k = mode == ROW_OUT ? row_batch_kernel<float, 8, TH, ROW_OUT> : row_batch_kernel<float, 8, TH, ROW_PLAIN>;
+        k<<<nitems, TH, batch_smem(TH, mode), st>>>(pulses, items, ops);
         return cudaGetLastError();
     });
 }

@@ -1229,6 +1229,14 @@ struct PlainSum {
 // pulse: TH = RowCfg<NT>::THREADS in the per-Nt kernels, 512 in the batched
 // work-list kernel.  Every thread of the CTA must call it (barriers inside).
 enum : int { ROW_PLAIN = 0, ROW_OUT = 1, ROW_DIFF = 2 };
+// The mode that launches with these operations take.
+__host__ __device__ constexpr int row_mode(int ops) {
+    return (ops & OP_DIFF) ? ROW_DIFF : (ops & (OP_RHO | OP_STATS | OP_SPEC)) ? ROW_OUT : ROW_PLAIN;
+}
+// Whether a mode's u rows have a place of their own behind the scratch
+// (otherwise the storage of S).  The kernel's layout and the shared memory of
+// its launches both follow from this.
+__host__ __device__ constexpr bool row_keeps_u(int mode) { return mode != ROW_PLAIN; }
 // The buffers of one pulse (RowArgs names them).
 template <typename T>
 struct RowBufs {
@@ -1260,21 +1268,21 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
     constexpr int RL = PassCfg<NT, PL>::R;
     constexpr int NSL = PassCfg<NT, PL>::NS;
     static_assert(RPC * C::TPR == TH, "CTA size must hold whole rows");
-    // shared memory: the rows S, the FP64 scratch, then the u rows U, which
-    // only launches with rho or statistics output allocate
+    // shared memory: the rows S, the FP64 scratch, then the u rows U of the
+    // modes that keep them (row_keeps_u)
     cx<V> *S_all = reinterpret_cast<cx<V> *>(smem_raw);
     double *scr = reinterpret_cast<double *>(S_all + RPC * C::PADN);
-    // u rows: behind the scratch where they are kept for an output, else in
-    // the storage of S (the samples are then in registers)
-    V *U_all = MODE == ROW_PLAIN ? reinterpret_cast<V *>(smem_raw) : reinterpret_cast<V *>(scr + kRowScratch);
+    // u rows: behind the scratch where an output may need them, else in the
+    // storage of S (the samples are then in registers)
+    V *U_all = row_keeps_u(MODE) ? reinterpret_cast<V *>(scr + kRowScratch) : reinterpret_cast<V *>(smem_raw);
 
 #ifdef FCN_CHECKED
     {
         unsigned dsm;
         asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dsm));
-        const bool with_u = (ops & (OP_RHO | OP_STATS)) != 0;
         if (threadIdx.x == 0)
-            FCN_IDX((sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * L * RPC * C::PADN + sizeof(double) * kRowScratch - 1,
+            FCN_IDX((sizeof(cx<T>) + (row_keeps_u(MODE) ? sizeof(T) : 0)) * L * RPC * C::PADN +
+                        sizeof(double) * kRowScratch - 1,
                     dsm, 25);
     }
 #endif
@@ -1392,7 +1400,7 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
             // every increment of the CTA's rows is exactly zero
             const bool idle = KT == 8 && m * float(a.nl.is_root) < float(u_idle<T>()) && sizeof(T) == 4;
             auto at = [&](int e) { return FCN_IDX(pidx(E * t + e, fft_nt(NT)), C::PADN, 7); };   // pass 0's positions
-            if (MODE == ROW_PLAIN) __syncthreads();      // U is the storage of S here
+            if (!row_keeps_u(MODE)) __syncthreads();      // U is the storage of S here
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 U[at(e)] = idle ? Pack<V>::splat(T(0)) : vfma(v[e].x, v[e].x, v[e].y * v[e].y);
@@ -1404,7 +1412,7 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
                 for (int e = 0; e < E; ++e)
                     v[e] = nl_full<KT, V>(v[e], with_u ? U[at(e)] : Pack<V>::splat(T(0)), a.nl);
             }
-            if (MODE == ROW_PLAIN) __syncthreads();
+            if (!row_keeps_u(MODE)) __syncthreads();
         }
         nl_kerr<V, E>(v, a.nl, plan);
     }
@@ -1708,13 +1716,13 @@ row_batch_kernel(const RowArgs<T> *__restrict__ pulses, const int2 *__restrict__
 
 namespace rowimpl {
 
-// Rows S and the FP64 scratch, plus the u rows when the launch outputs rho
-// or statistics, of a CTA of TH threads.
+// Rows S and the FP64 scratch, plus the u rows of the modes that keep them,
+// of a CTA of TH threads.
 template <typename V, int NT, int TH>
-size_t smem_bytes(bool with_u = true) {
+size_t smem_bytes(int mode) {
     using C = RowCfg<NT>;
     using T = typename Pack<V>::S;
-    return (sizeof(cx<T>) + (with_u ? sizeof(T) : 0)) * Pack<V>::L * (TH / C::TPR) * C::PADN +
+    return (sizeof(cx<T>) + (row_keeps_u(mode) ? sizeof(T) : 0)) * Pack<V>::L * (TH / C::TPR) * C::PADN +
            sizeof(double) * kRowScratch;
 }
 
@@ -1730,7 +1738,7 @@ struct RowForm {
     // Sets the dynamic shared-memory limit; must run before any launch (and
     // outside stream capture).
     static cudaError_t prepare() {
-        const int smem = (int)smem_bytes<V, NT, TH>();
+        const int smem = (int)smem_bytes<V, NT, TH>(ROW_OUT);
         cudaError_t e = cudaFuncSetAttribute(kernel<ROW_PLAIN>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kernel<ROW_OUT>(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1739,12 +1747,10 @@ struct RowForm {
         return e;
     }
     static cudaError_t launch(const RowMultiArgs<T> &m, int npulse, cudaStream_t st) {
-        const bool out = (m.a.ops & (OP_RHO | OP_STATS)) != 0;
-        const size_t smem = smem_bytes<V, NT, TH>(out);
+        const int mode = row_mode(m.a.ops);
         const dim3 grid((m.a.nr + ROWS - 1) / ROWS, npulse);
-        auto k = (m.a.ops & OP_DIFF) ? kernel<ROW_DIFF>()
-                 : (out || (m.a.ops & OP_SPEC)) ? kernel<ROW_OUT>() : kernel<ROW_PLAIN>();
-        return launch_k(k, grid, dim3(TH), smem, st, m);
+        auto k = mode == ROW_DIFF ? kernel<ROW_DIFF>() : mode == ROW_OUT ? kernel<ROW_OUT>() : kernel<ROW_PLAIN>();
+        return launch_k(k, grid, dim3(TH), smem_bytes<V, NT, TH>(mode), st, m);
     }
 };
 

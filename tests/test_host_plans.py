@@ -121,3 +121,26 @@ def test_chunked_row_io_is_a_permutation_and_cuts_bank_conflicts():
         assert key[2] == 0 and r["bad"] == 0, key
         assert r["wf_new"] <= r["wf_old"], key
     assert reals[("f32", 4096, 0)]["wf_new"] == 2 and reals[("f32", 4096, 0)]["wf_old"] == 8
+
+
+def test_row_launches_have_room_for_the_u_rows_their_kernel_places():
+    """The output modes of the row kernel keep the u rows behind the scratch,
+    whatever operation brought the launch to that mode: every launch asks for
+    that much, also one with the norm sums or the spectral moments and no
+    statistics; and no more than a block can have."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    d = tempfile.mkdtemp()
+    exe = os.path.join(d, "row_smem")
+    subprocess.run([nvcc, "-std=c++17", "-x", "cu", "-diag-suppress", "20013,1886",
+                    os.path.join(ROOT, "tests", "row_smem.cu"), "-o", exe], check=True, capture_output=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
+    shutil.rmtree(d, ignore_errors=True)
+    rho, stats, spec, diff = 16, 32, 64, 512
+    lines = [ln.split() for ln in out.splitlines()]
+    assert len(lines) == 5 * 1024
+    for f in lines:
+        ops, mode, asked, rows, u = map(int, f[3:])
+        assert (u > 0) == (mode != 0) == bool(ops & (rho | stats | spec | diff)), f
+        assert rows + u <= asked <= 227 * 1024, f
