@@ -279,25 +279,48 @@ __global__ void __launch_bounds__(MAXT, MINB) xy_line_kernel(const __grid_consta
 }
 
 // Without diffraction (s = 0) a line's factor is (1 + i delta_q) /
-// (1 - i delta_q) at every node and 0 at the walls (the table holds
-// 1/(1 - i delta_q)).
+// (1 - i delta_q) at every inner node and 0 at the walls (the table holds
+// 1/(1 - i delta_q)).  Pointwise, so bound by memory: a thread loads the
+// kXYPoint rows of its column before it stores the first.  A step in FP32,
+// us: 255 x 31 x 64 points 20, 255 x 255 x 256 221 (threads that walk the
+// batch with one load in flight 83 and 331, the line kernel with factors
+// alpha = 0 28 and 316; with diffraction 21 and 211).
+constexpr int kXYPoint = 4;
+constexpr int kXYPointTh = 256;
 template <typename T>
-__global__ void xy_point_kernel(const __grid_constant__ XYLine<T> a) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= a.width) return;
+__global__ void __launch_bounds__(kXYPointTh) xy_point_kernel(const __grid_constant__ XYLine<T> a) {
+    const int cw = min(a.width, kXYPointTh);                     // columns of the CTA, a power of two
+    const int c = blockIdx.y * cw + (int)(threadIdx.x & (cw - 1));
+    const int rb = kXYPointTh / cw;                              // rows side by side
     const int q = c & (a.nt - 1), nq = a.nt / 2 + 1;
     const int qq = (q <= a.nt / 2) ? q : a.nt - q;
     const double delta = a.dk64 * double(qq) * double(qq);
     const T dh = T(delta), dl = T(delta - double(dh));
     const DispPhase<T> ph = disp_phase<T>(a.disp, qq);
-    for (int j = blockIdx.y; j < a.n; j += gridDim.y) {
-        const Piv2<T> f = load_piv(a.invden, (size_t)(1 + j) * nq + qq);
-        for (int b = 0; b < a.batch; ++b) {
-            cx<T> *p = a.field + (size_t)b * (size_t)a.bstride + (size_t)j * (size_t)a.pitch + c;
-            const cx<T> x = *p;
-            const cx<T> r = mk(vfma(-dh, x.y, vfma(-dl, x.y, x.x)), vfma(dh, x.x, vfma(dl, x.x, x.y)));
-            *p = disp_apply(cmul2(f, r), ph);
-        }
+    const Piv2<T> inner = load_piv(a.invden, (size_t)2 * nq + qq);
+    // rows in the order in which they lie in memory
+    const bool jmajor = a.pitch > a.bstride;
+    const int fast = jmajor ? a.batch : a.n, rows = a.n * a.batch;
+    const int r0 = blockIdx.x * (rb * kXYPoint) + (int)threadIdx.x / cw;
+    cx<T> *p[kXYPoint];
+    cx<T> x[kXYPoint];
+    bool on[kXYPoint], wall[kXYPoint];
+#pragma unroll
+    for (int k = 0; k < kXYPoint; ++k) {
+        const int r = r0 + k * rb;
+        const int hi = r / fast, lo = r - hi * fast;
+        const int j = jmajor ? hi : lo, b = jmajor ? lo : hi;
+        on[k] = r < rows;
+        wall[k] = j == 0 || j == a.n - 1;
+        p[k] = a.field + ((size_t)b * (size_t)a.bstride + (size_t)j * (size_t)a.pitch + c);
+        x[k] = on[k] ? *p[k] : czero<T>();
+    }
+#pragma unroll
+    for (int k = 0; k < kXYPoint; ++k) {
+        const cx<T> r = mk(vfma(-dh, x[k].y, vfma(-dl, x[k].y, x[k].x)), vfma(dh, x[k].x, vfma(dl, x[k].x, x[k].y)));
+        Piv2<T> f = inner;
+        if (wall[k]) f.h = f.l = czero<T>();
+        if (on[k]) *p[k] = disp_apply(cmul2(f, r), ph);
     }
 }
 
@@ -334,7 +357,9 @@ cudaError_t launch_xy_line(const XYLine<T> &a, cudaStream_t st) {
     if (a.n < 3 || a.nt < 1 || (a.nt & (a.nt - 1)) || a.width < 1 || (a.width % a.nt) || a.batch < 1)
         return cudaErrorInvalidValue;
     if (!(a.s64 > kXYMinS)) {
-        xy_point_kernel<T><<<dim3((a.width + 127) / 128, a.n < 2048 ? a.n : 2048), 128, 0, st>>>(a);
+        const int cw = a.width < kXYPointTh ? a.width : kXYPointTh;
+        const int per = kXYPointTh / cw * kXYPoint;              // rows per CTA
+        xy_point_kernel<T><<<dim3((a.n * a.batch + per - 1) / per, a.width / cw), kXYPointTh, 0, st>>>(a);
         return cudaGetLastError();
     }
     constexpr bool F = sizeof(T) == 4;

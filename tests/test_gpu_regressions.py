@@ -1,0 +1,49 @@
+"""GPU: calls beside the usual ones (physics terms switched off, other photon
+numbers, uneven contexts) that have to stay as right and as fast as those."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1507_05988_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+FP64, FP32 = 0, 1
+
+
+@pytest.fixture(scope="module")
+def fcn():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    from paper_1507_05988_gb300 import build
+    build.build()
+    from paper_1507_05988_gb300 import fcn as m
+    return m
+
+
+def _best_ms(run, reps=9):
+    """Shortest of reps runs between CUDA events, after two untimed ones."""
+    out = []
+    for i in range(reps + 2):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        e0.record()
+        run()
+        e1.record()
+        torch.cuda.synchronize()
+        out.append(e0.elapsed_time(e1))
+    return min(out[2:])
+
+
+def test_cartesian_step_without_diffraction_is_no_slower(fcn):
+    """Without diffraction the line stage is pointwise.  Its step took four
+    times that with diffraction where each thread had one load in flight; a
+    factor of two leaves room for what the timing varies."""
+    wl = W.small_xy(255, 31, 64, p_over_pcr=3.0, dz=1e-3)
+    ms = {}
+    for flags in (W.ALL_PHYSICS, W.ALL_PHYSICS & ~W.DIFFRACTION):
+        s = fcn.SolverXY(wl.grid(), dict(wl.physics(), flags=flags), precision=FP32)
+        s.set_field(wl.field())
+        ms[flags] = _best_ms(lambda: s.step(wl.dz, 16))
+        s.close()
+    assert ms[W.ALL_PHYSICS & ~W.DIFFRACTION] < 2 * ms[W.ALL_PHYSICS], ms
