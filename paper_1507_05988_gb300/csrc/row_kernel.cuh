@@ -782,9 +782,15 @@ constexpr double u_idle();
 // first point), the thread's own exclusive (+)-scan in registers, then the
 // row scan for the carry that enters it.  Ends with a barrier.  Out of line:
 // few rows need it in most launches (nl_plan), and inlined it would weigh on
-// the register allocation of the path that all others take.
-template <typename V, int NT, int KT, int MB>
+// the register allocation of the path that all others take.  OUT: the launch
+// may write u or its maximum.  Otherwise only the plasma phase and the
+// saturation read it, and without them it stays unformed (decided here: as a
+// branch of the caller it cost its register allocation 1 % of a 128 x 256 FP64
+// run).  Loss alone, 1024 x 4096 points that all ionise, a step: FP32 93 -> 80
+// us, FP64 2320 -> 2005.
+template <typename V, int NT, int KT, int MB, bool OUT>
 __device__ __noinline__ void u_rows(V *U, int t, const NLCoef<typename Pack<V>::S> *cp, double *scr, int rloc) {
+    if (!OUT && !(cp->flags & (PH_PLASMA | PH_MPI_SAT))) return;
     using C = RowCfg<NT>;
     using T = typename Pack<V>::S;
     constexpr int E = C::E, L = Pack<V>::L;
@@ -1374,7 +1380,7 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
     };
 
     const bool keep_u = MODE != ROW_PLAIN && (ops & (OP_RHO | OP_STATS)) != 0;
-    const bool uses_u = (a.nl.flags & (PH_PLASMA | PH_MPI_SAT)) != 0;
+    const bool need_u = (a.nl.flags & (PH_PLASMA | PH_MPI_SAT)) || keep_u;
     const int nhalf = ((ops & OP_NL) ? 1 : 0) + ((ops & OP_NL2) ? 1 : 0);
     int plan = -1;
     bool known = false;
@@ -1395,28 +1401,25 @@ __device__ __forceinline__ void row_body(const RowArgs<typename Pack<V>::S> &a,
                     plan == nl_plan<T, NT, KT>(m * 2.002f, a.nl);
         }
         const bool out_u = MODE != ROW_PLAIN && keep_u && hs + 1 == nhalf;
-        // u is read by the plasma phase, the saturation and the outputs only
-        // (loss without either: 1024 x 4096 points that all ionise, a step
-        // 80 us in FP32 and 1990 us in FP64; with the scan 93 and 2320)
-        const bool scan = (plan < 0 && uses_u) || out_u;
-        auto at = [&](int e) { return FCN_IDX(pidx(E * t + e, fft_nt(NT)), C::PADN, 7); };   // pass 0's positions
-        if (scan) {
+        if (plan < 0 || out_u) {
             // u of every sample into U: through the scan along tau, unless
             // every increment of the CTA's rows is exactly zero
             const bool idle = KT == 8 && m * float(a.nl.is_root) < float(u_idle<T>()) && sizeof(T) == 4;
+            auto at = [&](int e) { return FCN_IDX(pidx(E * t + e, fft_nt(NT)), C::PADN, 7); };   // pass 0's positions
             if (!row_keeps_u(MODE)) __syncthreads();      // U is the storage of S here
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 U[at(e)] = idle ? Pack<V>::splat(T(0)) : vfma(v[e].x, v[e].x, v[e].y * v[e].y);
             __syncthreads();
-            if (!idle) u_rows<V, NT, KT, MB>(U, t, &a.nl, scr, rloc);
-        }
-        if (plan < 0) {
+            if (!idle) u_rows<V, NT, KT, MB, MODE != ROW_PLAIN>(U, t, &a.nl, scr, rloc);
+            if (plan < 0) {
+                const bool with_u = need_u;
 #pragma unroll
-            for (int e = 0; e < E; ++e)
-                v[e] = nl_full<KT, V>(v[e], uses_u ? U[at(e)] : Pack<V>::splat(T(0)), a.nl);
+                for (int e = 0; e < E; ++e)
+                    v[e] = nl_full<KT, V>(v[e], with_u ? U[at(e)] : Pack<V>::splat(T(0)), a.nl);
+            }
+            if (!row_keeps_u(MODE)) __syncthreads();
         }
-        if (scan && !row_keeps_u(MODE)) __syncthreads();
         nl_kerr<V, E>(v, a.nl, plan);
     }
     const bool have_u = nhalf > 0;
