@@ -948,7 +948,11 @@ __device__ __forceinline__ float cta_bound(unsigned m, double *scr, int slot) {
 
 // sin(phi) = phi (1 + phi^2 ps) and cos(phi) - 1 = phi^2 pc for |phi| below
 // the tier's bound (nl_plan): Taylor polynomials, the terms left out below
-// 2^-33 (FP32) and 2^-58 (FP64) of the result's scale.
+// 2^-33 (FP32) and 2^-58 (FP64), but for the FP32 sine, which stops at phi^9
+// also near pi/4 (tiers 3 and 4): there it is 2^-29 too large.  The roundings
+// of its coefficients and steps leave it as much too small: rows turned by
+// 0.70 to 0.785 lose 0.8e-10 to 1.2e-10 of |A|^2 per half step (2000 of them,
+// measured), and 2.6e-10 with the phi^11 term.
 template <int TIER, typename V>
 __device__ __forceinline__ void expi_poly(V p2, V *ps_out, V *pc_out) {
     using T = typename Pack<V>::S;
