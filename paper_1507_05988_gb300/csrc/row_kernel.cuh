@@ -941,7 +941,8 @@ __device__ __forceinline__ float cta_bound(unsigned m, double *scr, int slot) {
         m = __reduce_max_sync(0xffffffffu, ws[threadIdx.x & (TH / 32 - 1)]);
     }
     float f;
-    if constexpr (sizeof(T) == 8) f = __double2float_ru(__hiloint2double((int)(m + 1), 0));
+    // (the largest high word is a NaN's, and adding 1 would make it a zero)
+    if constexpr (sizeof(T) == 8) f = m < 0x7ff00000u ? __double2float_ru(__hiloint2double((int)(m + 1), 0)) : INFINITY;
     else f = __uint_as_float(m);
     return f * f * 2.00001f;
 }

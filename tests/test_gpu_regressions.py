@@ -1,5 +1,7 @@
 """GPU: calls beside the usual ones (physics terms switched off, other photon
 numbers, uneven contexts) that have to stay as right and as fast as those."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -64,3 +66,28 @@ def test_loss_without_plasma_does_not_scan(fcn, prec, nr, nt):
         ms[flags] = _best_ms(lambda: s.step(1e-6, 17))
         s.close()
     assert ms[W.KERR | W.MPI] < 0.95 * ms[W.KERR | W.MPI | W.MPI_SAT], ms
+
+
+@pytest.mark.parametrize("prec,bits", [(FP64, b << 32 | c) for b, c in ((0x7FF80000, 0), (0x7FFFFFFF, 0xFFFFFFFF),
+                                                                        (0xFFFFFFFF, 0xFFFFFFFF), (0x7FF00000, 0))] +
+                         [(FP32, b) for b in (0x7FC00000, 0x7FFFFFFF, 0xFFFFFFFF, 0x7F800000)])
+def test_a_row_that_is_not_finite_leaves_its_neighbours_alone(fcn, prec, bits):
+    """The rows of one CTA share the bound that picks their half step's form.
+    A NaN or infinity in one, whatever its bits, changes no other row (equal
+    forms: to some roundings, 1e-14 and 1e-6)."""
+    wl = W.small(8, 256, p_over_pcr=3.0, noise_seed=2)
+    g, p = fcn.grid_params(wl.physics())
+    out = []
+    for bad in (False, True):
+        f = wl.field().astype(np.complex128 if prec == FP64 else np.complex64)
+        if bad:
+            f.view(np.uint64 if prec == FP64 else np.uint32)[1, 14] = bits
+        f = torch.from_numpy(f).cuda()
+        assert fcn.fcn_op_rows(C.byref(g), C.byref(p), prec, fcn.FCN_OP_NL, 1e-2, fcn.tensor_ptr(f), None,
+                               fcn.stream_ptr()) == 0
+        torch.cuda.synchronize()
+        out.append(f.cpu().numpy().astype(np.complex128))
+    keep = [r for r in range(wl.nr) if r != 1]
+    ref, res = out[0][keep], out[1][keep]
+    assert np.linalg.norm(ref - wl.field()[keep]) > 1e-4 * np.linalg.norm(ref)        # the half step acts
+    assert np.linalg.norm(res - ref) < (1e-14 if prec == FP64 else 1e-6) * np.linalg.norm(ref)
