@@ -236,9 +236,10 @@ int fcn_set_state(fcn_ctx *ctx, int32_t pulse, const double state[4]);
  *        streamed through a shared-memory ring by TMA (Nt a multiple of 64;
  *        other grids fall back to variant 7).
  * By default (-1) the first fcn_step of a grid times every variant on a
- * scratch copy of the field and keeps the fastest per (precision, Nr, Nt)
- * for the process; if the environment variable FCN_TUNE_CACHE names a file,
- * choices are read from and appended to it.  row_variant in -1..5 and
+ * scratch copy of the field and keeps the fastest per (precision, Nr, Nt,
+ * K = 8 or not) for the process; if the environment variable FCN_TUNE_CACHE
+ * names a file, choices are read from and appended to it (lines of another
+ * version's format are passed over).  row_variant in -1..5 and
  * col_variant in -1..8 force a variant (-1: tune).  Every variant computes
  * the same step up to rounding.  Drops the context's captured graphs.
  * Synchronises. */

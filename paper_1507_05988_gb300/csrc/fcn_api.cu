@@ -13,6 +13,7 @@
 #include <cstring>
 #include <limits>
 #include <fstream>
+#include <sstream>
 #include <map>
 #include <tuple>
 #include <mutex>
@@ -1006,14 +1007,18 @@ int run_block(fcn_ctx *ctx, int kind, double dz, const std::vector<const cx<T> *
     return FCN_OK;
 }
 
-// ---- autotuner: kernel variants per (precision, Nr, Nt) ----
+// ---- autotuner: kernel variants per (precision, Nr, Nt, K = 8 or not) ----
 // Variants change register allocation (row stage) or the chunk length and
 // CTA size (column stage); all compute the same step, the column variants
 // with a different rounding order.  The first fcn_step of a grid times every
 // variant on a scratch copy of the field (a few launches each, CUDA events)
 // and keeps the fastest in a process-wide table, optionally persisted in the
-// text file named by FCN_TUNE_CACHE ("prec nr nt row col" per line).
-std::map<std::tuple<int, int, int>, std::pair<int, int>> g_tune;
+// text file named by FCN_TUNE_CACHE ("format prec nr nt k8 row col" per line).
+// k8: the row variants serve K = 8 only, and others' choice of column variant
+// comes with row variant 0.  The format's name changes with the variants'
+// meaning; lines of another one are passed over.
+constexpr char kTuneFormat[] = "fcn-variants-2";
+std::map<std::tuple<int, int, int, bool>, std::pair<int, int>> g_tune;
 bool g_tune_loaded = false;
 
 void tune_cache_load() {
@@ -1022,17 +1027,21 @@ void tune_cache_load() {
     const char *path = std::getenv("FCN_TUNE_CACHE");
     if (!path) return;
     std::ifstream f(path);
-    int prec, nr, nt, rv, cv;
-    while (f >> prec >> nr >> nt >> rv >> cv)
-        if (rv >= 0 && rv < kRowVariants && cv >= 0 && cv < kColVariants)
-            g_tune[std::make_tuple(prec, nr, nt)] = {rv, cv};
+    for (std::string line; std::getline(f, line);) {
+        std::istringstream in(line);
+        std::string format;
+        int prec, nr, nt, k8, rv, cv;
+        if (in >> format >> prec >> nr >> nt >> k8 >> rv >> cv && format == kTuneFormat && rv >= 0 &&
+            rv < kRowVariants && cv >= 0 && cv < kColVariants)
+            g_tune[std::make_tuple(prec, nr, nt, k8 != 0)] = {rv, cv};
+    }
 }
 
-void tune_cache_store(int prec, int nr, int nt, int rv, int cv) {
+void tune_cache_store(int prec, int nr, int nt, bool k8, int rv, int cv) {
     const char *path = std::getenv("FCN_TUNE_CACHE");
     if (!path) return;
     std::ofstream f(path, std::ios::app);
-    f << prec << " " << nr << " " << nt << " " << rv << " " << cv << "\n";
+    f << kTuneFormat << " " << prec << " " << nr << " " << nt << " " << k8 << " " << rv << " " << cv << "\n";
 }
 
 // 3 untimed then 15 timed launches (variants differ by a few per cent, so
@@ -1062,7 +1071,8 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
     const int prec = ctx->prec;
     std::lock_guard<std::mutex> lk(g_mu);
     tune_cache_load();
-    auto key = std::make_tuple(prec, pu.g.nr, pu.g.nt);
+    const bool k8 = pu.p.K == 8;
+    auto key = std::make_tuple(prec, (int)pu.g.nr, (int)pu.g.nt, k8);
     auto it = g_tune.find(key);
     if (it == g_tune.end()) {
         // a private scratch copy: the context's work buffers may hold state
@@ -1077,7 +1087,7 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
         // three interleaved rounds over the variants, each variant's best
         // round counts (a burst of noise on the GPU then decides nothing);
         // FP64 and other K have one row form
-        const int nrv = (sizeof(T) == 4 && pu.p.K == 8) ? kRowVariants : 1;
+        const int nrv = (sizeof(T) == 4 && k8) ? kRowVariants : 1;
         std::vector<float> tr(nrv, 1e30f), tc(kColVariants, 1e30f);
         for (int round = 0; round < 3; ++round) {
             for (int v = 0; nrv > 1 && v < nrv; ++v) {
@@ -1118,7 +1128,7 @@ int tune_pulse(fcn_ctx *ctx, Pulse &pu, const cx<T> *tab, double dz) {
         const int best_c = int(std::min_element(tc.begin(), tc.end()) - tc.begin());
         CK(cudaStreamSynchronize(ctx->st), "tuning sync");
         it = g_tune.emplace(key, std::make_pair(best_r, best_c)).first;
-        tune_cache_store(prec, pu.g.nr, pu.g.nt, best_r, best_c);
+        tune_cache_store(prec, pu.g.nr, pu.g.nt, k8, best_r, best_c);
     }
     pu.row_var = ctx->force_row >= 0 ? ctx->force_row : it->second.first;
     pu.col_var = ctx->force_col >= 0 ? ctx->force_col : it->second.second;

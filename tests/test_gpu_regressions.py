@@ -1,12 +1,16 @@
 """GPU: calls beside the usual ones (physics terms switched off, other photon
 numbers, uneven contexts) that have to stay as right and as fast as those."""
 import ctypes as C
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
 import torch
 
 from paper_1507_05988_gb300 import workloads as W
+from tests.conftest import ROOT
 
 pytestmark = pytest.mark.gpu
 
@@ -91,3 +95,30 @@ def test_a_row_that_is_not_finite_leaves_its_neighbours_alone(fcn, prec, bits):
     ref, res = out[0][keep], out[1][keep]
     assert np.linalg.norm(ref - wl.field()[keep]) > 1e-4 * np.linalg.norm(ref)        # the half step acts
     assert np.linalg.norm(res - ref) < (1e-14 if prec == FP64 else 1e-6) * np.linalg.norm(ref)
+
+
+_TUNE_RUN = """
+from paper_1507_05988_gb300 import fcn, workloads as W
+wl = W.small(64, 256)
+for K in (7, 8, 8):
+    s = fcn.Solver(dict(wl.physics(), K=K), precision=fcn.FCN_FP32_MIXED)
+    s.set_field(wl.field())
+    s.step(1e-3, 2)
+    s.close()
+"""
+
+
+def test_variant_choices_by_photon_number_and_format(fcn, tmp_path):
+    """The row variants serve K = 8 only: another K's choice (variant 0,
+    untimed) is not a K = 8 context's.  Lines of an older format, whose numbers
+    meant other kernels, are passed over, and this format's are read back."""
+    path = tmp_path / "variants"
+    path.write_text("1 64 256 5 3\n")
+    for _ in range(2):
+        subprocess.run([sys.executable, "-c", _TUNE_RUN], check=True, cwd=ROOT, timeout=300,
+                       env=dict(os.environ, FCN_TUNE_CACHE=str(path)))
+        lines = path.read_text().splitlines()
+        assert lines[0] == "1 64 256 5 3" and len(lines) == 3
+        fmt = {ln.split()[0] for ln in lines[1:]}
+        assert len(fmt) == 1 and not fmt.pop().isdigit()
+        assert [ln.split()[1:5] for ln in lines[1:]] == [["1", "64", "256", "0"], ["1", "64", "256", "1"]]
