@@ -1804,12 +1804,15 @@ int setup_batch(fcn_ctx *ctx) {
     return FCN_OK;
 }
 
-// Automatic choice: the work lists pay off when the grids differ and most
-// of the batch's points lie in pulses whose own row launch cannot fill the
-// GPU (fewer row CTAs than twice the SM count), which a launch per pulse
-// would serialise as part-empty launches.  Measured on GB300: 64 uneven
-// pulses of Nr 64-256 x Nt 512-1024 run 5.8x faster batched; the 64 pulses
-// of Nr 256-2048 x Nt 512-8192 run 6 % faster as tuned per-pulse launches.
+// Automatic choice: the work lists save launches, but their column CTAs are
+// sized for the tallest pulse.  They run when the grids differ and the points
+// per pulse, counted with the largest Nr in every one, are on average fewer
+// than the row kernels hold on the GPU at once (640 threads of 16 values per
+// SM: 1.56e6 on 152 SMs).  us per step, work lists / launches per pulse, of 4
+// pulses of P points each: Nt 2048 and 1024 (average 1.5 P): P = 4e5 35 / 47,
+// 8e5 54 / 60, 1.2e6 88 / 83, 1.6e6 128 / 105; 8192 and 4096: 8e5 56 / 73,
+// 1.2e6 95 / 90; 4096 and 512 (4.5 P): 2e5 36 / 43, 4e5 47 / 51, 8e5 90 / 63;
+// 8192 and 512 (8.5 P): 4e5 66 / 60, 8e5 129 / 72.
 // Identical grids always run per-pulse (paired) launches.
 bool grids_uneven(const fcn_ctx *ctx) {
     for (auto &pu : ctx->pulses)
@@ -1817,20 +1820,16 @@ bool grids_uneven(const fcn_ctx *ctx) {
     return false;
 }
 
-bool small_pulses_dominate(const fcn_ctx *ctx) {
+bool work_lists_pay(const fcn_ctx *ctx) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    double small = 0.0, all = 0.0;
+    double max_nr = 0.0, sum_nt = 0.0;
     for (auto &pu : ctx->pulses) {
-        const int tpr = pu.g.nt >= 16 ? pu.g.nt / 16 : 1;
-        const int rpc = tpr >= 256 ? 1 : 256 / tpr;           // rows per CTA of the per-Nt kernels
-        const int ctas = (pu.g.nr + rpc - 1) / rpc;
-        const double pts = (double)pu.points();
-        all += pts;
-        if (ctas < 2 * sms) small += pts;
+        max_nr = std::max(max_nr, (double)pu.g.nr);
+        sum_nt += (double)pu.g.nt;
     }
-    return small > 0.5 * all;
+    return max_nr * sum_nt < 640.0 * 16.0 * sms * (double)ctx->pulses.size();
 }
 
 int create_impl(int n, const fcn_grid *grids, const fcn_params *params, int prec, void *stream,
@@ -1909,7 +1908,7 @@ int create_impl(int n, const fcn_grid *grids, const fcn_params *params, int prec
     if (n > 1 && prec == FCN_FP32_MIXED) {
         int rc = setup_batch(ctx);
         if (rc) return bail(rc);
-        ctx->batched = ctx->row_items != nullptr && grids_uneven(ctx) && small_pulses_dominate(ctx);
+        ctx->batched = ctx->row_items != nullptr && grids_uneven(ctx) && work_lists_pay(ctx);
     }
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) { cuda_fail(ctx, e, "init sync"); return bail(FCN_ERR_CUDA); }
     *out = ctx;
@@ -2194,7 +2193,7 @@ int fcn_set_batching(fcn_ctx *ctx, int32_t mode) {
     const bool possible = ctx->row_items != nullptr;
     if (mode == 1 && !possible)
         return fail(ctx, FCN_ERR_UNSUPPORTED, "work lists need several FP32 pulses with K = 8 and Nt >= 512");
-    const bool want = mode == 1 || (mode == -1 && possible && grids_uneven(ctx) && small_pulses_dominate(ctx));
+    const bool want = mode == 1 || (mode == -1 && possible && grids_uneven(ctx) && work_lists_pay(ctx));
     if (want != ctx->batched) {
         drop_graphs(ctx, true, 0);
         ctx->batched = want;

@@ -9,8 +9,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1507_05988_gb300 import workloads as W
-from tests.conftest import ROOT
+from tests.conftest import ROOT, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -122,3 +123,36 @@ def test_variant_choices_by_photon_number_and_format(fcn, tmp_path):
         fmt = {ln.split()[0] for ln in lines[1:]}
         assert len(fmt) == 1 and not fmt.pop().isdigit()
         assert [ln.split()[1:5] for ln in lines[1:]] == [["1", "64", "256", "0"], ["1", "64", "256", "1"]]
+
+
+# both sides of the line between work lists and launches per pulse, and a pair
+# of like size whose tall pulse would leave the other's column CTAs half empty
+@pytest.mark.parametrize("shapes,lists", [(((390, 2048), (781, 1024)), True), (((585, 2048), (1171, 1024)), False),
+                                          (((97, 8192), (195, 4096)), True), (((195, 4096), (1562, 512)), False)])
+def test_work_lists_by_the_size_of_the_pulses(fcn, shapes, lists):
+    s = fcn.Solver([W.small(nr, nt).physics() for nr, nt in shapes], precision=FP32)
+    for i, (nr, nt) in enumerate(shapes):
+        s.set_field(np.zeros((nr, nt), np.complex128), pulse=i)
+    s.step(1e-3, 1)
+    s.profile(True)
+    s.profile_read()
+    s.step(1e-3, 1)
+    n = s.profile_read()
+    s.close()
+    assert [n[k][1] for k in ("row_head", "column", "row_tail")] == [1 if lists else 2] * 3
+
+
+@pytest.mark.parametrize("shapes", [((256, 512), (3, 1024)), ((512, 512), (257, 2048)), ((513, 512), (9, 4096))])
+def test_forced_work_lists(fcn, shapes):
+    """Column CTAs of each size, whatever the automatic choice: 1e-5 after
+    three steps, as for the launches per pulse."""
+    wls = [W.small(nr, nt, p_over_pcr=2.0 + k, noise_seed=k + 1) for k, (nr, nt) in enumerate(shapes)]
+    s = fcn.Solver([w.physics() for w in wls], precision=FP32)
+    s.set_batching(1)
+    for i, w in enumerate(wls):
+        s.set_field(w.field(), pulse=i)
+    s.step(2e-3, 3)
+    outs = [s.get_field(i) for i in range(len(wls))]
+    s.close()
+    for out, w in zip(outs, wls):
+        assert rel_l2(out, oracle.run(oracle.Problem(**w.physics()), 2e-3, 3, w.field())[0]) < 1e-5, w.name
