@@ -249,9 +249,9 @@ int fcn_set_variants(fcn_ctx *ctx, int32_t row_variant, int32_t col_variant);
  * Nt >= 512): mode 1 runs each stage of all pulses as one launch over a list
  * of (pulse, rows) and (pulse, column group) items; 0 launches each pulse
  * separately (tuned per-Nt kernels, all inside one CUDA graph); -1 (the
- * default) uses the work lists when the grids differ and the pulses, counted
- * with the largest Nr in every one, have on average too few points to fill the
- * GPU with a launch of their own.  Drops the captured graphs.  FCN_ERR_UNSUPPORTED if mode 1 is not possible. */
+ * default) uses the work lists when the grids differ and an estimate from the
+ * grids puts them ahead (pulses too small to fill the GPU with launches of
+ * their own).  Drops the captured graphs.  FCN_ERR_UNSUPPORTED if mode 1 is not possible. */
 int fcn_set_batching(fcn_ctx *ctx, int32_t mode);
 
 /* Paired column launches for FP32 contexts whose pulses all share one grid

@@ -1804,15 +1804,17 @@ int setup_batch(fcn_ctx *ctx) {
     return FCN_OK;
 }
 
-// Automatic choice: the work lists save launches, but their column CTAs are
-// sized for the tallest pulse.  They run when the grids differ and the points
-// per pulse, counted with the largest Nr in every one, are on average fewer
-// than the row kernels hold on the GPU at once (640 threads of 16 values per
-// SM: 1.56e6 on 152 SMs).  us per step, work lists / launches per pulse, of 4
-// pulses of P points each: Nt 2048 and 1024 (average 1.5 P): P = 4e5 35 / 47,
-// 8e5 54 / 60, 1.2e6 88 / 83, 1.6e6 128 / 105; 8192 and 4096: 8e5 56 / 73,
-// 1.2e6 95 / 90; 4096 and 512 (4.5 P): 2e5 36 / 43, 4e5 47 / 51, 8e5 90 / 63;
-// 8192 and 512 (8.5 P): 4e5 66 / 60, 8e5 129 / 72.
+// Automatic choice where the grids differ: the work lists save launches, but
+// their column CTAs are sized for the tallest pulse.  Estimates in us per step,
+// fitted to 2, 4 and 12 pulses of 1e5 to 8e6 points each (Nt 512 to 8192; the
+// larger grid's Nt twice to 16 times the other's) on 152 SMs, within 28 % of
+// the measured times.  A launch per pulse and stage: 9 + Nt/850 for the
+// launches and 14.7 per 1e6 points, joined as hypot; the lists: 12 per 1e6
+// points and 4.3 per 1e6 counted with the largest Nr in every pulse, and 13 for
+// the launches.  Measured, lists / per pulse, 4 pulses of P points: Nt 2048 and
+// 1024, P = 4e5 35 / 47, 8e5 54 / 60, 1.2e6 88 / 83, 1.6e6 128 / 105; 8192 and
+// 4096, 8e5 56 / 73, 1.6e6 155 / 121; 4096 and 512, 2e5 36 / 43, 8e5 90 / 63;
+// 63 pulses of Nr 64-256, Nt 512 and 1024 with one of 2048 x 1024: 513 / 636.
 // Identical grids always run per-pulse (paired) launches.
 bool grids_uneven(const fcn_ctx *ctx) {
     for (auto &pu : ctx->pulses)
@@ -1821,15 +1823,14 @@ bool grids_uneven(const fcn_ctx *ctx) {
 }
 
 bool work_lists_pay(const fcn_ctx *ctx) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    double max_nr = 0.0, sum_nt = 0.0;
+    double max_nr = 0.0, sum_nt = 0.0, points = 0.0, each = 0.0;
     for (auto &pu : ctx->pulses) {
         max_nr = std::max(max_nr, (double)pu.g.nr);
         sum_nt += (double)pu.g.nt;
+        points += (double)pu.points();
+        each += std::hypot(9.0 + pu.g.nt / 850.0, 14.7e-6 * (double)pu.points());
     }
-    return max_nr * sum_nt < 640.0 * 16.0 * sms * (double)ctx->pulses.size();
+    return std::hypot(13.0, 12e-6 * points + 4.3e-6 * max_nr * sum_nt) < each;
 }
 
 int create_impl(int n, const fcn_grid *grids, const fcn_params *params, int prec, void *stream,

@@ -125,10 +125,12 @@ def test_variant_choices_by_photon_number_and_format(fcn, tmp_path):
         assert [ln.split()[1:5] for ln in lines[1:]] == [["1", "64", "256", "0"], ["1", "64", "256", "1"]]
 
 
-# both sides of the line between work lists and launches per pulse, and a pair
-# of like size whose tall pulse would leave the other's column CTAs half empty
-@pytest.mark.parametrize("shapes,lists", [(((390, 2048), (781, 1024)), True), (((585, 2048), (1171, 1024)), False),
-                                          (((97, 8192), (195, 4096)), True), (((195, 4096), (1562, 512)), False)])
+# both sides of the line between work lists and launches per pulse, pulses of
+# like size whose tall one would leave the other's column CTAs half empty, and
+# many small pulses beside a tall one
+@pytest.mark.parametrize("shapes,lists", [(((195, 2048), (390, 1024)), True), (((585, 2048), (1171, 1024)), False),
+                                          (((97, 8192), (195, 4096)), True), (((195, 4096), (1562, 512)), False),
+                                          (((128, 512),) * 16 + ((2048, 1024),), True)])
 def test_work_lists_by_the_size_of_the_pulses(fcn, shapes, lists):
     s = fcn.Solver([W.small(nr, nt).physics() for nr, nt in shapes], precision=FP32)
     for i, (nr, nt) in enumerate(shapes):
@@ -139,7 +141,7 @@ def test_work_lists_by_the_size_of_the_pulses(fcn, shapes, lists):
     s.step(1e-3, 1)
     n = s.profile_read()
     s.close()
-    assert [n[k][1] for k in ("row_head", "column", "row_tail")] == [1 if lists else 2] * 3
+    assert [n[k][1] for k in ("row_head", "column", "row_tail")] == [1 if lists else len(shapes)] * 3
 
 
 @pytest.mark.parametrize("shapes", [((256, 512), (3, 1024)), ((512, 512), (257, 2048)), ((513, 512), (9, 4096))])
