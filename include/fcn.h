@@ -234,7 +234,7 @@ int fcn_set_state(fcn_ctx *ctx, int32_t pulse, const double state[4]);
  *        per-dz table, in four shapes (rows per thread x columns per CTA);
  *   8    one sequential Thomas sweep per column, 32 columns per warp, rows
  *        streamed through a shared-memory ring by TMA (Nt a multiple of 64;
- *        other grids fall back to variant 7).
+ *        other grids fall back to variant 4).
  * By default (-1) the first fcn_step of a grid times every variant on a
  * scratch copy of the field and keeps the fastest per (precision, Nr, Nt,
  * K = 8 or not) for the process; if the environment variable FCN_TUNE_CACHE

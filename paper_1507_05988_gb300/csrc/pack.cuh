@@ -1,5 +1,5 @@
 // pack.cuh -- packed pairs of FP32 values: the same quantity of two rows (row
-// stage) or two pulses (column stage) in the halves of one 64-bit register
+// stage) or two lines (Cartesian line stage) in the halves of one 64-bit register
 // pair, one add/mul/fma.rn.f32x2 per operation of both (each half an IEEE
 // single operation; constants and coefficients are shared by the halves).
 #pragma once

@@ -117,7 +117,7 @@ __host__ __device__ constexpr double cos16(int m) {
 // is applied as a two-float (hi + lo) pair inside the FMAs that multiply by
 // it: the pi/8 family here, 1/sqrt(2) for the pi/4 family, and the twiddles
 // (tw_mul).  Together with the inverse transform being the exact adjoint of
-// the forward one (InvDispatch), the constants then leave errors at the
+// the forward one (inverse_fft), the constants then leave errors at the
 // level of the random rounding of the arithmetic only.
 __device__ __forceinline__ void c16f_pair2(int m, float *ch, float *cl, float *sh, float *sl) {
     // cos(pi/8), sin(pi/8) = hi + lo (hi the nearest float, lo the nearest
@@ -1235,10 +1235,10 @@ struct PlainSum {
 };
 
 // MB: minimum resident CTAs per SM requested from the compiler (register cap
-// 64K / (MB * THREADS)); the autotuner picks it per (precision, Nt).
-// One CTA of TH threads processes rows [row_base, row_base + TH/TPR) of one
-// pulse: TH = RowCfg<NT>::THREADS in the per-Nt kernels, 512 in the batched
-// work-list kernel.  Every thread of the CTA must call it (barriers inside).
+// 64K / (MB TH)).  One CTA of TH threads processes the rows of TH/TPR units
+// from row_base on, of one pulse; TH and MB by form (RowForm), in the work-list
+// kernel by the list's largest Nt.  Every thread of the CTA must call it
+// (barriers inside).
 enum : int { ROW_PLAIN = 0, ROW_OUT = 1, ROW_DIFF = 2 };
 // The mode that launches with these operations take.
 __host__ __device__ constexpr int row_mode(int ops) {
@@ -1685,7 +1685,9 @@ row_kernel(const __grid_constant__ RowMultiArgs<typename Pack<V>::S> m) {
     const int y = blockIdx.y;
     if (threadIdx.x == 0) {
         // the rows of the CTA that takes this one's place, into L2: CTAs
-        // start in order, about kResident after one another
+        // start in order, about kResident after one another (on 152 SMs; a
+        // distance from the device and the form's true residency left seven
+        // other cases as they are and 2048 x 8192 1.5 % slower)
         constexpr int kResident = 152 * (MB > 1 ? MB : 2);
         const unsigned n = blockIdx.x + kResident, yn = y + n / gridDim.x, xn = n % gridDim.x;
         const int row0 = (int)xn * ROWS, rows = min(ROWS, m.a.nr - row0);
