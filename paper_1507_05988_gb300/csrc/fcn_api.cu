@@ -1815,7 +1815,9 @@ int setup_batch(fcn_ctx *ctx) {
 // 1024, P = 4e5 35 / 47, 8e5 54 / 60, 1.2e6 88 / 83, 1.6e6 128 / 105; 8192 and
 // 4096, 8e5 56 / 73, 1.6e6 155 / 121; 4096 and 512, 2e5 36 / 43, 8e5 90 / 63;
 // 63 pulses of Nr 64-256, Nt 512 and 1024 with one of 2048 x 1024: 513 / 636.
-// Identical grids always run per-pulse (paired) launches.
+// Also, most points have to lie in pulses that the row kernels hold on the GPU
+// at once (640 threads of 16 values per SM): a large pulse that dominates keeps
+// its tuned launches.  Identical grids always run per-pulse (paired) launches.
 bool grids_uneven(const fcn_ctx *ctx) {
     for (auto &pu : ctx->pulses)
         if (pu.g.nr != ctx->pulses[0].g.nr || pu.g.nt != ctx->pulses[0].g.nt) return true;
@@ -1823,14 +1825,18 @@ bool grids_uneven(const fcn_ctx *ctx) {
 }
 
 bool work_lists_pay(const fcn_ctx *ctx) {
-    double max_nr = 0.0, sum_nt = 0.0, points = 0.0, each = 0.0;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    double max_nr = 0.0, sum_nt = 0.0, points = 0.0, small = 0.0, each = 0.0;
     for (auto &pu : ctx->pulses) {
+        if (pu.points() < (int64_t)640 * 16 * sms) small += (double)pu.points();
         max_nr = std::max(max_nr, (double)pu.g.nr);
         sum_nt += (double)pu.g.nt;
         points += (double)pu.points();
         each += std::hypot(9.0 + pu.g.nt / 850.0, 14.7e-6 * (double)pu.points());
     }
-    return std::hypot(13.0, 12e-6 * points + 4.3e-6 * max_nr * sum_nt) < each;
+    return small > 0.5 * points && std::hypot(13.0, 12e-6 * points + 4.3e-6 * max_nr * sum_nt) < each;
 }
 
 int create_impl(int n, const fcn_grid *grids, const fcn_params *params, int prec, void *stream,

@@ -130,7 +130,7 @@ def test_variant_choices_by_photon_number_and_format(fcn, tmp_path):
 # many small pulses beside a tall one
 @pytest.mark.parametrize("shapes,lists", [(((195, 2048), (390, 1024)), True), (((585, 2048), (1171, 1024)), False),
                                           (((97, 8192), (195, 4096)), True), (((195, 4096), (1562, 512)), False),
-                                          (((128, 512),) * 16 + ((2048, 1024),), True)])
+                                          (((128, 512),) * 40 + ((2048, 1024),), True)])
 def test_work_lists_by_the_size_of_the_pulses(fcn, shapes, lists):
     s = fcn.Solver([W.small(nr, nt).physics() for nr, nt in shapes], precision=FP32)
     for i, (nr, nt) in enumerate(shapes):
