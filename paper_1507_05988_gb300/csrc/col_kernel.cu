@@ -96,7 +96,6 @@ __device__ __forceinline__ CnCoef<T> cn_coef_row(const TableArgs &a, int j) {
         c.sh = T(vh);
         c.sll = T(vl - double(c.sl));
         c.shl = T(vh - double(c.sh));
-        c.c0 = T((j == 0 ? 4.0 : 2.0) * a.s);
         c.d = T(1);
     }
     return c;

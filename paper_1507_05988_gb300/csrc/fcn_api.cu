@@ -85,21 +85,12 @@ template <typename T>
 NLCoef<T> nl_coef(const fcn_grid &g, const fcn_params &p, double h) {
     const Consts c = derive(g, p);
     NLCoef<T> n;
-    n.h = T(h);
-    double isj = kIs;
-    for (int j = 0; j < 4; ++j) {
-        n.kerr[j] = T((c.k0 / p.n0) * p.n2j[j] * isj);
-        isj *= kIs;
-    }
-    n.plasma = T(c.k0 / (2.0 * p.n0 * p.n0 * c.rho_c) * p.rho_nt);
-    n.loss = T(0.5 * c.beta_k * std::pow(kIs, p.K - 1));
-    n.sdt = T(p.sigma_k * c.dtau * std::pow(kIs, p.K));
     n.inv_is = T(1.0 / kIs);
     n.inv_nt = T(1.0 / double(g.nt));
     n.rho_nt = T(p.rho_nt);
     n.K = p.K;
     n.flags = p.flags;
-    isj = kIs;
+    double isj = kIs;
     for (int j = 0; j < 4; ++j) {
         n.hk[j] = (p.flags & FCN_KERR) ? T(h * (c.k0 / p.n0) * p.n2j[j] * isj) : T(0);
         isj *= kIs;
@@ -735,11 +726,10 @@ template <typename T>
 bool same_row_launch(const RowArgs<T> &a, const RowArgs<T> &b) {
     const NLCoef<T> &x = a.nl, &y = b.nl;
     bool same = a.nr == b.nr && a.nt == b.nt && a.tw == b.tw && a.ops == b.ops && a.variant == b.variant &&
-                x.h == y.h && x.plasma == y.plasma && x.loss == y.loss && x.sdt == y.sdt &&
                 x.inv_is == y.inv_is && x.inv_nt == y.inv_nt && x.rho_nt == y.rho_nt &&
                 x.hplasma == y.hplasma && x.hloss == y.hloss && x.sat == y.sat && x.is_root == y.is_root &&
                 x.K == y.K && x.flags == y.flags;
-    for (int j = 0; j < 4; ++j) same = same && x.kerr[j] == y.kerr[j] && x.hk[j] == y.hk[j];
+    for (int j = 0; j < 4; ++j) same = same && x.hk[j] == y.hk[j];
     return same;
 }
 

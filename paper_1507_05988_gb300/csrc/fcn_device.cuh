@@ -125,22 +125,18 @@ enum : int {
 
 // Coefficients of one nonlinear half step in scaled intensity units
 // Ihat = I / I_s (I_s a power of two, so the scaling is exact).
-//   phase rate  = sum_j kerr[j] Ihat^(j+1) - plasma * u        [rad/m]
-//   loss rate   = loss * Ihat^(K-1) [* (1 - u)]                [1/m]
-//   RK4 step of u = rho/rho_nt along tau uses x = sdt * Ihat^K (= dtau w)
+//   phase rate  = sum_j kerr_j Ihat^(j+1) - plasma u           [rad/m]
+//   loss rate   = loss Ihat^(K-1) [* (1 - u)]                  [1/m]
+//   RK4 step of u = rho/rho_nt along tau uses x = sdt Ihat^K (= dtau w)
+// with kerr_j = (k0/n0) n_2j I_s^j, plasma = k0/(2 n0^2 rho_c) rho_nt, loss =
+// (beta_K/2) I_s^(K-1), sdt = sigma_K dtau I_s^K; the half-step length h and the
+// physics switches are folded in (a switched-off term has a zero coefficient,
+// so the kernel needs no per-point flag tests).
 template <typename T>
 struct NLCoef {
-    T h;        // half-step length dz/2 [m]
-    T kerr[4];  // (k0/n0) n_2j I_s^j
-    T plasma;   // k0/(2 n0^2 rho_c) rho_nt
-    T loss;     // (beta_K/2) I_s^(K-1)
-    T sdt;      // sigma_K dtau I_s^K
     T inv_is;   // 1 / I_s
     T inv_nt;   // 1 / Nt (applied after the inverse FFT)
     T rho_nt;   // rho = u rho_nt for the rho output
-    // The same terms as the row kernel uses them, with the half-step length
-    // and the physics switches folded in (a switched-off term has a zero
-    // coefficient, so the kernel needs no per-point flag tests):
     T hk[4];    // h kerr_j, or 0 without the Kerr term
     T hplasma;  // h plasma, or 0 without plasma defocusing
     T hloss;    // h loss, or 0 without MPI loss
@@ -265,7 +261,8 @@ struct RowMultiArgs {
 //   sweep factors  alpha_j = i sl / piv_j,  gamma_j = i sh / piv_j.
 // Row 0 (symmetry axis): sl = 0, sh = c0 = 4s, d = 1; rows 1..Nr-2:
 // sl = s lo_j, sh = s hi_j, c0 = 2s, d = 1; the boundary row Nr-1 and the
-// padding rows of a ragged last chunk are all zero (A = 0 there).
+// padding rows of a ragged last chunk are all zero (A = 0 there).  c0 comes
+// with delta_q per column (CdCol).
 //
 // In FP32 the explicit side takes every coefficient as a two-float pair
 // (hi + lo, lo = the FP32 rounding error of the FP64 value): rounded once,
@@ -276,8 +273,8 @@ struct RowMultiArgs {
 // column from the FP64 s and dk (CdCol).  The sweep factors keep sl and sh.
 template <typename T>
 struct alignas(8 * sizeof(T)) CnCoef {
-    T sl, sh, c0, d;
-    T sll, shl, pad0, pad1;
+    T sl, sh, pad0, d;
+    T sll, shl, pad1, pad2;
 };
 
 // c0 - delta_q of one column as two-float pairs, for the axis row (c0 = 4s)
@@ -571,9 +568,8 @@ struct XYLine {
     int n, nt, width, batch;
     long long pitch, bstride;
     long long total;         // elements of the field buffer
-    T s;                     // dz / (4 k0 h^2), 0 without diffraction
-    T dk;                    // delta_q = dk q^2 (0 in a line without dispersion)
-    double s64, dk64;        // s and dk in FP64 (two-float explicit side in FP32)
+    double s64;              // dz / (4 k0 h^2), 0 without diffraction
+    double dk64;             // delta_q = dk64 q^2 (0 in a line without dispersion)
     double disp;             // exact dispersion factor exp(2 i disp q^2), 0: none
     // chunk length, columns per CTA and CTA size (launch_xy_line)
     int variant;

@@ -69,7 +69,6 @@ struct RowCfg {
     static constexpr int E = PLAN == 2 ? 4 : N < 16 ? N : 16;   // values per thread
     static constexpr int TPR = N / E;                       // threads per row
     static constexpr int THREADS = TPR >= 256 ? TPR : 256;  // CTA size
-    static constexpr int RPC = THREADS / TPR;               // rows per CTA
     static constexpr int PADN = N >= 16 ? N + N / 16 : N;
     static constexpr int NPASS = fft_npass(NT);
     static constexpr int WARPS_PER_ROW = TPR > 32 ? TPR / 32 : 1;

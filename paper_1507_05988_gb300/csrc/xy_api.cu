@@ -151,8 +151,6 @@ XYLine<T> line_args(fcn_xy_ctx *ctx, void *field, int axis, double dz) {
         a.pitch = ctx->g.nt;
         a.bstride = (long long)ctx->g.ny * ctx->g.nt;
     }
-    a.s = T(s);
-    a.dk = T(dk);
     a.s64 = s;
     a.dk64 = dk;
     a.disp = disp;

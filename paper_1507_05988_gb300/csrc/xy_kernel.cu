@@ -367,7 +367,7 @@ cudaError_t launch_xy_line(const XYLine<T> &a, cudaStream_t st) {
     cudaError_t e = cudaErrorInvalidConfiguration;
     switch (a.variant) {
         case 1: e = launch_form<T, LS, 8 / CF, 256, 2>(a, st); break;
-        case 2: e = launch_form<T, F ? 8 : 8, 8 / CF, 512, 1>(a, st); break;
+        case 2: e = launch_form<T, 8, 8 / CF, 512, 1>(a, st); break;
         case 3: e = launch_form<T, LS, 4 / CF, 256, 2>(a, st); break;
         case 4: e = launch_form<T, LL, 8 / CF, 256, 1>(a, st); break;
         case 5: e = launch_form<T, LL, 16 / CF, 512, 1>(a, st); break;
