@@ -9,7 +9,8 @@
 // Optional self-checking build (-DFCN_CHECKED, used to locate memory faults):
 // every indexed access in the kernels goes through FCN_IDX, which prints the
 // site and index of the first violations and redirects the access to index 0
-// instead of leaving the buffer.  Off by default (FCN_IDX is the identity).
+// instead of leaving the buffer; FCN_PTR does the same for a pointer p into the
+// n elements from base on.  Off by default (both are the identity).
 #ifdef FCN_CHECKED
 #include <cstdio>
 static __device__ int g_fcn_reports;
@@ -23,8 +24,10 @@ __device__ __forceinline__ long long fcn_chk(long long i, long long n, int site)
     return i;
 }
 #define FCN_IDX(i, n, site) fcn_chk((long long)(i), (long long)(n), (site))
+#define FCN_PTR(p, base, n, site) ((base) + fcn_chk((long long)((p) - (base)), (long long)(n), (site)))
 #else
 #define FCN_IDX(i, n, site) (i)
+#define FCN_PTR(p, base, n, site) (p)
 #endif
 
 namespace fcn {

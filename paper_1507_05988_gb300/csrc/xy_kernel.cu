@@ -186,9 +186,9 @@ __global__ void __launch_bounds__(MAXT, MINB) xy_line_kernel(const __grid_consta
         for (int k = 0; k < L + 2; ++k, p1 += a.pitch, p2 += a.pitch) {
             x[k] = vzero<V>();
             if ((k > 0 || j0 > 0) && j0 - 1 + k < n) {
-                const cx<T> u = *p1;
+                const cx<T> u = *FCN_PTR(p1, a.field, a.total, 73);
                 if constexpr (NP == 2) {
-                    const cx<T> v = *p2;
+                    const cx<T> v = *FCN_PTR(p2, a.field, a.total, 74);
                     x[k] = mk(V{u.x, v.x}, V{u.y, v.y});
                 } else {
                     x[k] = u;
@@ -249,10 +249,10 @@ __global__ void __launch_bounds__(MAXT, MINB) xy_line_kernel(const __grid_consta
     cx<T> *p1 = l1 + (long long)(j0 + L - 1) * a.pitch, *p2 = l2 + (long long)(j0 + L - 1) * a.pitch;
     auto put = [&](cx<V> r) {
         if constexpr (NP == 2) {
-            *p1 = mk(r.x.a, r.y.a);
-            if (two) *p2 = mk(r.x.b, r.y.b);
+            *FCN_PTR(p1, a.field, a.total, 75) = mk(r.x.a, r.y.a);
+            if (two) *FCN_PTR(p2, a.field, a.total, 76) = mk(r.x.b, r.y.b);
         } else {
-            *p1 = r;
+            *FCN_PTR(p1, a.field, a.total, 75) = r;
         }
     };
     if (a.disp == 0.0) {
@@ -313,14 +313,14 @@ __global__ void __launch_bounds__(kXYPointTh) xy_point_kernel(const __grid_const
         on[k] = r < rows;
         wall[k] = j == 0 || j == a.n - 1;
         p[k] = a.field + ((size_t)b * (size_t)a.bstride + (size_t)j * (size_t)a.pitch + c);
-        x[k] = on[k] ? *p[k] : czero<T>();
+        x[k] = on[k] ? *FCN_PTR(p[k], a.field, a.total, 77) : czero<T>();
     }
 #pragma unroll
     for (int k = 0; k < kXYPoint; ++k) {
         const cx<T> r = mk(vfma(-dh, x[k].y, vfma(-dl, x[k].y, x[k].x)), vfma(dh, x[k].x, vfma(dl, x[k].x, x[k].y)));
         Piv2<T> f = inner;
         if (wall[k]) f.h = f.l = czero<T>();
-        if (on[k]) *p[k] = disp_apply(cmul2(f, r), ph);
+        if (on[k]) *FCN_PTR(p[k], a.field, a.total, 78) = disp_apply(cmul2(f, r), ph);
     }
 }
 

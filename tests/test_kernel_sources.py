@@ -41,3 +41,15 @@ def test_kernels_of_programmatic_launches_wait_for_their_predecessor():
         head, sep, _ = body.partition("pdl_enter();")
         assert sep, f"{name} does not wait"
         assert not re.search(r"\w+\[|->|\*\s*\w+\s*=|\b[am]\.\w+", re.sub(r"extern __shared__[^;]*;", "", head)), name
+
+
+def test_cartesian_field_accesses_are_checked():
+    """The self-checking build sees every access of the Cartesian kernels to
+    the field: no pointer in them is followed but through FCN_PTR, and the
+    field is not indexed."""
+    kernels = _kernels()
+    for name in ("xy_line_kernel", "xy_point_kernel"):
+        body = re.sub(r",\s*\*\w+\s*=", ",", kernels[name])            # further pointers of a declaration
+        followed = re.findall(r"(?:^|[=(;{?:,)])\s*\*(\w+)", body)
+        assert followed and set(followed) == {"FCN_PTR"}, (name, followed)
+        assert not re.search(r"\b(field|p|p1|p2|l1|l2)\[(?!k)", body), name
